@@ -914,6 +914,27 @@ static bool cluster_fits(int L, int K, int C, int precision, int dev_smem, int s
     return L % C == 0 && cluster_dyn_bytes(L, K, C, precision) + (size_t)static_smem <= (size_t)dev_smem;
 }
 
+// Whether chain h on a cluster of C CTAs runs on the packed engine (even L,
+// plain sums, the pencil and its ring fit beside the engine's own pk_static
+// bytes): sets the CTAs along y and the dynamic shared memory.
+static bool packed_cluster(const gfmc_ctx* h, int C, int dev_smem, const int* pk_static, int* cy, int* bytes)
+{
+    const bool fp32 = h->precision != GFMC_PREC_FP64;
+    return !h->P.comp && gfmc::pk_split(h->L, C, h->K, fp32, cy, bytes) && *bytes + pk_static[fp32 ? 1 : 0] <= dev_smem;
+}
+
+// A launch group's key: the precision, bit 4 compensated sums, bit 5 packed engine
+static cudaError_t launch_group(int key, const gfmc::TeamJob* d_jobs, int n, int C, int smem, cudaStream_t s)
+{
+    if (key & 32) return gfmc::launch_packed(key & 15, d_jobs, n, C, smem, s);
+    return (key & 15) == GFMC_PREC_FP64 ? gfmc::launch_cluster_f64(d_jobs, n, C, smem, smem, s)
+                                        : gfmc::launch_cluster_f32(d_jobs, n, C, smem, smem, s, (key & 16) != 0);
+}
+static cudaError_t group_max_active(int key, int C, int smem, int* out)
+{
+    return (key & 32) ? gfmc::packed_max_active(key & 15, C, smem, out) : gfmc::cluster_max_active(key & 15, C, smem, out);
+}
+
 gfmc_status gfmc_cluster_min_ctas(int L, int M, int precision, int* cluster_ctas)
 {
     if (!cluster_ctas || L < 3 || L > gfmc::kMaxL || M < 16 || (M & (M - 1)) != 0 ||
@@ -966,12 +987,15 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
     if ((e = gfmc::cluster_static_smem(GFMC_PREC_FP64, &static_smem[0])) != cudaSuccess ||
         (e = gfmc::cluster_static_smem(GFMC_PREC_FP32_MIXED, &static_smem[1])) != cudaSuccess)
         return cuda_fail(nullptr, e, "querying shared memory");
+    int pk_static[2] = {0, 0};
+    if ((e = gfmc::packed_static_smem(GFMC_PREC_FP64, &pk_static[0])) != cudaSuccess ||
+        (e = gfmc::packed_static_smem(GFMC_PREC_FP32_MIXED, &pk_static[1])) != cudaSuccess)
+        return cuda_fail(nullptr, e, "querying shared memory");
     cudaStream_t s = (cudaStream_t)stream;
-    // groups of chains with the same precision and cluster size: one launch each
+    // groups of chains with the same engine, precision and cluster size: one launch each
     struct Group {
         int prec, C;
         size_t vec_bytes;
-        int work;
         std::vector<int> members;
     };
     std::vector<Group> groups;
@@ -982,23 +1006,23 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
         const int T = h->N / C;
         if ((unsigned long long)h->N * (unsigned long long)T >= (1ull << 32))
             return fail(nullptr, GFMC_EINVAL, "chain %d: %d sites per CTA are too many for a cluster", c, T);
-        const size_t vb = cluster_dyn_bytes(h->L, h->K, C, h->precision);
-        const int work = 0;
+        size_t vb = cluster_dyn_bytes(h->L, h->K, C, h->precision);
         const int st_smem = static_smem[h->precision == GFMC_PREC_FP64 ? 0 : 1];
         if (!cluster_fits(h->L, h->K, C, h->precision, dev_smem, st_smem))
             return fail(nullptr, GFMC_EINVAL, "chain %d: %zu B of lattice per CTA (and %d B of the engine's own) exceed "
                         "the %d B of shared memory; use a larger cluster", c, vb, st_smem, dev_smem);
-        // launch key: the precision, and the compensated sums in bit 4
-        const int key = h->precision | (h->P.comp << 4);
+        int cy = 0, pk_bytes = 0;
+        const bool packed = packed_cluster(h, C, dev_smem, pk_static, &cy, &pk_bytes);
+        if (packed) vb = (size_t)pk_bytes;
+        const int key = h->precision | (h->P.comp << 4) | (packed ? 32 : 0);
         Group* g = nullptr;
         for (auto& x : groups)
             if (x.prec == key && x.C == C) g = &x;
         if (!g) {
-            groups.push_back({key, C, 0, 0, {}});
+            groups.push_back({key, C, 0, {}});
             g = &groups.back();
         }
         g->vec_bytes = std::max(g->vec_bytes, vb);
-        g->work = std::max(g->work, work);
         g->members.push_back(c);
         gfmc_status st = ensure_trace(h, std::max<int64_t>(n_updates[c], 1));
         if (st == GFMC_OK) st = ensure_team_capacity(h, C);
@@ -1007,6 +1031,7 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
         P.ncta = C;
         P.divT = (unsigned)(((1ull << 32) + (unsigned long long)T - 1) / (unsigned long long)T);
         P.nv = 2;
+        P.pk_cy = packed ? cy : 0;
         P.mode = gfmc::MODE_SWEEP;
         P.upd0 = h->counter;
         P.n_updates = n_updates[c];
@@ -1030,8 +1055,8 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
     // priority: a scheduler puts its longest chains first)
     for (const auto& g : groups) {
         int active = 0;
-        const int smem = (int)g.vec_bytes + g.work;
-        if ((e = gfmc::cluster_max_active(g.prec & 15, g.C, smem, &active)) != cudaSuccess)
+        const int smem = (int)g.vec_bytes;
+        if ((e = group_max_active(g.prec, g.C, smem, &active)) != cudaSuccess)
             return cuda_fail(nullptr, e, "cluster occupancy");
         if (active < 1)
             return fail(nullptr, GFMC_EINVAL, "a cluster of %d CTAs with %d B of shared memory each cannot be scheduled",
@@ -1072,14 +1097,11 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
         return cuda_fail(nullptr, e, "ordering the cluster launches");
     for (size_t k = 0; k < groups.size(); ++k) {
         const auto& g = groups[k];
-        const int smem = (int)g.vec_bytes + g.work;
+        const int smem = (int)g.vec_bytes;
         if ((e = cudaStreamCreateWithFlags(&gs[k], cudaStreamNonBlocking)) != cudaSuccess ||
             (e = cudaStreamWaitEvent(gs[k], ev[0], 0)) != cudaSuccess)
             return cuda_fail(nullptr, e, "ordering the cluster launches");
-        e = (g.prec & 15) == GFMC_PREC_FP64
-                ? gfmc::launch_cluster_f64(d_jobs + goff[k], (int)g.members.size(), g.C, (int)g.vec_bytes, smem, gs[k])
-                : gfmc::launch_cluster_f32(d_jobs + goff[k], (int)g.members.size(), g.C, (int)g.vec_bytes, smem, gs[k],
-                                           (g.prec >> 4) != 0);
+        e = launch_group(g.prec, d_jobs + goff[k], (int)g.members.size(), g.C, smem, gs[k]);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "launching clusters");
         if ((e = cudaEventCreateWithFlags(&ev[k + 1], cudaEventDisableTiming)) != cudaSuccess ||
             (e = cudaEventRecord(ev[k + 1], gs[k])) != cudaSuccess || (e = cudaStreamWaitEvent(s, ev[k + 1], 0)) != cudaSuccess)
@@ -1266,9 +1288,17 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
         if ((e = gfmc::cluster_static_smem(GFMC_PREC_FP64, &static_smem[0])) != cudaSuccess ||
             (e = gfmc::cluster_static_smem(GFMC_PREC_FP32_MIXED, &static_smem[1])) != cudaSuccess)
             return bail(cuda_fail(nullptr, e, "querying shared memory"));
-        std::vector<std::pair<int, int>> keys;  // (precision, C) in order of first appearance
+        int pk_static[2] = {0, 0};
+        if ((e = gfmc::packed_static_smem(GFMC_PREC_FP64, &pk_static[0])) != cudaSuccess ||
+            (e = gfmc::packed_static_smem(GFMC_PREC_FP32_MIXED, &pk_static[1])) != cudaSuccess)
+            return bail(cuda_fail(nullptr, e, "querying shared memory"));
+        std::vector<std::pair<int, int>> keys;  // (engine and precision, C) in order of first appearance
+        std::vector<int> cy(n_chains, 0), pk_bytes(n_chains, 0), key(n_chains, 0);
         for (int c = 0; c < n_chains; ++c) {
-            const std::pair<int, int> k(chains[c]->precision | (chains[c]->P.comp << 4), ctas[c]);
+            const bool packed = packed_cluster(chains[c], ctas[c], dev_smem, pk_static, &cy[c], &pk_bytes[c]);
+            if (!packed) cy[c] = 0;
+            key[c] = chains[c]->precision | (chains[c]->P.comp << 4) | (packed ? 32 : 0);
+            const std::pair<int, int> k(key[c], ctas[c]);
             if (std::find(keys.begin(), keys.end(), k) == keys.end()) keys.push_back(k);
         }
         // groups launch in the order of their first chain in `chains` (the caller's priority)
@@ -1276,20 +1306,22 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
             Group g{k.first, k.second, (int)jobs.size(), 0, 0};
             for (int c = 0; c < n_chains; ++c) {
                 gfmc_ctx* h = chains[c];
-                if ((h->precision | (h->P.comp << 4)) != k.first || ctas[c] != k.second) continue;
+                if (key[c] != k.first || ctas[c] != k.second) continue;
                 const int C = ctas[c], T = h->N / C;
                 if ((unsigned long long)h->N * (unsigned long long)T >= (1ull << 32))
                     return bail(fail(nullptr, GFMC_EINVAL, "chain %d: %d sites per CTA are too many", c, T));
                 const int st_smem = static_smem[h->precision == GFMC_PREC_FP64 ? 0 : 1];
                 if (!cluster_fits(h->L, h->K, C, h->precision, dev_smem, st_smem))
                     return bail(fail(nullptr, GFMC_EINVAL, "chain %d does not fit a cluster of %d CTAs", c, C));
-                g.vec_bytes = std::max(g.vec_bytes, cluster_dyn_bytes(h->L, h->K, C, h->precision));
+                g.vec_bytes = std::max(g.vec_bytes, cy[c] ? (size_t)pk_bytes[c]
+                                                          : cluster_dyn_bytes(h->L, h->K, C, h->precision));
                 gfmc_status st = ensure_trace(h, n_updates[c]);
                 if (st == GFMC_OK) st = ensure_team_capacity(h, C);
                 if (st != GFMC_OK) return bail(fail(nullptr, st, "chain %d: %s", c, h->err.c_str()));
                 Params P = make_params(h, c, C);
                 P.divT = (unsigned)(((1ull << 32) + (unsigned long long)T - 1) / (unsigned long long)T);
                 P.nv = 2;
+                P.pk_cy = cy[c];
                 gfmc::TeamJob j{};
                 j.p = P;
                 j.cta0 = 0;
@@ -1301,7 +1333,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
                 ++g.count;
             }
             int active = 0;
-            if ((e = gfmc::cluster_max_active(g.prec & 15, g.C, (int)g.vec_bytes, &active)) != cudaSuccess)
+            if ((e = group_max_active(g.prec, g.C, (int)g.vec_bytes, &active)) != cudaSuccess)
                 return bail(cuda_fail(nullptr, e, "cluster occupancy"));
             if (active < 1)
                 return bail(fail(nullptr, GFMC_EINVAL, "a cluster of %d CTAs with %zu B each cannot be scheduled", g.C,
@@ -1409,10 +1441,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
             if ((ce = cudaStreamCreateWithFlags(&gs, cudaStreamNonBlocking)) != cudaSuccess) break;
             p->streams.push_back(gs);
             if ((ce = cudaStreamWaitEvent(gs, fork, 0)) != cudaSuccess) break;
-            ce = (g.prec & 15) == GFMC_PREC_FP64
-                     ? gfmc::launch_cluster_f64(p->d_jobs + g.first, g.count, g.C, (int)g.vec_bytes, (int)g.vec_bytes, gs)
-                     : gfmc::launch_cluster_f32(p->d_jobs + g.first, g.count, g.C, (int)g.vec_bytes, (int)g.vec_bytes, gs,
-                                                (g.prec >> 4) != 0);
+            ce = launch_group(g.prec, p->d_jobs + g.first, g.count, g.C, (int)g.vec_bytes, gs);
             if (ce != cudaSuccess) break;
             if ((ce = cudaEventCreateWithFlags(&join, cudaEventDisableTiming)) != cudaSuccess) break;
             p->events.push_back(join);

@@ -110,6 +110,7 @@ struct Params {
     long long budget; // clock64 cycles a single wait may spin before giving up
     int stall;        // test hook: CTA 0 withholds its completion flags
     int nv;           // recursion vectors of team launches: 7 (unit vectors) or 2 (o and v)
+    int pk_cy;        // packed cluster engine: CTAs of the cluster along y (0: another engine)
 
     // work description
     int mode;
@@ -128,6 +129,49 @@ struct Params {
     unsigned long long* n_acc; // [1]
     long long* n_mag;          // [1]
 };
+
+// Shared memory of a CTA of the packed cluster engine (gfmc_packed.cuh) for a
+// pencil of PY x PZ rows of L sites: the two ring buffers, which are the tail's
+// work area (16 K bytes at least) between recursions; then the forward bonds
+// (rows), and for FP64 the site table.
+__host__ __device__ inline int pk_work_bytes(int L, int PY, int PZ, int K, bool fp32)
+{
+    const int ring = 2 * (PY + 2) * (PZ + 2) * L * (fp32 ? 8 : 16), fft = 16 * K;
+    return ((ring > fft ? ring : fft) + 127) & ~127;
+}
+__host__ __device__ inline int pk_smem_bytes(int L, int PY, int PZ, int K, bool fp32)
+{
+    const int rows = 3 * PY * PZ + PZ + PY;
+    return pk_work_bytes(L, PY, PZ, K, fp32) + rows * L * (fp32 ? 8 : 16) + (fp32 ? 0 : 8 * L * PY * PZ);
+}
+constexpr int kPkThreads32 = 512, kPkThreads64 = 256;
+// The split of an L^3 chain over a cluster of C CTAs into pencils of L / cy x
+// L / (C / cy) rows with the smallest ring (the values exchanged per step);
+// false when the packed cluster engine does not take the chain (odd L, or more
+// pairs per thread than its kernel holds, or 16-bit site indices exceeded).
+inline bool pk_split(int L, int C, int K, bool fp32, int* cy, int* bytes)
+{
+    if (L % 2 != 0 || C < 1 || C > 16) return false;
+    long long best = -1;
+    for (int a = 1; a <= C; ++a) {
+        if (C % a != 0 || L % a != 0 || L % (C / a) != 0) continue;
+        const int PY = L / a, PZ = L / (C / a);
+        if (fp32) {
+            const int ncol = (L / 2) * PY;
+            if (ncol > kPkThreads32) continue;
+            const int nseg = kPkThreads32 / ncol < PZ ? kPkThreads32 / ncol : PZ;
+            if ((PZ + nseg - 1) / nseg > 4) continue;
+        } else if ((PY + 2) * (PZ + 2) * L > 65535) {
+            continue;
+        }
+        const long long ring = (a > 1 ? PZ : 0) + (C / a > 1 ? PY : 0);
+        if (best >= 0 && ring >= best) continue;
+        best = ring;
+        *cy = a;
+        *bytes = pk_smem_bytes(L, PY, PZ, K, fp32);
+    }
+    return best >= 0;
+}
 
 // One chain of a batch launch: its parameters (ncta = its team size, tile plan
 // for that team) and its CTAs [cta0, cta0 + p.ncta) of the grid.
@@ -177,6 +221,10 @@ cudaError_t launch_cluster_f64(const TeamJob* d_jobs, int njobs, int C, int vec_
 cudaError_t launch_cluster_f32(const TeamJob* d_jobs, int njobs, int C, int vec_bytes, int smem, cudaStream_t s,
                                bool comp);
 cudaError_t cluster_max_active(int precision, int C, int smem, int* out);
+// the packed cluster engine (even L; p.pk_cy set): one cluster of C CTAs per job
+cudaError_t launch_packed(int precision, const TeamJob* d_jobs, int njobs, int C, int smem, cudaStream_t s);
+cudaError_t packed_max_active(int precision, int C, int smem, int* out);
+cudaError_t packed_static_smem(int precision, int* out);
 // static shared memory of the cluster engine of a precision (bytes)
 cudaError_t cluster_static_smem(int precision, int* out);
 cudaError_t server_max_ctas(int smem, int* out);

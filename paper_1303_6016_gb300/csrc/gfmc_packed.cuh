@@ -1,0 +1,868 @@
+// gfmc_packed.cuh -- the parity-packed recursion: one complex vector per update.
+//
+// On an even periodic cubic lattice the sites fall into two parity classes and
+// Htilde only couples different classes.  The recursion on the proposal's
+// vectors |o> and |v> = Delta~|o> (Algorithm 1, Eq. recursive) starts on
+// opposite classes (o on its own, v on its neighbours'), so T_n(Htilde)|o> and
+// T_n(Htilde)|v> live on opposite classes for every n.  Their sum
+//     S_n = T_n(Htilde) (|o> + |v>),   S_{n+1} = 2 Htilde S_n - S_{n-1}
+// therefore holds both: the sites of parity(o) + n carry r_n^o, the others
+// r_n^v.  One scalar stencil over the lattice advances both vectors, and the
+// products that do not vanish by parity are local to a site:
+//     |r_m^o|^2 over class A (parity(o) + m),  |r_m^v|^2 over class B,
+//     <r_m^o|r_{m+1}^v> over class A.
+// Delta Omega needs nothing else: <o|T_n|o> and <v|T_n|v> vanish for odd n and
+// <o|T_n|v> for even n.
+//
+// Tile.  A CTA holds the pencil of whole x-rows y in [y0, y0 + PY),
+// z in [z0, z0 + PZ) with a ring of one row on the four sides.  After a step the owner of
+// a face value stores it into the neighbour's ring as well, so the stencil reads the CTA's
+// own shared memory only.  On a thread-block cluster the ring stores go over
+// distributed shared memory and one hardware cluster barrier ends the step.
+//
+// Bound: FP32 by shared-memory wavefronts and instruction issue on large
+// pencils, by the latency of one step (loads, sums, barrier) on small ones;
+// FP64 by the FP64 pipe.  Against the two-vector cluster engine, which advances
+// both vectors on every site (half of the values are zeros), ms per update at
+// M = 1024: FP32 L = 32 on 16 CTAs 1.44 -> 0.70, on 8 CTAs 2.03 -> 1.20, L = 16 on
+// 1 CTA 1.92 -> 1.23, L = 8 on 1 CTA 0.80 -> 0.36; FP64 L = 16 on 16 CTAs 3.12 -> 1.66.
+#pragma once
+
+#include "gfmc_engine.cuh"
+
+namespace gfmc {
+
+// ---------------------------------------------------------------------------
+// sums
+// ---------------------------------------------------------------------------
+
+// round(x 2^58) from the bits of a float (as fixed58 for doubles): the value is
+// mant 2^(ex - 150); ok: |x| <= 16
+__device__ __forceinline__ long long fixed58(float x, bool& ok)
+{
+    const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
+    ok = mag <= 0x41800000u;
+    const int ex = (int)(mag >> 23);
+    const unsigned long long mant = (mag & 0x7fffffu) | (ex ? 0x800000u : 0u);
+    const int sh = (ex ? ex : 1) - 92;  // <= 39 for |x| <= 16
+    unsigned long long q;
+    if (sh >= 0) q = mant << sh;
+    else if (sh <= -25) q = 0;
+    else q = (mant + (1ull << (-sh - 1))) >> -sh;
+    return (b >> 31) ? -(long long)q : (long long)q;
+}
+
+// Values kept apart by the lane groups of 8 of a warp: on return lanes 8 v .. 8 v + 7
+// hold the warp's sum of value v (v < 4).
+template <class T> __device__ __forceinline__ T warp_reduce_scatter4(T (&v)[4], int lane)
+{
+    const bool u16 = lane & 16, u8 = lane & 8;
+    const T a = u16 ? v[2] : v[0], b = u16 ? v[3] : v[1];
+    const T sa = u16 ? v[0] : v[2], sb = u16 ? v[1] : v[3];
+    const T x = a + __shfl_xor_sync(0xffffffffu, sa, 16), y = b + __shfl_xor_sync(0xffffffffu, sb, 16);
+    T r = (u8 ? y : x) + __shfl_xor_sync(0xffffffffu, u8 ? x : y, 8);
+    r += __shfl_xor_sync(0xffffffffu, r, 4);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    return r;
+}
+
+// The four sums of a step by warp, kept for the flush (a ring of four steps: a
+// warp writes step m after it arrived at the barrier that ends the step, the
+// flush of step m - 1 runs after the arrival of step m + 1, and the slot is
+// written again in step m + 3, after a barrier the flushing warp reached later).
+template <class R, int NW> struct PkSums {
+    std::conditional_t<sizeof(R) == 4, float, long long> w[4][NW][4];
+};
+
+// Add the warps' sums of step m (run by one warp) into the chain's fixed-point
+// Gram sums: entries 0 |r_m^o|^2, 1 |r_m^v|^2, 6 and 7 <r_m^o|r_{m+1}^v>.  The
+// sums over warps and CTAs are integer sums, so their order does not matter.
+template <class R, int NW>
+__device__ __forceinline__ void pk_flush(const Params& p, const PkSums<R, NW>& s, int m, int lane)
+{
+    const int v = lane >> 3;
+    long long q = 0;
+    bool fine = true;
+#pragma unroll
+    for (int w = 0; w < NW; w += 8) {
+        const auto x = s.w[m & 3][w + (lane & 7)][v];
+        if constexpr (sizeof(R) == 4) {
+            bool ok;
+            const long long t = fixed58(x, ok);
+            fine = fine && ok;
+            q += ok ? t : 0;
+        } else {
+            q += x;
+        }
+    }
+    q += __shfl_xor_sync(0xffffffffu, q, 4);
+    q += __shfl_xor_sync(0xffffffffu, q, 2);
+    q += __shfl_xor_sync(0xffffffffu, q, 1);
+    if (!fine) set_error(p, ERR_NUMERIC, 90, m);
+    if ((lane & 7) == 0)
+        atomicAdd(p.gram + (size_t)(m - 1) * kEntries + (v < 2 ? v : v + 4), (unsigned long long)q);
+}
+
+// ---------------------------------------------------------------------------
+// the tile
+// ---------------------------------------------------------------------------
+struct PkTile {
+    int L, half, PY, PZ, Cy, Cz, cy, cz, y0, z0, C, rank;
+    int zstr;          // ring rows per plane, PY + 2
+    unsigned ring;     // shared address of the ring buffers
+    unsigned bufB;     // bytes of one ring buffer
+    unsigned r_ym, r_yp, r_zm, r_zp;  // shared::cluster ring addresses of the four neighbours
+    char* ringp;
+    char* bonds;       // BX [PZ][PY], BY [PZ][PY + 1] (from y0 - 1), BZ [PZ + 1][PY] (from z0 - 1) rows
+    unsigned rowB;     // bytes of a row
+    __device__ __forceinline__ int ring_row(int y, int z) const { return (z + 1) * zstr + y + 1; }
+    __device__ __forceinline__ int bx_row(int y, int z) const { return z * PY + y; }
+    __device__ __forceinline__ int by_row(int y, int z) const { return PY * PZ + z * (PY + 1) + y + 1; }
+    __device__ __forceinline__ int bz_row(int y, int z) const
+    {
+        return PY * PZ + PZ * (PY + 1) + (z + 1) * PY + y;
+    }
+    __device__ __forceinline__ int bond_rows() const { return 3 * PY * PZ + PZ + PY; }
+};
+
+template <class R> __device__ __forceinline__ PkTile pk_tile(const Params& p, int rank, char* smem)
+{
+    PkTile t;
+    t.L = p.L;
+    t.half = p.L / 2;
+    t.C = p.ncta;
+    t.rank = rank;
+    t.Cy = p.pk_cy;
+    t.Cz = t.C / t.Cy;
+    t.PY = t.L / t.Cy;
+    t.PZ = t.L / t.Cz;
+    t.cy = rank % t.Cy;
+    t.cz = rank / t.Cy;
+    t.y0 = t.cy * t.PY;
+    t.z0 = t.cz * t.PZ;
+    t.zstr = t.PY + 2;
+    t.rowB = (unsigned)(t.L * 2 * sizeof(R));
+    t.ringp = smem;
+    t.ring = smem_u32(smem);
+    t.bufB = (unsigned)(t.zstr * (t.PZ + 2)) * t.rowB;
+    t.bonds = smem + pk_work_bytes(t.L, t.PY, t.PZ, p.K, sizeof(R) == 4);
+    t.r_ym = cluster_addr(t.ring, (t.cy + t.Cy - 1) % t.Cy + t.cz * t.Cy);
+    t.r_yp = cluster_addr(t.ring, (t.cy + 1) % t.Cy + t.cz * t.Cy);
+    t.r_zm = cluster_addr(t.ring, t.cy + ((t.cz + t.Cz - 1) % t.Cz) * t.Cy);
+    t.r_zp = cluster_addr(t.ring, t.cy + ((t.cz + 1) % t.Cz) * t.Cy);
+    return t;
+}
+
+__device__ __forceinline__ void pk_st(unsigned a, float4 v)
+{
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ void pk_st(unsigned a, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
+// End of a step on the chain's cluster: arrive once this thread's stores are
+// issued, wait before the next step's loads.
+__device__ __forceinline__ void pk_arrive(int C)
+{
+    __syncwarp();
+    if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void pk_wait(int C)
+{
+    if (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
+}
+
+// 2 Htilde's forward bonds of the tile's rows (and of the rows below it in y
+// and z) into shared memory.  FP32 rows hold the pairs (x = 2j, 2j + 1) as
+// (re, re, im, im), FP64 rows the complex values in order.
+template <class R, int NT> __device__ __forceinline__ void pk_load_bonds(const Params& p, const PkTile& t)
+{
+    const int L = t.L, PY = t.PY, PZ = t.PZ, n1 = PY * PZ, n2 = PZ * (PY + 1), rows = t.bond_rows();
+    for (int e = threadIdx.x; e < rows * L; e += NT) {
+        const int row = e / L, x = e - row * L;
+        int a, y, z;
+        if (row < n1) {
+            a = 0;
+            z = row / PY;
+            y = row - z * PY;
+        } else if (row < n1 + n2) {
+            a = 1;
+            z = (row - n1) / (PY + 1);
+            y = row - n1 - z * (PY + 1) - 1;
+        } else {
+            a = 2;
+            z = (row - n1 - n2) / PY;
+            y = row - n1 - n2 - z * PY;
+            --z;
+        }
+        const int gy = (t.y0 + y + L) % L, gz = (t.z0 + z + L) % L;
+        const size_t at = (size_t)a * p.N + (size_t)(gz * L + gy) * L + x;
+        if constexpr (sizeof(R) == 4) {
+            const float2 h = ldcg2(p.hop32 + at);
+            float* d = (float*)(t.bonds + (size_t)row * t.rowB) + 4 * (x >> 1) + (x & 1);
+            d[0] = 2.f * h.x;
+            d[2] = 2.f * h.y;
+        } else {
+            const double2 h = ldcg2(p.hop64 + at);
+            ((double2*)(t.bonds + (size_t)row * t.rowB))[x] = make_double2(2.0 * h.x, 2.0 * h.y);
+        }
+    }
+}
+
+// value of S_0 = |o> + |v> at global site i
+__device__ __forceinline__ double2 pk_s0(int i, const int* s_loc, const double2* s_c)
+{
+    double2 r = make_double2(i == s_loc[0] ? 1.0 : 0.0, 0.0);
+#pragma unroll
+    for (int k = 1; k < 7; ++k)
+        if (i == s_loc[k]) r = s_c[k];
+    return r;
+}
+
+// ---------------------------------------------------------------------------
+// FP32 steps
+// ---------------------------------------------------------------------------
+// A thread advances up to KZ pairs of x-neighbours (x = 2j, 2j + 1) stacked in
+// z: both sites of a pair by one packed FMA, the z-neighbours inside the stack
+// and S_{m-1} from registers.  BREG: the pairs' bonds stay in registers for the
+// whole update (KZ <= 2 at 512 threads); otherwise the y and z bonds are read
+// from shared memory in every step.
+struct Pk32Bond {
+    float2 re, im;
+};
+__device__ __forceinline__ float4 pk_ld(const char* a) { return *(const float4*)a; }
+__device__ __forceinline__ Pk32Bond pk_bond(const char* a)
+{
+    const float4 b = *(const float4*)a;
+    return {make_float2(b.x, b.y), make_float2(b.z, b.w)};
+}
+
+struct Pk32Acc {
+    float2 P, Q, Sf, Wf, Sb, Wb;
+    __device__ __forceinline__ void fwd(const Pk32Bond& h, float2 re, float2 im)
+    {
+        P = __ffma2_rn(h.re, re, P);
+        Q = __ffma2_rn(h.re, im, Q);
+        Sf = __ffma2_rn(h.im, im, Sf);
+        Wf = __ffma2_rn(h.im, re, Wf);
+    }
+    __device__ __forceinline__ void bwd(const Pk32Bond& h, float2 re, float2 im)
+    {
+        P = __ffma2_rn(h.re, re, P);
+        Q = __ffma2_rn(h.re, im, Q);
+        Sb = __ffma2_rn(h.im, im, Sb);
+        Wb = __ffma2_rn(h.im, re, Wb);
+    }
+};
+
+template <int NT, int KZ, bool BREG>
+__device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, const int* s_loc, const double2* s_c,
+                                           PkSums<float, NT / 32>& sums, int nseg)
+{
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int half = t.half, ncol = half * t.PY;
+    const int seg = tid / ncol, col = tid - seg * ncol, y = col / half, j = col - y * half;
+    const int z0 = seg * KZ;
+    const int nz = seg < nseg ? min(KZ, t.PZ - z0) : 0;
+    const int jl = j == 0 ? half - 1 : j - 1, jr = j == half - 1 ? 0 : j + 1;
+    const unsigned strY = t.rowB, strZ = (unsigned)t.zstr * t.rowB;
+    const unsigned own = nz > 0 ? (unsigned)t.ring_row(y, z0) * t.rowB + 16u * (unsigned)j : 0u;
+    const int dl = 16 * (jl - j), dr = 16 * (jr - j);
+    const bool fy0 = y == 0, fy1 = y == t.PY - 1, fz0 = z0 == 0, fz1 = z0 + nz == t.PZ;
+    // where this column's face values go: the neighbour's ring row beyond the far side
+    const unsigned p_ym = t.r_ym + own + strY * (unsigned)t.PY;                      // y = PY of the CTA below
+    const unsigned p_yp = t.r_yp + own - strY * (unsigned)t.PY;                      // y = -1 of the CTA above
+    const unsigned p_zm = t.r_zm + own + strZ * (unsigned)t.PZ;                      // z = PZ of the CTA below
+    const unsigned p_zp = t.r_zp + own - strZ * (unsigned)t.PZ;                      // z = -1 of the CTA above
+    auto put = [&](unsigned buf, int k, float4 v) {
+        const unsigned o = buf + strZ * (unsigned)k;
+        *(float4*)(t.ringp + own + o) = v;
+        if (fy0) pk_st(p_ym + o, v);
+        if (fy1) pk_st(p_yp + o, v);
+        if (fz0 && k == 0) pk_st(p_zm + o, v);
+        if (fz1 && k == nz - 1) pk_st(p_zp + o, v);
+    };
+
+    // bonds: inner (2j -> 2j + 1), outer (left neighbour's, conjugated, and right), y and z
+    float2 bin[KZ];
+    Pk32Bond bout[KZ], byf[BREG ? KZ : 1], byb[BREG ? KZ : 1], bz[BREG ? KZ + 1 : 1];
+    const char *a_yf = t.bonds, *a_zf = t.bonds;
+    if (nz > 0) {
+        a_yf += (size_t)t.by_row(y, z0) * t.rowB + 16 * j;
+        a_zf += (size_t)t.bz_row(y, z0) * t.rowB + 16 * j;
+    }
+    const int sYz = (t.PY + 1) * (int)t.rowB, sZz = t.PY * (int)t.rowB;
+    if constexpr (BREG) bz[0] = pk_bond(a_zf - (nz > 0 ? sZz : 0));
+#pragma unroll
+    for (int k = 0; k < KZ; ++k) {
+        bin[k] = make_float2(0.f, 0.f);
+        bout[k] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (k < nz) {
+            const char* bx = t.bonds + (size_t)t.bx_row(y, z0 + k) * t.rowB;
+            const Pk32Bond c = pk_bond(bx + 16 * j), l = pk_bond(bx + 16 * jl);
+            bin[k] = make_float2(c.re.x, c.im.x);
+            bout[k] = {make_float2(l.re.y, c.re.y), make_float2(-l.im.y, c.im.y)};
+        }
+        if constexpr (BREG) {
+            const Pk32Bond z = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            byf[k] = k < nz ? pk_bond(a_yf + k * sYz) : z;
+            byb[k] = k < nz ? pk_bond(a_yf + k * sYz - (int)t.rowB) : z;
+            bz[k + 1] = k < nz ? pk_bond(a_zf + k * sZz) : z;
+        }
+    }
+
+    float4 va[KZ], vb[KZ];  // S_m and S_{m-1}, by turns
+#pragma unroll
+    for (int k = 0; k < KZ; ++k) {
+        vb[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        va[k] = vb[k];
+        if (k < nz) {
+            const int i = 2 * j + t.L * (t.y0 + y + t.L * (t.z0 + z0 + k));
+            const double2 e = pk_s0(i, s_loc, s_c), o = pk_s0(i + 1, s_loc, s_c);
+            va[k] = make_float4((float)e.x, (float)o.x, (float)e.y, (float)o.y);
+            put(0, k, va[k]);
+        }
+    }
+    pk_arrive(t.C);
+    pk_wait(t.C);
+
+    const int lo = s_loc[0];
+    const int par_o = (lo % t.L + (lo / t.L) % t.L + lo / (t.L * t.L)) & 1;
+    const int par_t = (t.y0 + y + t.z0 + z0) & 1;  // parity of the first pair's even site
+
+    // one step: S_m in cur (and the ring), S_{m-1} in prv, which receives S_{m+1}
+    auto step = [&](int m, float4 (&cur)[KZ], float4 (&prv)[KZ]) {
+        const char* rb = t.ringp + own + (m & 1) * t.bufB;
+        const unsigned wb = (unsigned)((m + 1) & 1) * t.bufB;
+        float2 U[2] = {}, Xr[2] = {}, Xi[2] = {};
+        float4 below = nz > 0 ? pk_ld(rb - strZ) : make_float4(0.f, 0.f, 0.f, 0.f);
+        Pk32Bond zb;
+        if constexpr (BREG) zb = bz[0];
+        else zb = pk_bond(a_zf - (nz > 0 ? sZz : 0));
+#pragma unroll
+        for (int k = 0; k < KZ; ++k) {
+            if (k < nz) {
+                const char* r = rb + strZ * (unsigned)k;
+                const float4 vl = pk_ld(r + dl), vr = pk_ld(r + dr), yp = pk_ld(r + strY), ym = pk_ld(r - strY);
+                const float4 c = cur[k];
+                float4 above;
+                if (k + 1 < KZ && k + 1 < nz) above = cur[k + 1 < KZ ? k + 1 : k];
+                else above = pk_ld(r + strZ);
+                Pk32Bond hf, hb, zf;
+                if constexpr (BREG) {
+                    hf = byf[k];
+                    hb = byb[k];
+                    zf = bz[k + 1];
+                } else {
+                    hf = pk_bond(a_yf + k * sYz);
+                    hb = pk_bond(a_yf + k * sYz - (int)t.rowB);
+                    zf = pk_bond(a_zf + k * sZz);
+                }
+                Pk32Acc a;
+                a.P = make_float2(-prv[k].x, -prv[k].y);
+                a.Q = make_float2(-prv[k].z, -prv[k].w);
+                a.Sf = a.Wf = a.Sb = a.Wb = make_float2(0.f, 0.f);
+                // even site: odd of the own pair; odd site: even of the own pair (conjugated bond)
+                a.fwd({make_float2(bin[k].x, bin[k].x), make_float2(bin[k].y, -bin[k].y)}, make_float2(c.y, c.x),
+                      make_float2(c.w, c.z));
+                a.bwd(zb, make_float2(below.x, below.y), make_float2(below.z, below.w));
+                a.fwd(zf, make_float2(above.x, above.y), make_float2(above.z, above.w));
+                a.fwd(bout[k], make_float2(vl.y, vr.x), make_float2(vl.w, vr.z));
+                a.fwd(hf, make_float2(yp.x, yp.y), make_float2(yp.z, yp.w));
+                a.bwd(hb, make_float2(ym.x, ym.y), make_float2(ym.z, ym.w));
+                const float2 m1 = make_float2(-1.f, -1.f);
+                float2 re = __fadd2_rn(__ffma2_rn(a.Sf, m1, a.P), a.Sb);
+                float2 im = __ffma2_rn(a.Wb, m1, __fadd2_rn(a.Q, a.Wf));
+                if (m == 0) {  // S_1 = Htilde S_0
+                    re = make_float2(0.5f * re.x, 0.5f * re.y);
+                    im = make_float2(0.5f * im.x, 0.5f * im.y);
+                }
+                const float4 nx = make_float4(re.x, re.y, im.x, im.y);
+                if (m < p.nsteps) put(wb, k, nx);
+                const float2 cr = make_float2(c.x, c.y), ci = make_float2(c.z, c.w);
+                U[k & 1] = __ffma2_rn(ci, ci, __ffma2_rn(cr, cr, U[k & 1]));
+                Xr[k & 1] = __ffma2_rn(ci, im, __ffma2_rn(cr, re, Xr[k & 1]));
+                Xi[k & 1] = __ffma2_rn(cr, im, Xi[k & 1]);
+                Xi[k & 1] = __ffma2_rn(make_float2(-ci.x, -ci.y), re, Xi[k & 1]);
+                below = c;
+                zb = zf;
+                prv[k] = nx;
+            }
+        }
+        pk_arrive(t.C);
+        if (m > 0) {
+            // class A: the sites of parity par_o + m; an even site has the parity of its row
+            const bool ea = par_t == ((par_o + m) & 1);
+            float v[4];
+            v[0] = ea ? U[0].x + U[1].y : U[0].y + U[1].x;
+            v[1] = ea ? U[0].y + U[1].x : U[0].x + U[1].y;
+            v[2] = ea ? Xr[0].x + Xr[1].y : Xr[0].y + Xr[1].x;
+            v[3] = ea ? Xi[0].x + Xi[1].y : Xi[0].y + Xi[1].x;
+            const float s = warp_reduce_scatter4(v, lane);
+            if ((lane & 7) == 0) sums.w[m & 3][warp][lane >> 3] = s;
+            if (m >= 3 && warp == (m & (NW - 1))) pk_flush<float, NW>(p, sums, m - 2, lane);
+        }
+        pk_wait(t.C);
+    };
+    int m = 0;
+    for (; m + 1 <= p.nsteps; m += 2) {
+        step(m, va, vb);
+        step(m + 1, vb, va);
+    }
+    if (m <= p.nsteps) step(m, va, vb);
+    __syncthreads();
+    if (warp < 2 && p.nsteps - warp >= 1) pk_flush<float, NW>(p, sums, p.nsteps - warp, lane);
+}
+
+// ---------------------------------------------------------------------------
+// FP64 steps
+// ---------------------------------------------------------------------------
+// The FP64 pipe retires one warp instruction per sub-partition every 64 cycles
+// whatever the active lanes, so the step is dealt out in items (site, real or
+// imaginary part) of 12 multiply-adds, class by class so that the warps of
+// class A (which form <r_m^o|r_{m+1}^v> too) and of class B are apart; operands come from
+// shared memory, nothing is held in registers between steps.
+struct Pk64Site {
+    unsigned short ring, nat;  // ring index (row L + x), bond row index z PY + y
+    unsigned short x;
+    unsigned short face;       // 1: y = 0, 2: y = PY - 1, 4: z = 0, 8: z = PZ - 1
+};
+
+template <int NT>
+__device__ __forceinline__ void pk64_table(const PkTile& t, Pk64Site* tab)
+{
+    const int T = t.L * t.PY * t.PZ, T2 = T / 2;
+    for (int s = threadIdx.x; s < T; s += NT) {
+        const int c = s >= T2 ? 1 : 0, g = s - c * T2, r = g / t.half, j = g - r * t.half;
+        const int z = r / t.PY, y = r - z * t.PY;
+        const int x = 2 * j + ((c + t.y0 + y + t.z0 + z) & 1);
+        Pk64Site q;
+        q.ring = (unsigned short)(t.ring_row(y, z) * t.L + x);
+        q.nat = (unsigned short)r;
+        q.x = (unsigned short)x;
+        q.face = (unsigned short)((y == 0 ? 1 : 0) | (y == t.PY - 1 ? 2 : 0) | (z == 0 ? 4 : 0) |
+                                  (z == t.PZ - 1 ? 8 : 0));
+        tab[s] = q;
+    }
+}
+
+template <int NT>
+__device__ __forceinline__ void pk64_steps(const Params& p, const PkTile& t, const int* s_loc, const double2* s_c,
+                                           PkSums<double, NT / 32>& sums, const Pk64Site* tab)
+{
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int L = t.L, T = L * t.PY * t.PZ, T2 = T / 2;
+    const int c = tid & 1;  // real or imaginary part (NT is even)
+    const unsigned flip = c ? 0u : 0x80000000u;  // sign of the Im h terms of a forward bond
+    const int rowY = 2 * L, rowZ = 2 * L * t.zstr;  // ring strides in doubles
+    const unsigned pushY = t.rowB * (unsigned)t.PY, pushZ = t.rowB * (unsigned)(t.zstr * t.PZ);
+    const unsigned bufD = t.bufB / 8;
+    double* ring = (double*)t.ringp;
+    auto put = [&](unsigned buf, const Pk64Site& q, double v) {
+        const unsigned at = buf * bufD + 2u * q.ring + (unsigned)c;
+        ring[at] = v;
+        if (q.face) {
+            const unsigned b = 8u * at;
+            if (q.face & 1) pk_st(t.r_ym + b + pushY, v);
+            if (q.face & 2) pk_st(t.r_yp + b - pushY, v);
+            if (q.face & 4) pk_st(t.r_zm + b + pushZ, v);
+            if (q.face & 8) pk_st(t.r_zp + b - pushZ, v);
+        }
+    };
+    for (int it = tid; it < 2 * T; it += NT) {
+        const Pk64Site q = tab[it >> 1];
+        const int z = q.nat / t.PY, y = q.nat - z * t.PY;
+        const double2 v = pk_s0(q.x + L * (t.y0 + y + L * (t.z0 + z)), s_loc, s_c);
+        put(0, q, c ? v.y : v.x);
+    }
+    pk_arrive(t.C);
+    pk_wait(t.C);
+    const int lo = s_loc[0];
+    const int par_o = (lo % L + (lo / L) % L + lo / (L * L)) & 1;
+    auto sgn = [&](double h, unsigned f) { return __hiloint2double(__double2hiint(h) ^ (int)f, __double2loint(h)); };
+
+    for (int m = 0; m <= p.nsteps; ++m) {
+        const unsigned rb = (unsigned)(m & 1), wb = rb ^ 1u;
+        const double* rd = ring + rb * bufD;
+        const int clsA = (par_o + m) & 1;
+        double aA = 0.0, aB = 0.0, xr = 0.0, xi = 0.0;
+        for (int it = tid; it < 2 * T; it += NT) {
+            const int s = it >> 1;
+            const Pk64Site q = tab[s];
+            const double* r = rd + 2 * q.ring;
+            const int xp = q.x == L - 1 ? -2 * (L - 1) : 2, xm = q.x == 0 ? 2 * (L - 1) : -2;
+            const double2* bx = (const double2*)t.bonds + (size_t)q.nat * L + q.x;
+            const int z = q.nat / t.PY;
+            const double2* by = bx + (size_t)(t.PY * t.PZ + z + 1) * L;             // row z (PY + 1) + y + 1
+            const double2* bz = bx + (size_t)(t.PY * t.PZ + t.PZ * (t.PY + 1) + t.PY) * L;
+            double acc = m == 0 ? 0.0 : dneg(ring[wb * bufD + 2 * q.ring + c]);
+            auto fwd = [&](double2 h, const double* v) {
+                acc = fma(h.x, v[c], acc);
+                acc = fma(sgn(h.y, flip), v[1 - c], acc);
+            };
+            auto bwd = [&](double2 h, const double* v) {
+                acc = fma(h.x, v[c], acc);
+                acc = fma(sgn(h.y, flip ^ 0x80000000u), v[1 - c], acc);
+            };
+            fwd(bx[0], r + xp);
+            bwd(*(bx + xm / 2), r + xm);
+            fwd(by[0], r + rowY);
+            bwd(*(by - L), r - rowY);
+            fwd(bz[0], r + rowZ);
+            bwd(*(bz - (size_t)t.PY * L), r - rowZ);
+            if (m == 0) acc *= 0.5;
+            if (m < p.nsteps) put(wb, q, acc);
+            if (m > 0) {
+                const double u = r[c], w = r[1 - c];
+                if ((s >= T2) == (clsA != 0)) {
+                    aA = fma(u, u, aA);
+                    xr = fma(u, acc, xr);
+                    xi = fma(sgn(w, flip), acc, xi);  // Re S Im S' - Im S Re S'
+                } else {
+                    aB = fma(u, u, aB);
+                }
+            }
+        }
+        pk_arrive(t.C);
+        if (m > 0) {
+            bool o0, o1, o2, o3;
+            long long v[4] = {fixed58(aA, o0), fixed58(aB, o1), fixed58(xr, o2), fixed58(xi, o3)};
+            if (!(o0 && o1 && o2 && o3)) {
+                set_error(p, ERR_NUMERIC, 90, m);
+                v[0] = v[1] = v[2] = v[3] = 0;
+            }
+            const long long s = warp_reduce_scatter4(v, lane);
+            if ((lane & 7) == 0) sums.w[m & 3][warp][lane >> 3] = s;
+            if (m >= 3 && warp == (m & (NW - 1))) pk_flush<double, NW>(p, sums, m - 2, lane);
+        }
+        pk_wait(t.C);
+    }
+    __syncthreads();
+    if (warp < 2 && p.nsteps - warp >= 1) pk_flush<double, NW>(p, sums, p.nsteps - warp, lane);
+}
+
+// ---------------------------------------------------------------------------
+// the tail
+// ---------------------------------------------------------------------------
+// With <o|T_n|o> and <v|T_n|v> zero for odd n and X_n = <o|T_n|v> zero for
+// even n, the four sequences oo, vv, Re X, Im X have K/2 terms each and
+//     f(theta) = sum_p a_p e^{-2 i p theta}           (oo, vv; n = 2p)
+//     f(theta) = e^{-i theta} sum_p b_p e^{-2 i p theta}   (Re X, Im X; n = 2p + 1)
+// at the even nodes k = 2j (theta_k = pi (k + 1/2)/K) is a K/2-point FFT of the
+// twisted terms a_p e^{-i pi p / K} (Eqs. green_fft, mu_to_mu_tilde).  With
+// s = 2 / sin theta_k the Green's functions are i s f (Eq. green_short),
+// G_ov = i s (f_A + i f_B), G_vo = i s (f_A - i f_B) for f_A, f_B of Re X and Im X, and
+//     d = (1 + G_ov)(1 + G_vo) - G_oo G_vv
+//       = 1 + 2 i s f_A + s^2 (f_oo f_vv - f_A^2 - f_B^2)       (Eq. d_z_green).
+// The odd nodes follow from theta_{K-1-k} = pi - theta_k: f -> conj f for oo, vv
+// and -conj f for A, B, hence d_{K-1-k} = conj d_k and arg d_{K-1-k} = -arg d_k.
+
+// FFT of the chain's sequences: tasks (sequence V, residue r mod Rz of the node
+// index j), task = V Rz + r, dealt round robin to the C CTAs; f of the even
+// nodes goes to p.gnode[V K + j].  work: room for work_n double2 (at least K/2).
+template <int NT>
+__device__ __forceinline__ void pk_tail_fft(const Params& p, int rank, int C, double2* work, int work_n, double vv0,
+                                            double2 ov1)
+{
+    const int tid = threadIdx.x, K = p.K, H = K / 2, MH = p.M / 2;
+    int Rz = 1;
+    while (4 * Rz * 2 <= C && Rz < 8 && H / (2 * Rz) >= 8) Rz *= 2;
+    const int n = H / Rz, ntask = 4 * Rz;
+    int lg = 0;
+    while ((1 << lg) < n) ++lg;
+    const int mine = rank < ntask ? (ntask - 1 - rank) / C + 1 : 0;
+    const int g = min(mine, work_n >> lg);
+    const double2 tw1 = __ldg(p.twc + 1);
+    for (int b = 0; b < mine; b += g) {
+        const int nb = min(g, mine - b), tot = nb << lg;
+        for (int e = tid; e < tot; e += NT) {
+            const int task = rank + (b + (e >> lg)) * C, V = task / Rz, r = task - V * Rz, q = e & (n - 1);
+            double2 x = make_double2(0.0, 0.0);
+            for (int pp = q; pp < MH; pp += n) {
+                const int nn = 2 * pp + (V >> 1);
+                const double first = V == 0 ? 1.0 : V == 1 ? vv0 : V == 2 ? ov1.x : ov1.y;
+                double a = first;
+                if (pp > 0) {
+                    const long long s = (long long)__ldcg(p.gram + (size_t)(pp - 1) * kEntries + (V < 2 ? V : V + 4));
+                    a = fma((double)s, 0x1p-57, -first);  // 2 <.|.> - mu_0 (or mu_1)
+                }
+                a *= __ldg(p.gker + nn) * (nn == 0 ? 0.5 : 1.0);
+                double2 w = __ldg(p.twc + 2 * pp);
+                if (r) {
+                    const int at = (2 * pp * r) & (K - 1);
+                    const double2 u = __ldg(p.fftw + (at & (H - 1)));
+                    w = dmul(w, at >= H ? make_double2(dneg(u.x), dneg(u.y)) : u);
+                }
+                x.x = fma(a, w.x, x.x);
+                x.y = fma(a, w.y, x.y);
+            }
+            work[(e & ~(n - 1)) + (lg ? (int)(__brev((unsigned)q) >> (32 - lg)) : 0)] = x;
+        }
+        __syncthreads();
+        for (int lh = 0; lh < lg; ++lh) {
+            const int hf = 1 << lh;
+            for (int e = tid; e < (tot >> 1); e += NT) {
+                const int pos = e & (hf - 1), i0 = ((e >> lh) << (lh + 1)) + pos, i1 = i0 + hf;
+                const double2 w = __ldg(p.fftw + ((size_t)pos * (K >> (lh + 1))));
+                const double2 u = work[i0], tt = dmul(w, work[i1]);
+                work[i0] = dadd(u, tt);
+                work[i1] = dsub(u, tt);
+            }
+            __syncthreads();
+        }
+        for (int e = tid; e < tot; e += NT) {
+            const int task = rank + (b + (e >> lg)) * C, V = task / Rz, r = task - V * Rz;
+            const int jn = Rz * (e & (n - 1)) + r;
+            double2 x = work[e];
+            if (V >= 2) x = dmul(x, dmul(__ldg(p.fftw + jn), tw1));  // e^{-i theta_{2j}}
+            __stcg(p.gnode + (size_t)V * K + jn, x);
+        }
+        __syncthreads();
+    }
+}
+
+// arg d at the even node k = 2j
+__device__ __forceinline__ double pk_arg(const Params& p, int jn)
+{
+    const int K = p.K;
+    const double2 oo = __ldcg(p.gnode + jn), vv = __ldcg(p.gnode + (size_t)K + jn);
+    const double2 A = __ldcg(p.gnode + 2 * (size_t)K + jn), B = __ldcg(p.gnode + 3 * (size_t)K + jn);
+    const double s = 2.0 / __ldg(p.sinth + 2 * jn);
+    const double2 t = dsub(dsub(dmul(oo, vv), dmul(A, A)), dmul(B, B));
+    const double2 d = make_double2(fma(s * s, t.x, fma(-2.0 * s, A.y, 1.0)), fma(s * s, t.y, 2.0 * s * A.x));
+    if (!isfinite(d.x) || !isfinite(d.y)) set_error(p, ERR_NUMERIC, 40, 2 * jn);
+    return atan2(d.y, d.x);
+}
+
+__device__ __forceinline__ double pk_wrap(double x)
+{
+    if (x > CUDART_PI) x -= 2.0 * CUDART_PI;
+    else if (x <= -CUDART_PI) x += 2.0 * CUDART_PI;
+    return x;
+}
+
+// The CTA's part of sum_k inc_k C_k (Eq. d_seff2; inc_k = phi_k - phi_{k+1}
+// mapped into (-pi, pi], inc_{K-1} = phi_{K-1}) over the nodes 2j, 2j + 1 and
+// their mirrors K-1-2j, K-2-2j for its j in [j0, j1) of [0, K/4): with
+// E_j = phi_{2j} and j' = K/2 - 1 - j, phi_{2j+1} = -E_{j'}.
+template <int NT>
+__device__ __forceinline__ void pk_tail_phase(const Params& p, int rank, int C, double* sarg)
+{
+    const int tid = threadIdx.x, K = p.K, Q = K / 4;
+    const int j0 = (int)(((long long)rank * Q) / C), j1 = (int)(((long long)(rank + 1) * Q) / C), n = j1 - j0;
+    double* A = sarg;          // E_{j0 .. j1}
+    double* B = sarg + n + 1;  // E_{j'} for j = j0 - 1 .. j1 - 1
+    for (int e = tid; e < 2 * n + 2 && n > 0; e += NT) {
+        const int jn = e <= n ? j0 + e : K / 2 - 1 - (j0 - 1 + e - (n + 1));
+        sarg[e] = jn < K / 2 ? pk_arg(p, jn) : 0.0;
+    }
+    __syncthreads();
+    double part = 0.0, mx = 0.0;
+    for (int q = tid; q < n; q += NT) {
+        const int j = j0 + q;
+        const double a = A[q], b = B[q + 1];
+        const double i0 = pk_wrap(a + b), i1 = pk_wrap(-b - A[q + 1]);
+        const double i3 = j == 0 ? -a : pk_wrap(-a - B[q]);
+        part = fma(i0, __ldg(p.cumw + 2 * j), part);
+        part = fma(i1, __ldg(p.cumw + 2 * j + 1), part);
+        part = fma(i0, __ldg(p.cumw + (K - 2 - 2 * j)), part);
+        part = fma(i3, __ldg(p.cumw + (K - 1 - 2 * j)), part);
+        mx = fmax(mx, fmax(fabs(i0), fmax(fabs(i1), fabs(i3))));
+    }
+    double ps, pm;
+    block_sum_max<NT>(part, mx, &ps, &pm);
+    if (tid == 0) {
+        p.qpart[2 * rank] = ps;
+        p.qpart[2 * rank + 1] = pm;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// one chain on a cluster
+// ---------------------------------------------------------------------------
+template <class R> constexpr int pk_threads() { return sizeof(R) == 4 ? kPkThreads32 : kPkThreads64; }
+
+template <class R> __device__ __forceinline__ void pk_run_chain(const Params& p, const int rank, char* smem)
+{
+    constexpr int NT = pk_threads<R>(), NW = NT / 32;
+    __shared__ PkSums<R, NW> sums;
+    __shared__ double2 s_c[kVec], s_hop[kVec];
+    __shared__ double s_chi[8][3];
+    __shared__ int s_loc[kVec];
+    __shared__ double s_draw[3];
+    __shared__ double s_vv0;
+    __shared__ double2 s_ov1;
+    __shared__ int s_acc;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = p.N, L = p.L, C = p.ncta;
+    const PkTile t = pk_tile<R>(p, rank, smem);
+    double2* work = (double2*)smem;
+    const int work_n = pk_work_bytes(L, t.PY, t.PZ, p.K, sizeof(R) == 4) / (int)sizeof(double2);
+    [[maybe_unused]] Pk64Site* tab = (Pk64Site*)(t.bonds + (size_t)t.bond_rows() * t.rowB);
+    if constexpr (sizeof(R) == 8) pk64_table<NT>(t, tab);
+    const long long nupd = (p.mode == MODE_SWEEP) ? p.n_updates : 1;
+    long long nmag = 0;
+    unsigned long long nacc = 0;
+    bool reload = true;
+    auto sync = [&]() {
+        if (C > 1) cl.sync();
+        else __syncthreads();
+    };
+    sync();  // every CTA of the cluster has started before any remote store
+
+    for (long long q = 0; q < nupd; ++q) {
+        const unsigned long long upd = p.upd0 + (unsigned long long)q;
+        const int o = (p.mode == MODE_SWEEP) ? (int)(upd % (unsigned long long)N) : (int)p.site;
+        // ---- set-up: the spinors of the 7 local sites and of the proposal, a
+        //      sincos per lane of warp 0 (lane k the polar, lane 8 + k the azimuthal angle) ----
+        if (warp == 0) {
+            const int k = lane & 7;
+            const int lk = k == 0 ? o : nbr_site(o, min(k, 6) - 1, L);
+            double th = p.theta_new, ph = p.phi_new, u = 0.0;
+            if (p.mode == MODE_SWEEP) draw_update(p.seed, p.chain_id, upd, th, ph, u);
+            if (lane == 7) {
+                s_draw[0] = th;
+                s_draw[1] = ph;
+                s_draw[2] = u;
+            }
+            if (k < 7) {
+                th = __ldcg(p.spins + 2 * lk);
+                ph = __ldcg(p.spins + 2 * lk + 1);
+            }
+            double sn, cs;
+            sincos((lane & 8) ? ph : 0.5 * th, &sn, &cs);
+            const double sp = __shfl_sync(0xffffffffu, sn, k + 8), cp = __shfl_sync(0xffffffffu, cs, k + 8);
+            if (lane < 8) {
+                s_chi[k][0] = cs;
+                s_chi[k][1] = cp * sn;
+                s_chi[k][2] = sp * sn;
+            }
+            if (lane < 7) s_loc[lane] = lk;
+            __syncwarp();
+            if (lane < 7) {
+                double2 cv = make_double2(0.0, 0.0), hv = cv;
+                if (lane > 0) {
+                    // Delta~_{l_j,o} = -t (<chi_j|chi'_o> - <chi_j|chi_o>) / a
+                    const double* cj = s_chi[lane];
+                    const double2 on = overlap3(cj[0], cj[1], cj[2], s_chi[7][0], s_chi[7][1], s_chi[7][2]);
+                    const double2 oo = overlap3(cj[0], cj[1], cj[2], s_chi[0][0], s_chi[0][1], s_chi[0][2]);
+                    cv = make_double2((-p.t * on.x + p.t * oo.x) / p.a, (-p.t * on.y + p.t * oo.y) / p.a);
+                    hv = hop_of(p.hop64, N, o, lane - 1, lk);  // Htilde_{o, l_k}
+                }
+                s_c[lane] = cv;
+                s_hop[lane] = hv;
+            }
+        }
+        if (reload) pk_load_bonds<R, NT>(p, t);
+        reload = false;
+        __syncthreads();
+
+        // ---- the recursion ----
+        if constexpr (sizeof(R) == 4) {
+            const int ncol = t.half * t.PY, room = NT / ncol;
+            const int nseg0 = min(room, t.PZ), S = (t.PZ + nseg0 - 1) / nseg0, nseg = (t.PZ + S - 1) / S;
+            if (S == 1) pk32_steps<NT, 1, true>(p, t, s_loc, s_c, sums, nseg);
+            else if (S == 2) pk32_steps<NT, 2, true>(p, t, s_loc, s_c, sums, nseg);
+            else if (S == 3) pk32_steps<NT, 3, false>(p, t, s_loc, s_c, sums, nseg);
+            else pk32_steps<NT, 4, false>(p, t, s_loc, s_c, sums, nseg);
+        } else {
+            pk64_steps<NT>(p, t, s_loc, s_c, sums, tab);
+        }
+        if (tid == 0) {
+            double v0 = 0.0;
+            double2 o1 = make_double2(0.0, 0.0);
+            for (int k = 1; k < 7; ++k) {
+                v0 += s_c[k].x * s_c[k].x + s_c[k].y * s_c[k].y;  // <v|v>
+                o1 = dadd(o1, dmul(s_c[k], s_hop[k]));            // <o|Htilde|v>
+            }
+            s_vv0 = v0;
+            s_ov1 = o1;
+        }
+        sync();
+
+        // ---- FFT to the nodes, phases, Delta Omega, decision ----
+        pk_tail_fft<NT>(p, rank, C, work, work_n, s_vv0, s_ov1);
+        sync();
+        for (int e = rank * NT + tid; e < 4 * p.nsteps; e += C * NT) {  // the sums are read: clear them
+            const int v = e & 3;
+            __stcg(p.gram + (size_t)(e >> 2) * kEntries + (v < 2 ? v : v + 4), 0ull);
+        }
+        pk_tail_phase<NT>(p, rank, C, (double*)work);
+        sync();
+        if (warp == 0) {
+            double s = lane < C ? __ldcg(p.qpart + 2 * lane) : 0.0;
+            double mx = lane < C ? __ldcg(p.qpart + 2 * lane + 1) : 0.0;
+#pragma unroll
+            for (int b = 8; b > 0; b >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, b);
+                mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, b));
+            }
+            if (lane == 0) {
+                const double dom = p.a / p.K * s;
+                int acc = 0;
+                if (p.mode == MODE_SWEEP) acc = exp(-p.beta * dom) > s_draw[2];
+                s_acc = acc;
+                if (rank == 0) {
+                    const long long slot = (p.mode == MODE_SWEEP) ? q : 0;
+                    p.domega_out[slot] = dom;
+                    if (p.maxinc_out) p.maxinc_out[slot] = mx;
+                    if (p.mode == MODE_SWEEP && p.dec_out) p.dec_out[q] = (unsigned char)acc;
+                }
+            }
+        }
+        __syncthreads();
+        if (p.mode == MODE_DELTA) break;
+        if (s_acc) {
+            ++nacc;
+            reload = true;
+            if (rank == 0 && tid < 7) patch_site(p, o, s_loc, s_draw[0], s_draw[1], tid);
+            sync();
+        }
+        if ((upd + 1ull) % (unsigned long long)N == 0ull) {
+            magnetisation_partial<NT>(p, (int)((long long)rank * N / C), (int)((long long)(rank + 1) * N / C), rank);
+            sync();
+            if (rank == 0 && tid == 0) {
+                double X = 0.0, Y = 0.0, Z = 0.0;
+                for (int c = 0; c < C; ++c) {
+                    X += __ldcg(p.magpart + 3 * c);
+                    Y += __ldcg(p.magpart + 3 * c + 1);
+                    Z += __ldcg(p.magpart + 3 * c + 2);
+                }
+                p.mag_out[nmag] = sqrt(X * X + Y * Y + Z * Z) / N;
+            }
+            ++nmag;
+            sync();  // magpart is read before the next sweep's partials
+        }
+    }
+    if (rank == 0 && tid == 0 && p.mode == MODE_SWEEP) {
+        *p.n_acc = nacc;
+        *p.n_mag = nmag;
+    }
+    sync();  // no CTA leaves while another may still write into its shared memory
+}
+
+// A batch of chains, one thread-block cluster per chain (cluster size = the
+// chains' p.ncta).
+template <class R>
+__global__ void __launch_bounds__(pk_threads<R>(), 1) gfmc_packed_cluster(const TeamJob* __restrict__ jobs)
+{
+    extern __shared__ double2 dyn_all[];
+    __shared__ Params sp;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int job = (int)(blockIdx.x / cl.dim_blocks().x);
+    if (threadIdx.x == 0) sp = jobs[job].p;
+    __syncthreads();
+    pk_run_chain<R>(sp, (int)cl.block_rank(), (char*)dyn_all);
+}
+
+}  // namespace gfmc
