@@ -56,15 +56,24 @@ enum { GFMC_PREC_FP64 = 0, GFMC_PREC_FP32_MIXED = 1 };
 enum { GFMC_KERNEL_JACKSON = 0, GFMC_KERNEL_LORENTZ = 1 };
 /* Vectors the Chebyshev recursion of an update runs on (Sec. 2.2, Eq. recursive):
  * UNIT_VECTORS -- the 7 unit vectors of o and its neighbours, all 7x7 moments
- *                 (independent of the proposal);
+ *                 (independent of the proposal).  With GFMC_ENGINE_AUTO the
+ *                 library may take the proposal's vectors for Delta Omega, which
+ *                 depends on their moments only: the same values to rounding;
  * PROPOSAL     -- the proposal's vectors |o> and |v> = Delta~|o> only: the
  *                 paper's recursion on o, v, o+v, o+iv (Algorithm 1, Fig. 2)
  *                 with the last two formed by linearity, so two recursions and
  *                 <o|T_n|v> give all four sequences. */
 enum { GFMC_RECURSION_UNIT_VECTORS = 0, GFMC_RECURSION_PROPOSAL = 1 };
 /* Engine of a single chain's gfmc_moments / gfmc_delta_omega / gfmc_updates /
- * gfmc_sweep calls on the unit-vector recursion:
- * AUTO            -- VECTOR_CLUSTERS where it applies, else GRID;
+ * gfmc_sweep calls:
+ * AUTO            -- the fastest engine that gives the call's results.  Delta Omega
+ *                    calls on an even lattice (plain sums, automatic CTA count):
+ *                    the proposal's vectors o and v, which live on opposite
+ *                    parities, as one vector on one thread-block cluster or on
+ *                    the whole GPU; FP64 chains hold it in 62-bit fixed point
+ *                    (|value| <= 1, 60 fraction bits).  Else VECTOR_CLUSTERS
+ *                    where it applies, else GRID.  The two below run the
+ *                    recursion that gfmc_options.recursion names;
  * GRID            -- one persistent launch over the whole GPU: each CTA a tile
  *                    of sites, neighbour CTAs synchronised through flags in
  *                    global memory, the moments from the doubling of Eq. mu2
@@ -96,9 +105,8 @@ typedef struct {
     uint32_t chain_id;     /* second key word (XORed with the seed's high word) */
     void* stream;          /* cudaStream_t to run on; NULL = the legacy default stream */
     int num_ctas;          /* <= 0: chosen by the library */
-    /* GFMC_RECURSION_*: used by gfmc_delta_omega and gfmc_updates/gfmc_sweep of
-     * chains on at most 256 sites per CTA; gfmc_moments, batches and servers
-     * always use the unit vectors. */
+    /* GFMC_RECURSION_*: used by gfmc_delta_omega and gfmc_updates/gfmc_sweep,
+     * batches and servers; gfmc_moments always uses the unit vectors. */
     int recursion;
     /* Chebyshev nodes K of the Green's function and of the Delta Omega
      * quadrature, w_k = cos(pi (k + 1/2) / K): 0 or M selects K = M, the nodes

@@ -31,6 +31,10 @@ struct gfmc_ctx {
     // FP32-mixed L = 32 chain on seven thread-block clusters (one per unit
     // vector): single-chain calls on the unit-vector recursion use it
     bool vcl = false;
+    // even lattices on the automatic engine: Delta Omega calls run the packed
+    // recursion on one cluster (1) or on the whole grid (2); 0: another engine
+    int pk = 0, pk_engine = 0, pk_ctas = 0, pk_cy = 0, pk_cz = 0, pk_smem = 0;
+    size_t pk_inbox_bytes = 0;
     Params P{};
     std::vector<void*> allocs;
     uint64_t alloc_bytes = 0;
@@ -226,7 +230,21 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
     P.budget = h->budget;
     P.stall = h->stall_next;
     h->stall_next = 0;
-    if (h->multi_site) {
+    // a cluster of the packed engine has no flags to withhold: the stall hook runs the grid engine
+    const bool packed = h->pk != 0 && P.mode != gfmc::MODE_MOMENTS && !(P.stall && h->pk == 1);
+    if (packed) {
+        P.ncta = h->pk_ctas;
+        P.pk_cy = h->pk_cy;
+        P.pk_cz = h->pk_cz;
+        if (h->pk == 1) {
+            e = gfmc::launch_packed_single(h->pk_engine, P, h->pk_smem, h->stream);
+        } else {
+            // the tags of the face values count from a cleared inbox
+            if ((e = cudaMemsetAsync(P.pk_inbox, 0, h->pk_inbox_bytes, h->stream)) != cudaSuccess)
+                return cuda_fail(h, e, "clearing the inboxes");
+            e = gfmc::launch_packed64_grid(P, h->pk_smem, h->stream);
+        }
+    } else if (h->multi_site) {
         gfmc::TeamJob job{};
         P.nv = (h->recursion == GFMC_RECURSION_PROPOSAL && P.mode != gfmc::MODE_MOMENTS) ? 2 : gfmc::kVec;
         job.p = P;
@@ -339,6 +357,58 @@ gfmc_status use_team_plan(gfmc_ctx* h, int tc)
     h->d_team_nptr = p;
     h->d_team_nidx = x;
     h->team_tc = tc;
+    return GFMC_OK;
+}
+
+// The packed engine of a chain's Delta Omega calls (automatic engine, even L,
+// plain sums), if one takes it.  Measured, us per update at M = 1024:
+//   FP32-mixed, one cluster of C CTAs: L = 4: 276 on 1, 331-342 on 2-16; L = 8:
+//   326 on 1, 333-348 on 2-16; L = 16: 1173 on 1, 443 on 4, 353 on 16; L = 24: 628 on
+//   8, 446 on 16.  So one CTA up to 512 sites, else the most CTAs that split the
+//   lattice.  L = 32 stays on the seven vector clusters (767; one packed cluster
+//   643), whose moments without the doubling are twice as accurate in FP32.
+//   FP64: the cluster of the most CTAs up to L = 16 (L = 8: 418 on 16, 668 on the
+//   grid; L = 16: 614 and 651), where a CTA still has at most 256 sites, one per
+//   thread; the whole grid above.
+gfmc_status plan_packed(gfmc_ctx* h)
+{
+    const bool fp32 = h->precision != GFMC_PREC_FP64;
+    if (h->L % 2 != 0 || h->vcl) return GFMC_OK;
+    int dev_smem = 0, st = 0;
+    cudaError_t e;
+    const int engine = fp32 ? 1 : 2;
+    if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device)) != cudaSuccess ||
+        (e = gfmc::packed_static_smem(engine, &st)) != cudaSuccess)
+        return cuda_fail(h, e, "querying shared memory");
+    for (int C = fp32 && h->N <= 512 ? 1 : 16; C >= 1; --C) {
+        int cy = 0, bytes = 0, active = 0;
+        if (!gfmc::pk_split(h->L, C, h->K, fp32, &cy, &bytes)) continue;
+        if (!fp32) {
+            if (h->N / C > 256) break;
+            bytes = gfmc::pk64_smem_bytes(h->L, h->L / cy, h->L / (C / cy), h->K);
+        }
+        if (bytes + st > dev_smem) continue;
+        if (gfmc::packed_max_active(engine, C, bytes, &active) != cudaSuccess || active < 1) {
+            cudaGetLastError();
+            continue;
+        }
+        h->pk = 1;
+        h->pk_engine = engine;
+        h->pk_ctas = C;
+        h->pk_cy = cy;
+        h->pk_cz = C / cy;
+        h->pk_smem = bytes;
+        return GFMC_OK;
+    }
+    if (fp32) return GFMC_OK;
+    int max_ctas = 0;
+    if ((e = gfmc::packed64_grid_max_ctas(0, &max_ctas)) != cudaSuccess) return cuda_fail(h, e, "querying grid occupancy");
+    if (gfmc::pk_grid_split(h->L, h->K, max_ctas, dev_smem - st, &h->pk_cy, &h->pk_cz, &h->pk_smem)) {
+        h->pk = 2;
+        h->pk_ctas = h->pk_cy * h->pk_cz;
+        h->P.pk_rows = std::max((h->L + h->pk_cy - 1) / h->pk_cy, (h->L + h->pk_cz - 1) / h->pk_cz);
+        h->pk_inbox_bytes = (size_t)h->pk_ctas * 8 * h->P.pk_rows * h->L * 16;
+    }
     return GFMC_OK;
 }
 
@@ -503,6 +573,10 @@ gfmc_status gfmc_create(int L, const double* spins, double t, double mu, double 
         prefetch = gfmc::single_smem_bytes(K, GFMC_PREC_FP64, win_max) + static_smem <= dev_smem;
     }
 
+    if (opt.engine == GFMC_ENGINE_AUTO && opt.num_ctas <= 0 && !opt.compensated &&
+        (st = plan_packed(h)) != GFMC_OK)
+        return bail(st);
+
     Params& P = h->P;
     P.L = L;
     P.N = N;
@@ -533,8 +607,9 @@ gfmc_status gfmc_create(int L, const double* spins, double t, double mu, double 
         (e = dalloc(h, &P.gram, (size_t)P.nsteps * gfmc::kEntries)) != cudaSuccess ||
         (e = dalloc(h, &P.fftin, 4 * (size_t)M)) != cudaSuccess ||
         (e = dalloc(h, &P.gnode, 4 * (size_t)K)) != cudaSuccess ||
-        (e = dalloc(h, &P.qpart, 2 * (size_t)std::max(ncta, 16))) != cudaSuccess ||
-        (e = dalloc(h, &P.magpart, 3 * (size_t)std::max(ncta, 16))) != cudaSuccess ||
+        (e = dalloc(h, &P.qpart, 2 * (size_t)std::max({ncta, 16, h->pk_ctas}))) != cudaSuccess ||
+        (e = dalloc(h, &P.magpart, 3 * (size_t)std::max({ncta, 16, h->pk_ctas}))) != cudaSuccess ||
+        (h->pk == 2 && (e = dalloc(h, (char**)&P.pk_inbox, h->pk_inbox_bytes)) != cudaSuccess) ||
         (h->vcl && (e = dalloc(h, &P.mom32, 49 * (size_t)M)) != cudaSuccess) ||
         (e = dalloc(h, &P.mom_out, 49 * (size_t)M)) != cudaSuccess ||
         (e = dalloc(h, &d_ts, tstart.size())) != cudaSuccess || (e = dalloc(h, &d_np, nptr.size())) != cudaSuccess ||
@@ -917,16 +992,25 @@ static bool cluster_fits(int L, int K, int C, int precision, int dev_smem, int s
 // Whether chain h on a cluster of C CTAs runs on the packed engine (even L,
 // plain sums, the pencil and its ring fit beside the engine's own pk_static
 // bytes): sets the CTAs along y and the dynamic shared memory.
-static bool packed_cluster(const gfmc_ctx* h, int C, int dev_smem, const int* pk_static, int* cy, int* bytes)
+static bool packed_cluster(const gfmc_ctx* h, int C, int dev_smem, const int* pk_static, int* engine, int* cy, int* bytes)
 {
     const bool fp32 = h->precision != GFMC_PREC_FP64;
-    return !h->P.comp && gfmc::pk_split(h->L, C, h->K, fp32, cy, bytes) && *bytes + pk_static[fp32 ? 1 : 0] <= dev_smem;
+    if (h->P.comp || !gfmc::pk_split(h->L, C, h->K, fp32, cy, bytes)) return false;
+    *engine = fp32 ? 1 : 0;
+    if (!fp32) {
+        const int small = gfmc::pk64_smem_bytes(h->L, h->L / *cy, h->L / (C / *cy), h->K);
+        if (small + pk_static[2] <= dev_smem) {
+            *engine = 2;
+            *bytes = small;
+        }
+    }
+    return *bytes + pk_static[*engine] <= dev_smem;
 }
 
-// A launch group's key: the precision, bit 4 compensated sums, bit 5 packed engine
+// A launch group's key: the precision, bit 4 compensated sums; 32 + engine: a packed engine
 static cudaError_t launch_group(int key, const gfmc::TeamJob* d_jobs, int n, int C, int smem, cudaStream_t s)
 {
-    if (key & 32) return gfmc::launch_packed(key & 15, d_jobs, n, C, smem, s);
+    if (key & 32) return gfmc::launch_packed(key & 15, d_jobs, n, C, smem, s);  // key & 15: the engine
     return (key & 15) == GFMC_PREC_FP64 ? gfmc::launch_cluster_f64(d_jobs, n, C, smem, smem, s)
                                         : gfmc::launch_cluster_f32(d_jobs, n, C, smem, smem, s, (key & 16) != 0);
 }
@@ -987,10 +1071,10 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
     if ((e = gfmc::cluster_static_smem(GFMC_PREC_FP64, &static_smem[0])) != cudaSuccess ||
         (e = gfmc::cluster_static_smem(GFMC_PREC_FP32_MIXED, &static_smem[1])) != cudaSuccess)
         return cuda_fail(nullptr, e, "querying shared memory");
-    int pk_static[2] = {0, 0};
-    if ((e = gfmc::packed_static_smem(GFMC_PREC_FP64, &pk_static[0])) != cudaSuccess ||
-        (e = gfmc::packed_static_smem(GFMC_PREC_FP32_MIXED, &pk_static[1])) != cudaSuccess)
-        return cuda_fail(nullptr, e, "querying shared memory");
+    int pk_static[3] = {0, 0, 0};
+    for (int k = 0; k < 3; ++k)
+        if ((e = gfmc::packed_static_smem(k, &pk_static[k])) != cudaSuccess)
+            return cuda_fail(nullptr, e, "querying shared memory");
     cudaStream_t s = (cudaStream_t)stream;
     // groups of chains with the same engine, precision and cluster size: one launch each
     struct Group {
@@ -1011,10 +1095,10 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
         if (!cluster_fits(h->L, h->K, C, h->precision, dev_smem, st_smem))
             return fail(nullptr, GFMC_EINVAL, "chain %d: %zu B of lattice per CTA (and %d B of the engine's own) exceed "
                         "the %d B of shared memory; use a larger cluster", c, vb, st_smem, dev_smem);
-        int cy = 0, pk_bytes = 0;
-        const bool packed = packed_cluster(h, C, dev_smem, pk_static, &cy, &pk_bytes);
+        int cy = 0, pk_bytes = 0, engine = 0;
+        const bool packed = packed_cluster(h, C, dev_smem, pk_static, &engine, &cy, &pk_bytes);
         if (packed) vb = (size_t)pk_bytes;
-        const int key = h->precision | (h->P.comp << 4) | (packed ? 32 : 0);
+        const int key = packed ? 32 + engine : h->precision | (h->P.comp << 4);
         Group* g = nullptr;
         for (auto& x : groups)
             if (x.prec == key && x.C == C) g = &x;
@@ -1288,16 +1372,17 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
         if ((e = gfmc::cluster_static_smem(GFMC_PREC_FP64, &static_smem[0])) != cudaSuccess ||
             (e = gfmc::cluster_static_smem(GFMC_PREC_FP32_MIXED, &static_smem[1])) != cudaSuccess)
             return bail(cuda_fail(nullptr, e, "querying shared memory"));
-        int pk_static[2] = {0, 0};
-        if ((e = gfmc::packed_static_smem(GFMC_PREC_FP64, &pk_static[0])) != cudaSuccess ||
-            (e = gfmc::packed_static_smem(GFMC_PREC_FP32_MIXED, &pk_static[1])) != cudaSuccess)
-            return bail(cuda_fail(nullptr, e, "querying shared memory"));
+        int pk_static[3] = {0, 0, 0};
+        for (int k = 0; k < 3; ++k)
+            if ((e = gfmc::packed_static_smem(k, &pk_static[k])) != cudaSuccess)
+                return bail(cuda_fail(nullptr, e, "querying shared memory"));
         std::vector<std::pair<int, int>> keys;  // (engine and precision, C) in order of first appearance
         std::vector<int> cy(n_chains, 0), pk_bytes(n_chains, 0), key(n_chains, 0);
         for (int c = 0; c < n_chains; ++c) {
-            const bool packed = packed_cluster(chains[c], ctas[c], dev_smem, pk_static, &cy[c], &pk_bytes[c]);
+            int engine = 0;
+            const bool packed = packed_cluster(chains[c], ctas[c], dev_smem, pk_static, &engine, &cy[c], &pk_bytes[c]);
             if (!packed) cy[c] = 0;
-            key[c] = chains[c]->precision | (chains[c]->P.comp << 4) | (packed ? 32 : 0);
+            key[c] = packed ? 32 + engine : chains[c]->precision | (chains[c]->P.comp << 4);
             const std::pair<int, int> k(key[c], ctas[c]);
             if (std::find(keys.begin(), keys.end(), k) == keys.end()) keys.push_back(k);
         }

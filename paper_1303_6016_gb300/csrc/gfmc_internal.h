@@ -110,7 +110,10 @@ struct Params {
     long long budget; // clock64 cycles a single wait may spin before giving up
     int stall;        // test hook: CTA 0 withholds its completion flags
     int nv;           // recursion vectors of team launches: 7 (unit vectors) or 2 (o and v)
-    int pk_cy;        // packed cluster engine: CTAs of the cluster along y (0: another engine)
+    int pk_cy;        // packed engines: CTAs along y (0: another engine)
+    int pk_cz;        // and along z
+    int pk_rows;      // packed grid engine: rows per face of an inbox
+    unsigned long long* pk_inbox;  // [ncta][2][4][pk_rows][L][2] face values in flight
 
     // work description
     int mode;
@@ -132,8 +135,7 @@ struct Params {
 
 // Shared memory of a CTA of the packed cluster engine (gfmc_packed.cuh) for a
 // pencil of PY x PZ rows of L sites: the two ring buffers, which are the tail's
-// work area (16 K bytes at least) between recursions; then the forward bonds
-// (rows), and for FP64 the site table.
+// work area (16 K bytes at least) between recursions; then the forward bonds.
 __host__ __device__ inline int pk_work_bytes(int L, int PY, int PZ, int K, bool fp32)
 {
     const int ring = 2 * (PY + 2) * (PZ + 2) * L * (fp32 ? 8 : 16), fft = 16 * K;
@@ -142,13 +144,18 @@ __host__ __device__ inline int pk_work_bytes(int L, int PY, int PZ, int K, bool 
 __host__ __device__ inline int pk_smem_bytes(int L, int PY, int PZ, int K, bool fp32)
 {
     const int rows = 3 * PY * PZ + PZ + PY;
-    return pk_work_bytes(L, PY, PZ, K, fp32) + rows * L * (fp32 ? 8 : 16) + (fp32 ? 0 : 8 * L * PY * PZ);
+    return pk_work_bytes(L, PY, PZ, K, fp32) + rows * L * (fp32 ? 8 : 16);
+}
+// the same for the FP64 engines of gfmc_packed64.cuh: a record per site too
+__host__ __device__ inline int pk64_smem_bytes(int L, int PY, int PZ, int K)
+{
+    return pk_smem_bytes(L, PY, PZ, K, false) + 8 * L * PY * PZ;
 }
 constexpr int kPkThreads32 = 512, kPkThreads64 = 256;
 // The split of an L^3 chain over a cluster of C CTAs into pencils of L / cy x
 // L / (C / cy) rows with the smallest ring (the values exchanged per step);
 // false when the packed cluster engine does not take the chain (odd L, or more
-// pairs per thread than its kernel holds, or 16-bit site indices exceeded).
+// pairs per thread than its FP32 kernel holds).
 inline bool pk_split(int L, int C, int K, bool fp32, int* cy, int* bytes)
 {
     if (L % 2 != 0 || C < 1 || C > 16) return false;
@@ -161,8 +168,6 @@ inline bool pk_split(int L, int C, int K, bool fp32, int* cy, int* bytes)
             if (ncol > kPkThreads32) continue;
             const int nseg = kPkThreads32 / ncol < PZ ? kPkThreads32 / ncol : PZ;
             if ((PZ + nseg - 1) / nseg > 4) continue;
-        } else if ((PY + 2) * (PZ + 2) * L > 65535) {
-            continue;
         }
         const long long ring = (a > 1 ? PZ : 0) + (C / a > 1 ? PY : 0);
         if (best >= 0 && ring >= best) continue;
@@ -170,6 +175,30 @@ inline bool pk_split(int L, int C, int K, bool fp32, int* cy, int* bytes)
         *cy = a;
         *bytes = pk_smem_bytes(L, PY, PZ, K, fp32);
     }
+    return best >= 0;
+}
+
+// The split of an even lattice over at most max_ctas CTAs of the grid into
+// pencils of whole x-rows: the fewest rows in the largest pencil, then the
+// fewest face values; false when none fits (smem: the room per CTA).
+constexpr int kPkMaxFaces = 6 * 256;  // face values a CTA receives per step at most
+inline bool pk_grid_split(int L, int K, int max_ctas, int smem, int* cy, int* cz, int* bytes)
+{
+    if (L % 2 != 0) return false;
+    long long best = -1;
+    for (int a = 2; a <= L; ++a)
+        for (int b = 2; b <= L && a * b <= max_ctas; ++b) {
+            const int PY = (L + a - 1) / a, PZ = (L + b - 1) / b;
+            const int faces = L * (2 * PZ + 2 * PY);
+            const int need = pk64_smem_bytes(L, PY, PZ, K);
+            if (faces > kPkMaxFaces || need > smem || (PY + 2) * (PZ + 2) * L > 65535) continue;
+            const long long cost = (long long)PY * PZ * 1000000 + faces * 100 + a + b;
+            if (best >= 0 && cost >= best) continue;
+            best = cost;
+            *cy = a;
+            *cz = b;
+            *bytes = need;
+        }
     return best >= 0;
 }
 
@@ -221,10 +250,15 @@ cudaError_t launch_cluster_f64(const TeamJob* d_jobs, int njobs, int C, int vec_
 cudaError_t launch_cluster_f32(const TeamJob* d_jobs, int njobs, int C, int vec_bytes, int smem, cudaStream_t s,
                                bool comp);
 cudaError_t cluster_max_active(int precision, int C, int smem, int* out);
-// the packed cluster engine (even L; p.pk_cy set): one cluster of C CTAs per job
-cudaError_t launch_packed(int precision, const TeamJob* d_jobs, int njobs, int C, int smem, cudaStream_t s);
-cudaError_t packed_max_active(int precision, int C, int smem, int* out);
-cudaError_t packed_static_smem(int precision, int* out);
+// the packed engines (even L; p.pk_cy set): engine 0 FP64 and 1 FP32-mixed, one
+// cluster of C CTAs per job; 2 FP64 with small tiles (pk64_smem_bytes)
+cudaError_t launch_packed(int engine, const TeamJob* d_jobs, int njobs, int C, int smem, cudaStream_t s);
+cudaError_t launch_packed_single(int engine, const Params& p, int smem, cudaStream_t s);
+cudaError_t packed_max_active(int engine, int C, int smem, int* out);
+cudaError_t packed_static_smem(int engine, int* out);
+// a single FP64 chain on p.ncta CTAs of a cooperative grid
+cudaError_t launch_packed64_grid(const Params& p, int smem, cudaStream_t s);
+cudaError_t packed64_grid_max_ctas(int smem, int* out);
 // static shared memory of the cluster engine of a precision (bytes)
 cudaError_t cluster_static_smem(int precision, int* out);
 cudaError_t server_max_ctas(int smem, int* out);

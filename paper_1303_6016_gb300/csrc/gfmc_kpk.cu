@@ -1,76 +1,100 @@
-// Launch of the packed cluster engine (gfmc_packed.cuh), FP64 and FP32-mixed.
-#include "gfmc_packed.cuh"
+// Launch of the packed engines: clusters FP32-mixed and FP64 (gfmc_packed.cuh),
+// FP64 small tiles on a cluster or on the whole grid (gfmc_packed64.cuh).
+#include "gfmc_packed64.cuh"
 
 namespace gfmc {
 
 namespace {
 
-template <class R> cudaError_t pk_config(int C)
-{
-    cudaError_t e = allow_dynamic_smem((const void*)gfmc_packed_cluster<R>);
-    if (e == cudaSuccess && C > 8)
-        e = cudaFuncSetAttribute(gfmc_packed_cluster<R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    return e;
-}
+using PkKernel = void (*)(const TeamJob*);
 
-template <class R>
-cudaLaunchConfig_t pk_launch_config(int njobs, int C, int smem, cudaStream_t s, cudaLaunchAttribute* attr)
+// engine: 0 FP64 and 1 FP32-mixed clusters, 2 FP64 clusters with small tiles
+PkKernel pk_kernel(int engine)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(C * njobs));
-    cfg.blockDim = dim3(pk_threads<R>());
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = s;
+    return engine == 0 ? gfmc_packed_cluster<double> : engine == 1 ? gfmc_packed_cluster<float> : gfmc_packed64_cluster;
+}
+int pk_block(int engine) { return engine == 0 ? kPkThreads64 : engine == 1 ? kPkThreads32 : kPk64Threads; }
+
+cudaError_t pk_config(int engine, int njobs, int C, int smem, cudaStream_t s, cudaLaunchConfig_t* cfg,
+                      cudaLaunchAttribute* attr)
+{
+    cudaError_t e = allow_dynamic_smem((const void*)pk_kernel(engine));
+    if (e == cudaSuccess && C > 8)
+        e = cudaFuncSetAttribute((const void*)pk_kernel(engine), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    *cfg = {};
+    cfg->gridDim = dim3((unsigned)(C * njobs));
+    cfg->blockDim = dim3((unsigned)pk_block(engine));
+    cfg->dynamicSmemBytes = (size_t)smem;
+    cfg->stream = s;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
-}
-
-template <class R> cudaError_t pk_launch(const TeamJob* d_jobs, int njobs, int C, int smem, cudaStream_t s)
-{
-    cudaError_t e = pk_config<R>(C);
-    if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pk_launch_config<R>(njobs, C, smem, s, attr);
-    return cudaLaunchKernelEx(&cfg, gfmc_packed_cluster<R>, d_jobs);
-}
-
-template <class R> cudaError_t pk_max_active(int C, int smem, int* out)
-{
-    cudaError_t e = pk_config<R>(C);
-    if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = pk_launch_config<R>(1, C, smem, nullptr, attr);
-    return cudaOccupancyMaxActiveClusters(out, gfmc_packed_cluster<R>, &cfg);
-}
-
-template <class R> cudaError_t pk_static_smem(int* out)
-{
-    cudaFuncAttributes a;
-    const cudaError_t e = cudaFuncGetAttributes(&a, gfmc_packed_cluster<R>);
-    if (e == cudaSuccess) *out = (int)a.sharedSizeBytes;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
     return e;
 }
 
 }  // namespace
 
-cudaError_t launch_packed(int precision, const TeamJob* d_jobs, int njobs, int C, int smem, cudaStream_t s)
+cudaError_t launch_packed(int engine, const TeamJob* d_jobs, int njobs, int C, int smem, cudaStream_t s)
 {
-    return precision == 0 ? pk_launch<double>(d_jobs, njobs, C, smem, s) : pk_launch<float>(d_jobs, njobs, C, smem, s);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg;
+    cudaError_t e = pk_config(engine, njobs, C, smem, s, &cfg, attr);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, pk_kernel(engine), d_jobs);
 }
 
-cudaError_t packed_max_active(int precision, int C, int smem, int* out)
+cudaError_t launch_packed_single(int engine, const Params& p, int smem, cudaStream_t s)
 {
-    return precision == 0 ? pk_max_active<double>(C, smem, out) : pk_max_active<float>(C, smem, out);
+    const auto fn = engine == 1 ? gfmc_packed_single<float> : gfmc_packed_single<double>;
+    cudaError_t e = allow_dynamic_smem((const void*)fn);
+    if (e == cudaSuccess && p.ncta > 8)
+        e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg;
+    if (e == cudaSuccess) e = pk_config(engine, 1, p.ncta, smem, s, &cfg, attr);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, fn, p);
 }
 
-cudaError_t packed_static_smem(int precision, int* out)
+cudaError_t packed_max_active(int engine, int C, int smem, int* out)
 {
-    return precision == 0 ? pk_static_smem<double>(out) : pk_static_smem<float>(out);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg;
+    cudaError_t e = pk_config(engine, 1, C, smem, nullptr, &cfg, attr);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveClusters(out, pk_kernel(engine), &cfg);
+}
+
+cudaError_t packed_static_smem(int engine, int* out)
+{
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, (const void*)pk_kernel(engine));
+    if (e == cudaSuccess) *out = (int)a.sharedSizeBytes;
+    return e;
+}
+
+cudaError_t launch_packed64_grid(const Params& p, int smem, cudaStream_t s)
+{
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_packed64_grid);
+    if (e != cudaSuccess) return e;
+    Params q = p;
+    void* args[] = {(void*)&q};
+    return cudaLaunchCooperativeKernel((void*)gfmc_packed64_grid, dim3((unsigned)p.ncta), dim3(kPk64Threads), args,
+                                       (size_t)smem, s);
+}
+
+cudaError_t packed64_grid_max_ctas(int smem, int* out)
+{
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_packed64_grid);
+    int per_sm = 0, dev = 0, sms = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gfmc_packed64_grid, kPk64Threads, smem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    *out = per_sm > 0 ? sms : 0;  // one CTA per SM
+    return e;
 }
 
 }  // namespace gfmc

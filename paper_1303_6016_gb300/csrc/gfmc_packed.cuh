@@ -22,10 +22,11 @@
 //
 // Bound: FP32 by shared-memory wavefronts and instruction issue on large
 // pencils, by the latency of one step (loads, sums, barrier) on small ones;
-// FP64 by the FP64 pipe.  Against the two-vector cluster engine, which advances
+// FP64, in fixed point, by instruction issue and the exchange.  Against the two-vector cluster engine, which advances
 // both vectors on every site (half of the values are zeros), ms per update at
-// M = 1024: FP32 L = 32 on 16 CTAs 1.44 -> 0.70, on 8 CTAs 2.03 -> 1.20, L = 16 on
-// 1 CTA 1.92 -> 1.23, L = 8 on 1 CTA 0.80 -> 0.36; FP64 L = 16 on 16 CTAs 3.12 -> 1.66.
+// M = 1024: FP32 L = 32 on 16 CTAs 1.44 -> 0.64, on 8 CTAs 2.03 -> 1.25, L = 16 on
+// 1 CTA 1.92 -> 1.17, L = 8 on 1 CTA 0.80 -> 0.33; FP64 L = 16 on 16 CTAs 3.12 -> 1.66
+// with FP64 arithmetic, 0.61 in fixed point (below).
 #pragma once
 
 #include "gfmc_engine.cuh"
@@ -36,15 +37,15 @@ namespace gfmc {
 // sums
 // ---------------------------------------------------------------------------
 
-// round(x 2^58) from the bits of a float (as fixed58 for doubles): the value is
-// mant 2^(ex - 150); ok: |x| <= 16
-__device__ __forceinline__ long long fixed58(float x, bool& ok)
+// round(x 2^60) from the bits of a float with integer operations only: the
+// value is mant 2^(ex - 150); ok: |x| <= 4
+__device__ __forceinline__ long long fixed60(float x, bool& ok)
 {
     const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
-    ok = mag <= 0x41800000u;
+    ok = mag <= 0x40800000u;
     const int ex = (int)(mag >> 23);
     const unsigned long long mant = (mag & 0x7fffffu) | (ex ? 0x800000u : 0u);
-    const int sh = (ex ? ex : 1) - 92;  // <= 39 for |x| <= 16
+    const int sh = (ex ? ex : 1) - 90;  // <= 39 for |x| <= 4
     unsigned long long q;
     if (sh >= 0) q = mant << sh;
     else if (sh <= -25) q = 0;
@@ -67,17 +68,24 @@ template <class T> __device__ __forceinline__ T warp_reduce_scatter4(T (&v)[4], 
     return r;
 }
 
-// The four sums of a step by warp, kept for the flush (a ring of four steps: a
-// warp writes step m after it arrived at the barrier that ends the step, the
-// flush of step m - 1 runs after the arrival of step m + 1, and the slot is
-// written again in step m + 3, after a barrier the flushing warp reached later).
+// The four sums of each step by warp, kept until they are flushed: a warp
+// writes step m between its arrival at the barrier that ends the step and its
+// wait there, so the sums of step m are complete for every warp after the
+// barrier of step m + 1.  Every kPkGroup steps as many warps add one step each
+// into the chain's sums (at step m = 1 mod kPkGroup the steps m - kPkGroup - 1 .. m - 2; the
+// slots are written again kPkRing steps later), which keeps the additions and
+// conversions off the steps' critical path: one warp flushing one step in every step
+// cost 220-320 cycles of each.
+constexpr int kPkGroup = 8, kPkRing = 16;
 template <class R, int NW> struct PkSums {
-    std::conditional_t<sizeof(R) == 4, float, long long> w[4][NW][4];
+    std::conditional_t<sizeof(R) == 4, float, long long> w[kPkRing][NW][4];
 };
 
 // Add the warps' sums of step m (run by one warp) into the chain's fixed-point
-// Gram sums: entries 0 |r_m^o|^2, 1 |r_m^v|^2, 6 and 7 <r_m^o|r_{m+1}^v>.  The
-// sums over warps and CTAs are integer sums, so their order does not matter.
+// Gram sums, in units of 2^-60: entries 0 |r_m^o|^2, 1 |r_m^v|^2, 6 and 7
+// <r_m^o|r_{m+1}^v>.  The sums over warps and CTAs are integer sums, so their
+// order does not matter; every |sum| <= 1.
+constexpr int kPkFrac = 60;
 template <class R, int NW>
 __device__ __forceinline__ void pk_flush(const Params& p, const PkSums<R, NW>& s, int m, int lane)
 {
@@ -86,10 +94,10 @@ __device__ __forceinline__ void pk_flush(const Params& p, const PkSums<R, NW>& s
     bool fine = true;
 #pragma unroll
     for (int w = 0; w < NW; w += 8) {
-        const auto x = s.w[m & 3][w + (lane & 7)][v];
+        const auto x = s.w[m & (kPkRing - 1)][w + (lane & 7)][v];
         if constexpr (sizeof(R) == 4) {
             bool ok;
-            const long long t = fixed58(x, ok);
+            const long long t = fixed60(x, ok);
             fine = fine && ok;
             q += ok ? t : 0;
         } else {
@@ -102,6 +110,33 @@ __device__ __forceinline__ void pk_flush(const Params& p, const PkSums<R, NW>& s
     if (!fine) set_error(p, ERR_NUMERIC, 90, m);
     if ((lane & 7) == 0)
         atomicAdd(p.gram + (size_t)(m - 1) * kEntries + (v < 2 ? v : v + 4), (unsigned long long)q);
+}
+template <class R, int NW>
+__device__ __forceinline__ void pk_flush_due(const Params& p, const PkSums<R, NW>& s, int m, int warp, int lane)
+{
+    if ((m & (kPkGroup - 1)) == 1 && m > kPkGroup) {
+        if constexpr (sizeof(R) == 8) {
+            // lane (step, value) of one warp adds the warps' sums
+            const int f = m - kPkGroup - 1 + (lane >> 2), v = lane & 3;
+            if (warp == 0 && f > 0) {
+                long long q = 0;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) q += s.w[f & (kPkRing - 1)][w][v];
+                atomicAdd(p.gram + (size_t)(f - 1) * kEntries + (v < 2 ? v : v + 4), (unsigned long long)q);
+            }
+        } else if (warp < kPkGroup) {
+            const int f = m - kPkGroup - 1 + warp;
+            if (f > 0) pk_flush<R, NW>(p, s, f, lane);
+        }
+    }
+}
+// The steps that pk_flush_due, last called for step `last`, has not reached;
+// the warps have met since the last step's sums were written.
+template <class R, int NW>
+__device__ __forceinline__ void pk_flush_rest(const Params& p, const PkSums<R, NW>& s, int last, int warp, int lane)
+{
+    const int done = last > kPkGroup ? ((last - 1) & ~(kPkGroup - 1)) - 1 : 0;  // the last step flushed
+    for (int f = max(done, 0) + 1 + warp; f <= p.nsteps; f += NW) pk_flush<R, NW>(p, s, f, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -126,6 +161,7 @@ struct PkTile {
     __device__ __forceinline__ int bond_rows() const { return 3 * PY * PZ + PZ + PY; }
 };
 
+// The pencils of a grid chain may differ by one row in y and z.
 template <class R> __device__ __forceinline__ PkTile pk_tile(const Params& p, int rank, char* smem)
 {
     PkTile t;
@@ -135,12 +171,12 @@ template <class R> __device__ __forceinline__ PkTile pk_tile(const Params& p, in
     t.rank = rank;
     t.Cy = p.pk_cy;
     t.Cz = t.C / t.Cy;
-    t.PY = t.L / t.Cy;
-    t.PZ = t.L / t.Cz;
     t.cy = rank % t.Cy;
     t.cz = rank / t.Cy;
-    t.y0 = t.cy * t.PY;
-    t.z0 = t.cz * t.PZ;
+    t.y0 = t.cy * t.L / t.Cy;
+    t.z0 = t.cz * t.L / t.Cz;
+    t.PY = (t.cy + 1) * t.L / t.Cy - t.y0;
+    t.PZ = (t.cz + 1) * t.L / t.Cz - t.z0;
     t.zstr = t.PY + 2;
     t.rowB = (unsigned)(t.L * 2 * sizeof(R));
     t.ringp = smem;
@@ -154,14 +190,20 @@ template <class R> __device__ __forceinline__ PkTile pk_tile(const Params& p, in
     return t;
 }
 
-__device__ __forceinline__ void pk_st(unsigned a, float4 v)
+// A face value into a neighbour's ring where `on` (predicated: four branches
+// per site cost about 300 cycles of a small tile's step).  A pencil that is its
+// own neighbour stores to itself the same way.
+__device__ __forceinline__ void pk_st(bool on, unsigned a, float4 v)
 {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n @p st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};\n}" ::"r"(a),
+                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"((unsigned)on)
                  : "memory");
 }
-__device__ __forceinline__ void pk_st(unsigned a, double v)
+__device__ __forceinline__ void pk_st(bool on, unsigned a, int4 v)
 {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n @p st.shared::cluster.v4.s32 [%0], {%1, %2, %3, %4};\n}" ::"r"(a),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((unsigned)on)
+                 : "memory");
 }
 
 // End of a step on the chain's cluster: arrive once this thread's stores are
@@ -177,9 +219,16 @@ __device__ __forceinline__ void pk_wait(int C)
     else __syncthreads();
 }
 
+// the limbs of two fixed-point values: value = high 2^30 + low, the low limb in [-2^29, 2^29)
+__device__ __forceinline__ int4 pk_limbs(long long re, long long im)
+{
+    return make_int4((int)((re + (1ll << 29)) >> 30), (int)((unsigned)re << 2) >> 2, (int)((im + (1ll << 29)) >> 30),
+                     (int)((unsigned)im << 2) >> 2);
+}
+
 // 2 Htilde's forward bonds of the tile's rows (and of the rows below it in y
 // and z) into shared memory.  FP32 rows hold the pairs (x = 2j, 2j + 1) as
-// (re, re, im, im), FP64 rows the complex values in order.
+// (re, re, im, im), FP64 rows the fixed-point limbs, even sites first.
 template <class R, int NT> __device__ __forceinline__ void pk_load_bonds(const Params& p, const PkTile& t)
 {
     const int L = t.L, PY = t.PY, PZ = t.PZ, n1 = PY * PZ, n2 = PZ * (PY + 1), rows = t.bond_rows();
@@ -209,7 +258,8 @@ template <class R, int NT> __device__ __forceinline__ void pk_load_bonds(const P
             d[2] = 2.f * h.y;
         } else {
             const double2 h = ldcg2(p.hop64 + at);
-            ((double2*)(t.bonds + (size_t)row * t.rowB))[x] = make_double2(2.0 * h.x, 2.0 * h.y);
+            ((int4*)(t.bonds + (size_t)row * t.rowB))[(x & 1) * t.half + (x >> 1)] =
+                pk_limbs(__double2ll_rn(h.x * 0x1p61), __double2ll_rn(h.y * 0x1p61));
         }
     }
 }
@@ -264,6 +314,7 @@ template <int NT, int KZ, bool BREG>
 __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, const int* s_loc, const double2* s_c,
                                            PkSums<float, NT / 32>& sums, int nseg)
 {
+    const int nsteps = p.nsteps;
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int half = t.half, ncol = half * t.PY;
@@ -283,10 +334,10 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
     auto put = [&](unsigned buf, int k, float4 v) {
         const unsigned o = buf + strZ * (unsigned)k;
         *(float4*)(t.ringp + own + o) = v;
-        if (fy0) pk_st(p_ym + o, v);
-        if (fy1) pk_st(p_yp + o, v);
-        if (fz0 && k == 0) pk_st(p_zm + o, v);
-        if (fz1 && k == nz - 1) pk_st(p_zp + o, v);
+        pk_st(fy0, p_ym + o, v);
+        pk_st(fy1, p_yp + o, v);
+        pk_st(fz0 && k == 0, p_zm + o, v);
+        pk_st(fz1 && k == nz - 1, p_zp + o, v);
     };
 
     // bonds: inner (2j -> 2j + 1), outer (left neighbour's, conjugated, and right), y and z
@@ -384,7 +435,7 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
                     im = make_float2(0.5f * im.x, 0.5f * im.y);
                 }
                 const float4 nx = make_float4(re.x, re.y, im.x, im.y);
-                if (m < p.nsteps) put(wb, k, nx);
+                if (m < nsteps) put(wb, k, nx);
                 const float2 cr = make_float2(c.x, c.y), ci = make_float2(c.z, c.w);
                 U[k & 1] = __ffma2_rn(ci, ci, __ffma2_rn(cr, cr, U[k & 1]));
                 Xr[k & 1] = __ffma2_rn(ci, im, __ffma2_rn(cr, re, Xr[k & 1]));
@@ -395,7 +446,6 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
                 prv[k] = nx;
             }
         }
-        pk_arrive(t.C);
         if (m > 0) {
             // class A: the sites of parity par_o + m; an even site has the parity of its row
             const bool ea = par_t == ((par_o + m) & 1);
@@ -405,147 +455,226 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
             v[2] = ea ? Xr[0].x + Xr[1].y : Xr[0].y + Xr[1].x;
             v[3] = ea ? Xi[0].x + Xi[1].y : Xi[0].y + Xi[1].x;
             const float s = warp_reduce_scatter4(v, lane);
-            if ((lane & 7) == 0) sums.w[m & 3][warp][lane >> 3] = s;
-            if (m >= 3 && warp == (m & (NW - 1))) pk_flush<float, NW>(p, sums, m - 2, lane);
+            if ((lane & 7) == 0) sums.w[m & (kPkRing - 1)][warp][lane >> 3] = s;
         }
+        // the sums come before the arrival: its release waits for the remote stores
+        // to be acknowledged (400-560 cycles on a cluster), which the sums cover
+        pk_arrive(t.C);
+        pk_flush_due<float, NW>(p, sums, m, warp, lane);
         pk_wait(t.C);
     };
     int m = 0;
-    for (; m + 1 <= p.nsteps; m += 2) {
+    for (; m + 1 <= nsteps; m += 2) {
         step(m, va, vb);
         step(m + 1, vb, va);
     }
-    if (m <= p.nsteps) step(m, va, vb);
+    if (m <= nsteps) step(m, va, vb);
     __syncthreads();
-    if (warp < 2 && p.nsteps - warp >= 1) pk_flush<float, NW>(p, sums, p.nsteps - warp, lane);
+    pk_flush_rest<float, NW>(p, sums, nsteps, warp, lane);
 }
 
 // ---------------------------------------------------------------------------
-// FP64 steps
+// FP64 chains: the recursion in fixed point with 60 fraction bits
 // ---------------------------------------------------------------------------
-// The FP64 pipe retires one warp instruction per sub-partition every 64 cycles
-// whatever the active lanes, so the step is dealt out in items (site, real or
-// imaginary part) of 12 multiply-adds, class by class so that the warps of
-// class A (which form <r_m^o|r_{m+1}^v> too) and of class B are apart; operands come from
-// shared memory, nothing is held in registers between steps.
-struct Pk64Site {
-    unsigned short ring, nat;  // ring index (row L + x), bond row index z PY + y
-    unsigned short x;
-    unsigned short face;       // 1: y = 0, 2: y = PY - 1, 4: z = 0, 8: z = PZ - 1
+// GB300's FP64 pipe retires 2 multiply-adds per clock and SM, its integer
+// multiplier about 55 32 x 32 + 64-bit multiply-adds (both measured).
+// |S_n(i)| <= 1 on every site (|T_n(Htilde)| <= 1, |v| <= |Delta~| < 0.82), so FP64
+// chains hold S, and 2 Htilde (|2 Htilde| < 0.34; finer than a double above 2^-8), in
+// units of 2^-60 as two limbs, x = xh 2^30 + xl with the low limb centred in
+// [-2^29, 2^29).  In the same units
+//     h s = hh sh + (hh sl + hl sh) 2^-30 + hl sl 2^-60,
+// three wide multiply-adds per real product; the last term, below a quarter
+// unit and of either sign, is left out.  A step rounds once, by half a unit
+// (4.3e-19); the FP64 recursion rounds 12 times, each by half a unit in the last
+// place of its partial sums (4.3e-19 where |S_n(i)| is near 2^-8, more above).
+// Bounds: sum over the six bonds of |hh sl| <= 2.9 2^59 and of |hl sh| <= 3.5 2^59
+// (Cauchy-Schwarz, |S_n| <= 1 on a class), so a sum of the middle products stays below 2^62.
+struct PkBond64 {
+    int rh, rl, ih, il;
+};
+__device__ __forceinline__ long long pk_join(int h, int l) { return ((long long)h << 30) + l; }
+// acc += x y, 32 x 32 + 64 bits in one instruction (left to the compiler, a good
+// part of the products came out as separate multiplies and additions: a step
+// of L = 32 on 128 CTAs 4466 -> 3529 cycles)
+__device__ __forceinline__ void pk_wide(long long& acc, int x, int y)
+{
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(x), "r"(y));
+}
+__device__ __forceinline__ void pk_mac(long long& A, long long& B, int hh, int hl, int sh, int sl)
+{
+    pk_wide(A, hh, sh);
+    pk_wide(B, hh, sl);
+    pk_wide(B, hl, sh);
+}
+// value of sums of limb products: A in units, B in units of 2^30
+__device__ __forceinline__ long long pk_value(long long A, long long B) { return A + ((B + (1ll << 29)) >> 30); }
+// Sums of one step over a thread's sites, in units of 2^-60: |S_m|^2 by class and
+// <S_m|S_{m+1}> over class A, as sums of limb products put together once per
+// step.  The squares keep the square of the low limb, which does not average
+// out; of the products of S_m and S_{m+1} it is left out.  Over the n sites of a thread
+// sum |sh| <= 2^30 sqrt(2 n): the middle sums stay below 2^62 and the low
+// squares (their upper halves, 32 bits) below 2^31 for n <= 8; threads with more
+// sites put their sums together every kPkPut sites.
+constexpr int kPkPut = 8;
+struct Pk64Sums {
+    long long v[4] = {0, 0, 0, 0};
+    long long A[2] = {0, 0}, B[2] = {0, 0};        // squares, by class (0: A)
+    int C[2] = {0, 0};
+    long long RA = 0, RB = 0, IA = 0, IB = 0;      // Re and Im of the products
+    template <int K> __device__ __forceinline__ void square(int h, int l)
+    {
+        pk_wide(A[K], h, h);
+        pk_wide(B[K], h, l);
+        C[K] += __mulhi(l, l);
+    }
+    __device__ __forceinline__ void add(int4 c, int4 n, bool a)
+    {
+        if (a) {
+            square<0>(c.x, c.y);
+            square<0>(c.z, c.w);
+            pk_mac(RA, RB, c.x, c.y, n.x, n.y);
+            pk_mac(RA, RB, c.z, c.w, n.z, n.w);
+            pk_mac(IA, IB, c.x, c.y, n.z, n.w);
+            pk_mac(IA, IB, -c.z, -c.w, n.x, n.y);
+        } else {
+            square<1>(c.x, c.y);
+            square<1>(c.z, c.w);
+        }
+    }
+    __device__ __forceinline__ void put()
+    {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            // (h 2^30 + l)^2 2^-60 = h^2 + 2 h l 2^-30 + l^2 2^-60
+            v[k] += A[k] + ((B[k] + 2ll * C[k] + (1ll << 28)) >> 29);
+            A[k] = B[k] = 0;
+            C[k] = 0;
+        }
+        v[2] += pk_value(RA, RB);
+        v[3] += pk_value(IA, IB);
+        RA = RB = IA = IB = 0;
+    }
 };
 
-template <int NT>
-__device__ __forceinline__ void pk64_table(const PkTile& t, Pk64Site* tab)
+// Large tiles on a cluster (more sites than gfmc_packed64.cuh takes): whole sites
+// per thread, dealt out class by class, everything in shared memory.  A ring
+// row holds its even sites first, then the odd ones, so that the sites a warp
+// reads are contiguous.
+struct Pk64Site {
+    int at;          // byte offset of the site in a ring buffer
+    int dxp, dxm;    // byte offsets of its x-neighbours
+    int bond;        // byte offset of its x bond
+    int y, z, x, cls;
+};
+__device__ __forceinline__ Pk64Site pk64_site(const PkTile& t, int s, int T2)
 {
-    const int T = t.L * t.PY * t.PZ, T2 = T / 2;
-    for (int s = threadIdx.x; s < T; s += NT) {
-        const int c = s >= T2 ? 1 : 0, g = s - c * T2, r = g / t.half, j = g - r * t.half;
-        const int z = r / t.PY, y = r - z * t.PY;
-        const int x = 2 * j + ((c + t.y0 + y + t.z0 + z) & 1);
-        Pk64Site q;
-        q.ring = (unsigned short)(t.ring_row(y, z) * t.L + x);
-        q.nat = (unsigned short)r;
-        q.x = (unsigned short)x;
-        q.face = (unsigned short)((y == 0 ? 1 : 0) | (y == t.PY - 1 ? 2 : 0) | (z == 0 ? 4 : 0) |
-                                  (z == t.PZ - 1 ? 8 : 0));
-        tab[s] = q;
+    Pk64Site q;
+    q.cls = s >= T2 ? 1 : 0;
+    const int g = s - q.cls * T2, r = g / t.half, j = g - r * t.half;
+    q.z = r / t.PY;
+    q.y = r - q.z * t.PY;
+    const int odd = (q.cls + t.y0 + q.y + t.z0 + q.z) & 1;
+    q.x = 2 * j + odd;
+    const int col = odd * t.half + j, other = (1 - odd) * t.half;
+    const int jp = odd ? (j == t.half - 1 ? 0 : j + 1) : j, jm = odd ? j : (j == 0 ? t.half - 1 : j - 1);
+    q.at = 16 * (t.ring_row(q.y, q.z) * t.L + col);
+    q.dxp = 16 * (other + jp - col);
+    q.dxm = 16 * (other + jm - col);
+    q.bond = 16 * (r * t.L + col);
+    return q;
+}
+// the six bonds of a site, backward ones conjugated: re += rr sr - ii si, im += rr si + ii sr
+__device__ __forceinline__ void pk64_bonds(const PkTile& t, const Pk64Site& q, PkBond64 (&h)[6])
+{
+    const char* b = t.bonds + q.bond;
+    const int rowB = (int)t.rowB, plane = t.PY * t.PZ;
+    const char* by = b + (plane + q.z + 1) * rowB;                       // row z (PY + 1) + y + 1 of BY
+    const char* bz = b + (plane + t.PZ * (t.PY + 1) + t.PY) * rowB;      // row (z + 1) PY + y of BZ
+    const char* at[6] = {b, b + q.dxm, by, by - rowB, bz, bz - t.PY * rowB};
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+        const int4 v = *(const int4*)at[d];
+        h[d] = (d & 1) ? PkBond64{v.x, v.y, -v.z, -v.w} : PkBond64{v.x, v.y, v.z, v.w};
     }
+}
+// 2 Htilde S_m - S_{m-1} at a site: re, im hold S_{m-1} and receive the value
+__device__ __forceinline__ void pk64_stencil(const int4 (&v)[6], const PkBond64 (&h)[6], long long& re, long long& im)
+{
+    long long PA = -re, PB = 0, NA = 0, NB = 0, QA = -im, QB = 0;
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+        pk_mac(PA, PB, h[d].rh, h[d].rl, v[d].x, v[d].y);
+        pk_mac(NA, NB, h[d].ih, h[d].il, v[d].z, v[d].w);
+        pk_mac(QA, QB, h[d].rh, h[d].rl, v[d].z, v[d].w);
+        pk_mac(QA, QB, h[d].ih, h[d].il, v[d].x, v[d].y);
+    }
+    re = pk_value(PA - NA, PB - NB);
+    im = pk_value(QA, QB);
 }
 
 template <int NT>
-__device__ __forceinline__ void pk64_steps(const Params& p, const PkTile& t, const int* s_loc, const double2* s_c,
-                                           PkSums<double, NT / 32>& sums, const Pk64Site* tab)
+__device__ __noinline__ void pk64_steps(const Params& p, const PkTile& tile, const int* s_loc, const double2* s_c,
+                                           PkSums<double, NT / 32>& sums)
 {
+    const PkTile t = tile;
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int L = t.L, T = L * t.PY * t.PZ, T2 = T / 2;
-    const int c = tid & 1;  // real or imaginary part (NT is even)
-    const unsigned flip = c ? 0u : 0x80000000u;  // sign of the Im h terms of a forward bond
-    const int rowY = 2 * L, rowZ = 2 * L * t.zstr;  // ring strides in doubles
-    const unsigned pushY = t.rowB * (unsigned)t.PY, pushZ = t.rowB * (unsigned)(t.zstr * t.PZ);
-    const unsigned bufD = t.bufB / 8;
-    double* ring = (double*)t.ringp;
-    auto put = [&](unsigned buf, const Pk64Site& q, double v) {
-        const unsigned at = buf * bufD + 2u * q.ring + (unsigned)c;
-        ring[at] = v;
-        if (q.face) {
-            const unsigned b = 8u * at;
-            if (q.face & 1) pk_st(t.r_ym + b + pushY, v);
-            if (q.face & 2) pk_st(t.r_yp + b - pushY, v);
-            if (q.face & 4) pk_st(t.r_zm + b + pushZ, v);
-            if (q.face & 8) pk_st(t.r_zp + b - pushZ, v);
-        }
+    const int rowB = (int)t.rowB, planeB = t.zstr * rowB;
+    const unsigned yB = t.rowB * (unsigned)t.PY, zB = t.rowB * (unsigned)(t.zstr * t.PZ);
+    auto put = [&](int buf, const Pk64Site& q, int4 v) {
+        const unsigned b = (unsigned)buf * t.bufB + (unsigned)q.at;
+        *(int4*)(t.ringp + b) = v;
+        pk_st(q.y == 0, t.r_ym + b + yB, v);
+        pk_st(q.y == t.PY - 1, t.r_yp + b - yB, v);
+        pk_st(q.z == 0, t.r_zm + b + zB, v);
+        pk_st(q.z == t.PZ - 1, t.r_zp + b - zB, v);
     };
-    for (int it = tid; it < 2 * T; it += NT) {
-        const Pk64Site q = tab[it >> 1];
-        const int z = q.nat / t.PY, y = q.nat - z * t.PY;
-        const double2 v = pk_s0(q.x + L * (t.y0 + y + L * (t.z0 + z)), s_loc, s_c);
-        put(0, q, c ? v.y : v.x);
+    for (int s = tid; s < T; s += NT) {
+        const Pk64Site q = pk64_site(t, s, T2);
+        const double2 v = pk_s0(q.x + L * (t.y0 + q.y + L * (t.z0 + q.z)), s_loc, s_c);
+        put(0, q, pk_limbs(__double2ll_rn(v.x * 0x1p60), __double2ll_rn(v.y * 0x1p60)));
     }
     pk_arrive(t.C);
-    pk_wait(t.C);
     const int lo = s_loc[0];
     const int par_o = (lo % L + (lo / L) % L + lo / (L * L)) & 1;
-    auto sgn = [&](double h, unsigned f) { return __hiloint2double(__double2hiint(h) ^ (int)f, __double2loint(h)); };
-
     for (int m = 0; m <= p.nsteps; ++m) {
-        const unsigned rb = (unsigned)(m & 1), wb = rb ^ 1u;
-        const double* rd = ring + rb * bufD;
-        const int clsA = (par_o + m) & 1;
-        double aA = 0.0, aB = 0.0, xr = 0.0, xi = 0.0;
-        for (int it = tid; it < 2 * T; it += NT) {
-            const int s = it >> 1;
-            const Pk64Site q = tab[s];
-            const double* r = rd + 2 * q.ring;
-            const int xp = q.x == L - 1 ? -2 * (L - 1) : 2, xm = q.x == 0 ? 2 * (L - 1) : -2;
-            const double2* bx = (const double2*)t.bonds + (size_t)q.nat * L + q.x;
-            const int z = q.nat / t.PY;
-            const double2* by = bx + (size_t)(t.PY * t.PZ + z + 1) * L;             // row z (PY + 1) + y + 1
-            const double2* bz = bx + (size_t)(t.PY * t.PZ + t.PZ * (t.PY + 1) + t.PY) * L;
-            double acc = m == 0 ? 0.0 : dneg(ring[wb * bufD + 2 * q.ring + c]);
-            auto fwd = [&](double2 h, const double* v) {
-                acc = fma(h.x, v[c], acc);
-                acc = fma(sgn(h.y, flip), v[1 - c], acc);
-            };
-            auto bwd = [&](double2 h, const double* v) {
-                acc = fma(h.x, v[c], acc);
-                acc = fma(sgn(h.y, flip ^ 0x80000000u), v[1 - c], acc);
-            };
-            fwd(bx[0], r + xp);
-            bwd(*(bx + xm / 2), r + xm);
-            fwd(by[0], r + rowY);
-            bwd(*(by - L), r - rowY);
-            fwd(bz[0], r + rowZ);
-            bwd(*(bz - (size_t)t.PY * L), r - rowZ);
-            if (m == 0) acc *= 0.5;
-            if (m < p.nsteps) put(wb, q, acc);
-            if (m > 0) {
-                const double u = r[c], w = r[1 - c];
-                if ((s >= T2) == (clsA != 0)) {
-                    aA = fma(u, u, aA);
-                    xr = fma(u, acc, xr);
-                    xi = fma(sgn(w, flip), acc, xi);  // Re S Im S' - Im S Re S'
-                } else {
-                    aB = fma(u, u, aB);
-                }
-            }
-        }
-        pk_arrive(t.C);
-        if (m > 0) {
-            bool o0, o1, o2, o3;
-            long long v[4] = {fixed58(aA, o0), fixed58(aB, o1), fixed58(xr, o2), fixed58(xi, o3)};
-            if (!(o0 && o1 && o2 && o3)) {
-                set_error(p, ERR_NUMERIC, 90, m);
-                v[0] = v[1] = v[2] = v[3] = 0;
-            }
-            const long long s = warp_reduce_scatter4(v, lane);
-            if ((lane & 7) == 0) sums.w[m & 3][warp][lane >> 3] = s;
-            if (m >= 3 && warp == (m & (NW - 1))) pk_flush<double, NW>(p, sums, m - 2, lane);
-        }
         pk_wait(t.C);
+        const int wb = (m + 1) & 1;
+        const char* rd = t.ringp + (m & 1) * t.bufB;
+        const char* wr = t.ringp + wb * t.bufB;
+        const int clsA = (par_o + m) & 1;
+        Pk64Sums acc;
+        int nadd = 0;
+        for (int s = tid; s < T; s += NT) {
+            const Pk64Site q = pk64_site(t, s, T2);
+            PkBond64 h[6];
+            pk64_bonds(t, q, h);
+            const int4 pv = *(const int4*)(wr + q.at), c = *(const int4*)(rd + q.at);
+            long long a = m == 0 ? 0 : pk_join(pv.x, pv.y), b = m == 0 ? 0 : pk_join(pv.z, pv.w);
+            const char* r = rd + q.at;
+            const int4 v[6] = {*(const int4*)(r + q.dxp),  *(const int4*)(r + q.dxm),    *(const int4*)(r + rowB),
+                               *(const int4*)(r - rowB), *(const int4*)(r + planeB), *(const int4*)(r - planeB)};
+            pk64_stencil(v, h, a, b);
+            if (m == 0) {  // S_1 = Htilde S_0
+                a = (a + 1) >> 1;
+                b = (b + 1) >> 1;
+            }
+            const int4 n = pk_limbs(a, b);
+            if (m < p.nsteps) put(wb, q, n);
+            acc.add(c, n, q.cls == clsA);
+            if (++nadd % kPkPut == 0) acc.put();
+        }
+        acc.put();
+        if (m > 0) {
+            const long long s = warp_reduce_scatter4(acc.v, lane);
+            if ((lane & 7) == 0) sums.w[m & (kPkRing - 1)][warp][lane >> 3] = s;
+        }
+        if (m < p.nsteps) pk_arrive(t.C);
+        pk_flush_due<double, NW>(p, sums, m, warp, lane);
     }
     __syncthreads();
-    if (warp < 2 && p.nsteps - warp >= 1) pk_flush<double, NW>(p, sums, p.nsteps - warp, lane);
+    pk_flush_rest<double, NW>(p, sums, p.nsteps, warp, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -591,7 +720,7 @@ __device__ __forceinline__ void pk_tail_fft(const Params& p, int rank, int C, do
                 double a = first;
                 if (pp > 0) {
                     const long long s = (long long)__ldcg(p.gram + (size_t)(pp - 1) * kEntries + (V < 2 ? V : V + 4));
-                    a = fma((double)s, 0x1p-57, -first);  // 2 <.|.> - mu_0 (or mu_1)
+                    a = fma((double)s, 0x1p-59, -first);  // 2 <.|.> - mu_0 (or mu_1)
                 }
                 a *= __ldg(p.gker + nn) * (nn == 0 ? 0.5 : 1.0);
                 double2 w = __ldg(p.twc + 2 * pp);
@@ -684,6 +813,130 @@ __device__ __forceinline__ void pk_tail_phase(const Params& p, int rank, int C, 
     }
 }
 
+// the chain's sums have been read: clear them for the next update
+template <int NT> __device__ __forceinline__ void pk_tail_clear(const Params& p, int rank, int C)
+{
+    for (int e = rank * NT + (int)threadIdx.x; e < 4 * p.nsteps; e += C * NT) {
+        const int v = e & 3;
+        __stcg(p.gram + (size_t)(e >> 2) * kEntries + (v < 2 ? v : v + 4), 0ull);
+    }
+}
+
+// What an update starts from and ends with, in shared memory.
+struct PkHead {
+    double2 c[kVec], hop[kVec];  // Delta~ |o> and Htilde_{o, l_k} at the local sites
+    double chi[8][3];            // spinors of the local sites and of the proposal
+    int loc[kVec];
+    double draw[3];
+    double vv0;                  // <v|v>
+    double2 ov1;                 // <o|Htilde|v>
+    int acc;
+};
+
+// Local sites, proposal and Delta~ by warp 0, one sincos per lane (lane k the
+// polar, lane 8 + k the azimuthal angle): the FP64 pipe takes 64 cycles per
+// warp instruction, so seven threads with six sincos each took six times as
+// long.  The caller's barrier follows.
+__device__ __forceinline__ void pk_setup(const Params& p, PkHead& h, int o, unsigned long long upd)
+{
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x, k = lane & 7;
+    const int lk = k == 0 ? o : nbr_site(o, min(k, 6) - 1, p.L);
+    double th = p.theta_new, ph = p.phi_new, u = 0.0;
+    if (p.mode == MODE_SWEEP) draw_update(p.seed, p.chain_id, upd, th, ph, u);
+    if (lane == 7) {
+        h.draw[0] = th;
+        h.draw[1] = ph;
+        h.draw[2] = u;
+    }
+    if (k < 7) {
+        th = __ldcg(p.spins + 2 * lk);
+        ph = __ldcg(p.spins + 2 * lk + 1);
+    }
+    double sn, cs;
+    sincos((lane & 8) ? ph : 0.5 * th, &sn, &cs);
+    const double sp = __shfl_sync(0xffffffffu, sn, k + 8), cp = __shfl_sync(0xffffffffu, cs, k + 8);
+    if (lane < 8) {
+        h.chi[k][0] = cs;
+        h.chi[k][1] = cp * sn;
+        h.chi[k][2] = sp * sn;
+    }
+    if (lane < 7) h.loc[lane] = lk;
+    __syncwarp();
+    double2 cv = make_double2(0.0, 0.0), hv = cv;
+    if (lane > 0 && lane < 7) {
+        // Delta~_{l_j,o} = -t (<chi_j|chi'_o> - <chi_j|chi_o>) / a
+        const double* cj = h.chi[lane];
+        const double2 on = overlap3(cj[0], cj[1], cj[2], h.chi[7][0], h.chi[7][1], h.chi[7][2]);
+        const double2 oo = overlap3(cj[0], cj[1], cj[2], h.chi[0][0], h.chi[0][1], h.chi[0][2]);
+        cv = make_double2((-p.t * on.x + p.t * oo.x) / p.a, (-p.t * on.y + p.t * oo.y) / p.a);
+        hv = hop_of(p.hop64, p.N, o, lane - 1, lk);  // Htilde_{o, l_k}
+    }
+    if (lane < 7) h.c[lane] = cv;
+    // <v|v> and <o|Htilde|v> = sum_k Htilde_{o, l_k} c_k over lanes 1..6
+    double v0 = cv.x * cv.x + cv.y * cv.y;
+    double2 o1 = dmul(cv, hv);
+#pragma unroll
+    for (int b = 4; b > 0; b >>= 1) {
+        v0 += __shfl_xor_sync(0xffffffffu, v0, b);
+        o1.x += __shfl_xor_sync(0xffffffffu, o1.x, b);
+        o1.y += __shfl_xor_sync(0xffffffffu, o1.y, b);
+    }
+    if (lane == 0) {
+        h.vv0 = v0;
+        h.ov1 = o1;
+    }
+}
+
+// Delta Omega from the CTAs' phase sums (added in one order by every CTA) and
+// the Metropolis decision, by warp 0; the caller's barrier follows.
+__device__ __forceinline__ void pk_decide(const Params& p, PkHead& h, int rank, long long q)
+{
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    double s = 0.0, mx = 0.0;
+    for (int c = lane; c < p.ncta; c += 32) {
+        s += __ldcg(p.qpart + 2 * c);
+        mx = fmax(mx, __ldcg(p.qpart + 2 * c + 1));
+    }
+#pragma unroll
+    for (int b = 16; b > 0; b >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, b);
+        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, b));
+    }
+    if (lane == 0) {
+        const double dom = p.a / p.K * s;
+        int acc = 0;
+        if (p.mode == MODE_SWEEP) acc = exp(-p.beta * dom) > h.draw[2];
+        h.acc = acc;
+        if (rank == 0) {
+            const long long slot = (p.mode == MODE_SWEEP) ? q : 0;
+            p.domega_out[slot] = dom;
+            if (p.maxinc_out) p.maxinc_out[slot] = mx;
+            if (p.mode == MODE_SWEEP && p.dec_out) p.dec_out[q] = (unsigned char)acc;
+        }
+    }
+}
+
+// |sum_i S_i| / N after a sweep; sync(where): the chain's barrier.
+template <int NT, class Sync>
+__device__ __forceinline__ bool pk_magnetisation(const Params& p, int rank, long long nmag, Sync& sync)
+{
+    const int C = p.ncta, N = p.N;
+    magnetisation_partial<NT>(p, (int)((long long)rank * N / C), (int)((long long)(rank + 1) * N / C), rank);
+    if (!sync(6)) return false;
+    if (rank == 0 && threadIdx.x == 0) {
+        double X = 0.0, Y = 0.0, Z = 0.0;
+        for (int c = 0; c < C; ++c) {
+            X += __ldcg(p.magpart + 3 * c);
+            Y += __ldcg(p.magpart + 3 * c + 1);
+            Z += __ldcg(p.magpart + 3 * c + 2);
+        }
+        p.mag_out[nmag] = sqrt(X * X + Y * Y + Z * Z) / N;
+    }
+    return sync(7);  // magpart is read before the next sweep's partials
+}
+
 // ---------------------------------------------------------------------------
 // one chain on a cluster
 // ---------------------------------------------------------------------------
@@ -693,161 +946,66 @@ template <class R> __device__ __forceinline__ void pk_run_chain(const Params& p,
 {
     constexpr int NT = pk_threads<R>(), NW = NT / 32;
     __shared__ PkSums<R, NW> sums;
-    __shared__ double2 s_c[kVec], s_hop[kVec];
-    __shared__ double s_chi[8][3];
-    __shared__ int s_loc[kVec];
-    __shared__ double s_draw[3];
-    __shared__ double s_vv0;
-    __shared__ double2 s_ov1;
-    __shared__ int s_acc;
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int N = p.N, L = p.L, C = p.ncta;
-    const PkTile t = pk_tile<R>(p, rank, smem);
+    __shared__ PkHead head;
+    const int tid = threadIdx.x, N = p.N, C = p.ncta;
+    __shared__ PkTile t;
+    if (tid == 0) t = pk_tile<R>(p, rank, smem);
+    __syncthreads();
     double2* work = (double2*)smem;
-    const int work_n = pk_work_bytes(L, t.PY, t.PZ, p.K, sizeof(R) == 4) / (int)sizeof(double2);
-    [[maybe_unused]] Pk64Site* tab = (Pk64Site*)(t.bonds + (size_t)t.bond_rows() * t.rowB);
-    if constexpr (sizeof(R) == 8) pk64_table<NT>(t, tab);
+    const int work_n = (int)((t.bonds - smem) / (int)sizeof(double2));
+    auto sync = [&](int) {
+        if (C > 1) cooperative_groups::this_cluster().sync();
+        else __syncthreads();
+        return true;
+    };
+    sync(0);  // every CTA of the cluster has started before any remote store
+
     const long long nupd = (p.mode == MODE_SWEEP) ? p.n_updates : 1;
     long long nmag = 0;
     unsigned long long nacc = 0;
     bool reload = true;
-    auto sync = [&]() {
-        if (C > 1) cl.sync();
-        else __syncthreads();
-    };
-    sync();  // every CTA of the cluster has started before any remote store
-
     for (long long q = 0; q < nupd; ++q) {
         const unsigned long long upd = p.upd0 + (unsigned long long)q;
         const int o = (p.mode == MODE_SWEEP) ? (int)(upd % (unsigned long long)N) : (int)p.site;
-        // ---- set-up: the spinors of the 7 local sites and of the proposal, a
-        //      sincos per lane of warp 0 (lane k the polar, lane 8 + k the azimuthal angle) ----
-        if (warp == 0) {
-            const int k = lane & 7;
-            const int lk = k == 0 ? o : nbr_site(o, min(k, 6) - 1, L);
-            double th = p.theta_new, ph = p.phi_new, u = 0.0;
-            if (p.mode == MODE_SWEEP) draw_update(p.seed, p.chain_id, upd, th, ph, u);
-            if (lane == 7) {
-                s_draw[0] = th;
-                s_draw[1] = ph;
-                s_draw[2] = u;
-            }
-            if (k < 7) {
-                th = __ldcg(p.spins + 2 * lk);
-                ph = __ldcg(p.spins + 2 * lk + 1);
-            }
-            double sn, cs;
-            sincos((lane & 8) ? ph : 0.5 * th, &sn, &cs);
-            const double sp = __shfl_sync(0xffffffffu, sn, k + 8), cp = __shfl_sync(0xffffffffu, cs, k + 8);
-            if (lane < 8) {
-                s_chi[k][0] = cs;
-                s_chi[k][1] = cp * sn;
-                s_chi[k][2] = sp * sn;
-            }
-            if (lane < 7) s_loc[lane] = lk;
-            __syncwarp();
-            if (lane < 7) {
-                double2 cv = make_double2(0.0, 0.0), hv = cv;
-                if (lane > 0) {
-                    // Delta~_{l_j,o} = -t (<chi_j|chi'_o> - <chi_j|chi_o>) / a
-                    const double* cj = s_chi[lane];
-                    const double2 on = overlap3(cj[0], cj[1], cj[2], s_chi[7][0], s_chi[7][1], s_chi[7][2]);
-                    const double2 oo = overlap3(cj[0], cj[1], cj[2], s_chi[0][0], s_chi[0][1], s_chi[0][2]);
-                    cv = make_double2((-p.t * on.x + p.t * oo.x) / p.a, (-p.t * on.y + p.t * oo.y) / p.a);
-                    hv = hop_of(p.hop64, N, o, lane - 1, lk);  // Htilde_{o, l_k}
-                }
-                s_c[lane] = cv;
-                s_hop[lane] = hv;
-            }
-        }
+        pk_setup(p, head, o, upd);
         if (reload) pk_load_bonds<R, NT>(p, t);
         reload = false;
         __syncthreads();
-
-        // ---- the recursion ----
         if constexpr (sizeof(R) == 4) {
             const int ncol = t.half * t.PY, room = NT / ncol;
             const int nseg0 = min(room, t.PZ), S = (t.PZ + nseg0 - 1) / nseg0, nseg = (t.PZ + S - 1) / S;
-            if (S == 1) pk32_steps<NT, 1, true>(p, t, s_loc, s_c, sums, nseg);
-            else if (S == 2) pk32_steps<NT, 2, true>(p, t, s_loc, s_c, sums, nseg);
-            else if (S == 3) pk32_steps<NT, 3, false>(p, t, s_loc, s_c, sums, nseg);
-            else pk32_steps<NT, 4, false>(p, t, s_loc, s_c, sums, nseg);
+            if (S == 1) pk32_steps<NT, 1, true>(p, t, head.loc, head.c, sums, nseg);
+            else if (S == 2) pk32_steps<NT, 2, true>(p, t, head.loc, head.c, sums, nseg);
+            else if (S == 3) pk32_steps<NT, 3, false>(p, t, head.loc, head.c, sums, nseg);
+            else pk32_steps<NT, 4, false>(p, t, head.loc, head.c, sums, nseg);
         } else {
-            pk64_steps<NT>(p, t, s_loc, s_c, sums, tab);
+            pk64_steps<NT>(p, t, head.loc, head.c, sums);
         }
-        if (tid == 0) {
-            double v0 = 0.0;
-            double2 o1 = make_double2(0.0, 0.0);
-            for (int k = 1; k < 7; ++k) {
-                v0 += s_c[k].x * s_c[k].x + s_c[k].y * s_c[k].y;  // <v|v>
-                o1 = dadd(o1, dmul(s_c[k], s_hop[k]));            // <o|Htilde|v>
-            }
-            s_vv0 = v0;
-            s_ov1 = o1;
-        }
-        sync();
-
-        // ---- FFT to the nodes, phases, Delta Omega, decision ----
-        pk_tail_fft<NT>(p, rank, C, work, work_n, s_vv0, s_ov1);
-        sync();
-        for (int e = rank * NT + tid; e < 4 * p.nsteps; e += C * NT) {  // the sums are read: clear them
-            const int v = e & 3;
-            __stcg(p.gram + (size_t)(e >> 2) * kEntries + (v < 2 ? v : v + 4), 0ull);
-        }
+        sync(1);
+        pk_tail_fft<NT>(p, rank, C, work, work_n, head.vv0, head.ov1);
+        sync(2);
+        pk_tail_clear<NT>(p, rank, C);
         pk_tail_phase<NT>(p, rank, C, (double*)work);
-        sync();
-        if (warp == 0) {
-            double s = lane < C ? __ldcg(p.qpart + 2 * lane) : 0.0;
-            double mx = lane < C ? __ldcg(p.qpart + 2 * lane + 1) : 0.0;
-#pragma unroll
-            for (int b = 8; b > 0; b >>= 1) {
-                s += __shfl_xor_sync(0xffffffffu, s, b);
-                mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, b));
-            }
-            if (lane == 0) {
-                const double dom = p.a / p.K * s;
-                int acc = 0;
-                if (p.mode == MODE_SWEEP) acc = exp(-p.beta * dom) > s_draw[2];
-                s_acc = acc;
-                if (rank == 0) {
-                    const long long slot = (p.mode == MODE_SWEEP) ? q : 0;
-                    p.domega_out[slot] = dom;
-                    if (p.maxinc_out) p.maxinc_out[slot] = mx;
-                    if (p.mode == MODE_SWEEP && p.dec_out) p.dec_out[q] = (unsigned char)acc;
-                }
-            }
-        }
+        sync(3);
+        pk_decide(p, head, rank, q);
         __syncthreads();
         if (p.mode == MODE_DELTA) break;
-        if (s_acc) {
+        if (head.acc) {
             ++nacc;
             reload = true;
-            if (rank == 0 && tid < 7) patch_site(p, o, s_loc, s_draw[0], s_draw[1], tid);
-            sync();
+            if (rank == 0 && tid < 7) patch_site(p, o, head.loc, head.draw[0], head.draw[1], tid);
+            sync(5);
         }
         if ((upd + 1ull) % (unsigned long long)N == 0ull) {
-            magnetisation_partial<NT>(p, (int)((long long)rank * N / C), (int)((long long)(rank + 1) * N / C), rank);
-            sync();
-            if (rank == 0 && tid == 0) {
-                double X = 0.0, Y = 0.0, Z = 0.0;
-                for (int c = 0; c < C; ++c) {
-                    X += __ldcg(p.magpart + 3 * c);
-                    Y += __ldcg(p.magpart + 3 * c + 1);
-                    Z += __ldcg(p.magpart + 3 * c + 2);
-                }
-                p.mag_out[nmag] = sqrt(X * X + Y * Y + Z * Z) / N;
-            }
+            pk_magnetisation<NT>(p, rank, nmag, sync);
             ++nmag;
-            sync();  // magpart is read before the next sweep's partials
         }
     }
     if (rank == 0 && tid == 0 && p.mode == MODE_SWEEP) {
         *p.n_acc = nacc;
         *p.n_mag = nmag;
     }
-    sync();  // no CTA leaves while another may still write into its shared memory
+    sync(0);  // no CTA leaves while another may still write into its shared memory
 }
 
 // A batch of chains, one thread-block cluster per chain (cluster size = the

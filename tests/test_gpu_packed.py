@@ -58,3 +58,42 @@ def test_packed_clusters_match_oracle(G, precision, tol, tie):
         replay(L, sps[c], M, nodes, c, outs[c], tol, tie)
     for ch in chains:
         ch.close()
+
+
+@pytest.mark.parametrize("L,M,n", [(4, 64, 80), (6, 128, 12), (10, 64, 12), (14, 32, 12), (16, 64, 10), (18, 16, 10),
+                                   (20, 32, 8), (24, 16, 8), (34, 16, 4), (48, 16, 3)])
+def test_fp64_single_chains_match_oracle(G, L, M, n):
+    """FP64 chains on the automatic engine, the fixed-point recursion: one
+    cluster (parts of sites and whole sites per thread, a cluster of 6, 10 or 14
+    CTAs) and the whole grid (pencils of one to sixteen rows, of unequal size,
+    1 to 3 sites per thread), a full sweep with its magnetisation, Delta Omega of
+    a given proposal, and a rerun bit for bit."""
+    sp = inputs.von_mises_fisher(L, 2.0, L)
+    kw = dict(M=M, beta=12.0, mu=-2.0, seed=5, chain_id=3)
+    tol, tie = lambda r: 1e-10 * abs(r) + 1e-13 * A, 1e-9
+    with G.Chain(L, sp, **kw) as ch:
+        o = L ** 3 // 2 + 3
+        d, ref = ch.delta_omega(o, 1.1, 2.3), O.delta_omega(L, sp, o, 1.1, 2.3, M, beta=12.0, chem=-2.0)
+        assert abs(d - ref) <= tol(ref)
+        out = ch.updates(n)
+        replay(L, sp, M, 0, 3, out, tol, tie)
+        assert out["magnetization"].size == n // L ** 3
+    with G.Chain(L, sp, **kw) as ch:
+        again = ch.updates(n)
+    assert np.array_equal(again["d_omega"], out["d_omega"])
+
+
+def test_packed_grid_wait_runs_out(G):
+    """A chain on the whole grid whose CTA 0 sends no face values: the bounded
+    waits of its neighbours end the launch with GFMC_ETIMEOUT, and the chain then
+    runs on as if nothing had happened."""
+    L, M, n = 20, 16, 6
+    sp = inputs.uniform_sphere(L, 1)
+    with G.Chain(L, sp, M=M, seed=3) as a, G.Chain(L, sp, M=M, seed=3) as b:
+        a.set_wait_budget(20_000_000)
+        a.inject_stall(True)
+        with pytest.raises(G.GfmcError) as e:
+            a.updates(n)
+        assert e.value.status == G.GFMC_ETIMEOUT
+        a.set_wait_budget(4_000_000_000)
+        assert np.array_equal(a.updates(n)["d_omega"], b.updates(n)["d_omega"])
