@@ -31,6 +31,8 @@ struct gfmc_ctx {
     // FP32-mixed L = 32 chain on seven thread-block clusters (one per unit
     // vector): single-chain calls on the unit-vector recursion use it
     bool vcl = false;
+    // the engine, and the CTAs of a single chain, were left to the library
+    bool auto_engine = false, auto_ctas = false;
     // even lattices on the automatic engine: Delta Omega calls run the packed
     // recursion on one cluster (1) or on the whole grid (2); 0: another engine
     int pk = 0, pk_engine = 0, pk_ctas = 0, pk_cy = 0, pk_cz = 0, pk_smem = 0;
@@ -218,6 +220,39 @@ gfmc_status ensure_trace(gfmc_ctx* h, long long n)
     return GFMC_OK;
 }
 
+// Vectors the Delta Omega recursion of a chain on a team of CTAs runs on: the
+// proposal's two for a chain on that recursion, and where the engine was left to
+// the library (its Delta Omega is the same function of those four moment
+// sequences); else the seven unit vectors.
+int team_nv(const gfmc_ctx* h)
+{
+    return h->recursion == GFMC_RECURSION_PROPOSAL || h->auto_engine ? 2 : gfmc::kVec;
+}
+
+// Shared memory a team CTA of chain h needs for its vectors, or SIZE_MAX when
+// they stay in global memory.  Even lattices on the proposal's vectors: the packed
+// vector on the CTA's sites and the planes beside them (a tile of a plane at least:
+// the planes' values then come from the CTAs it waits for); else one-CTA teams
+// only, every vector on the whole lattice.
+size_t team_vec_bytes(const gfmc_ctx* h, int tc)
+{
+    const size_t vsz = h->precision == GFMC_PREC_FP64 ? sizeof(double2) : sizeof(float2);
+    const int nv = team_nv(h), LL = h->L * h->L;
+    if (nv == 2 && h->L % 2 == 0 && !h->P.comp) {
+        if (tc > 1 && h->N / tc < LL) return SIZE_MAX;
+        return 2 * (size_t)std::min(h->N, (h->N + tc - 1) / tc + 2 * LL) * vsz;
+    }
+    return tc <= 1 ? 2 * (size_t)nv * h->N * vsz : SIZE_MAX;
+}
+
+// the vectors of every job's recursion, 0 when they differ
+int common_nv(const std::vector<gfmc::TeamJob>& jobs)
+{
+    for (const auto& j : jobs)
+        if (j.p.nv != jobs[0].p.nv) return 0;
+    return jobs[0].p.nv;
+}
+
 // Run one engine launch and wait for it; translate the device error word.
 gfmc_status run_engine(gfmc_ctx* h, Params& P)
 {
@@ -230,6 +265,10 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
     P.budget = h->budget;
     P.stall = h->stall_next;
     h->stall_next = 0;
+    // the moments need the seven unit vectors; so does the vector clusters' engine
+    const int nv = P.mode != gfmc::MODE_MOMENTS &&
+                           (h->recursion == GFMC_RECURSION_PROPOSAL || (h->auto_engine && h->auto_ctas && !h->vcl))
+                       ? 2 : gfmc::kVec;
     // a cluster of the packed engine has no flags to withhold: the stall hook runs the grid engine
     const bool packed = h->pk != 0 && P.mode != gfmc::MODE_MOMENTS && !(P.stall && h->pk == 1);
     if (packed) {
@@ -246,7 +285,7 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
         }
     } else if (h->multi_site) {
         gfmc::TeamJob job{};
-        P.nv = (h->recursion == GFMC_RECURSION_PROPOSAL && P.mode != gfmc::MODE_MOMENTS) ? 2 : gfmc::kVec;
+        P.nv = nv;
         job.p = P;
         job.cta0 = 0;
         job.vec_smem = 0;
@@ -254,9 +293,8 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
             return cuda_fail(h, e, "uploading the job");
         const int smem = gfmc::engine_smem_bytes(P.K);
         e = h->precision == GFMC_PREC_FP64 ? gfmc::launch_team_f64(h->d_job, 1, P.ncta, 0, smem, h->stream)
-                                            : gfmc::launch_team_f32(h->d_job, 1, P.ncta, 0, smem, h->stream, P.comp != 0);
+                                            : gfmc::launch_team_f32(h->d_job, 1, P.ncta, 0, smem, h->stream, P.comp != 0, nv);
     } else {
-        const int nv = (h->recursion == GFMC_RECURSION_PROPOSAL && P.mode != gfmc::MODE_MOMENTS) ? 2 : gfmc::kVec;
         if (h->vcl && nv == gfmc::kVec)
             e = gfmc::launch_vcluster_f32(P, h->stream);
         else
@@ -573,9 +611,9 @@ gfmc_status gfmc_create(int L, const double* spins, double t, double mu, double 
         prefetch = gfmc::single_smem_bytes(K, GFMC_PREC_FP64, win_max) + static_smem <= dev_smem;
     }
 
-    if (opt.engine == GFMC_ENGINE_AUTO && opt.num_ctas <= 0 && !opt.compensated &&
-        (st = plan_packed(h)) != GFMC_OK)
-        return bail(st);
+    h->auto_engine = opt.engine == GFMC_ENGINE_AUTO && !opt.compensated;
+    h->auto_ctas = opt.num_ctas <= 0;
+    if (h->auto_engine && h->auto_ctas && (st = plan_packed(h)) != GFMC_OK) return bail(st);
 
     Params& P = h->P;
     P.L = L;
@@ -846,21 +884,19 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = cudaSetDevice(dev)) != cudaSuccess) return cuda_fail(nullptr, e, "cudaSetDevice");
-    const size_t vsz = prec == GFMC_PREC_FP64 ? sizeof(double2) : sizeof(float2);
     // Shared memory: the largest resident lattice plus the work area of the largest M.
     int work = 0;
     for (int c = 0; c < n_chains; ++c) work = std::max(work, gfmc::engine_smem_bytes(chains[c]->K));
     int dev_smem = 0;
     if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
         return cuda_fail(nullptr, e, "querying shared memory");
-    const int reserve = 20 * 1024;  // static shared memory of the kernel and the parameter copy
+    const int reserve = 24 * 1024;  // static shared memory of the kernel and the parameter copy
     size_t vec_bytes = 0;
     std::vector<int> resident(n_chains, 0);
     for (int c = 0; c < n_chains; ++c) {
         const int tc = team_ctas ? team_ctas[c] : 1;
-        const int nvc = chains[c]->recursion == GFMC_RECURSION_PROPOSAL ? 2 : gfmc::kVec;
-        const size_t vb = 2 * (size_t)nvc * chains[c]->N * vsz;
-        if (tc <= 1 && vb + work + reserve <= (size_t)dev_smem) {
+        const size_t vb = team_vec_bytes(chains[c], std::max(tc, 1));
+        if (vb != SIZE_MAX && vb + work + reserve <= (size_t)dev_smem) {
             resident[c] = 1;
             vec_bytes = std::max(vec_bytes, (vb + 255) & ~(size_t)255);
         }
@@ -900,7 +936,7 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
         P.n_mag = h->d_nmag;
         P.budget = h->budget;
         P.stall = 0;
-        P.nv = h->recursion == GFMC_RECURSION_PROPOSAL ? 2 : gfmc::kVec;
+        P.nv = team_nv(h);
         jobs[c].p = P;
         if (given > 0) {
             last0 = cta0;
@@ -927,7 +963,7 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
         return cuda_fail(nullptr, e, "uploading the job table");
     e = prec == GFMC_PREC_FP64 ? gfmc::launch_team_f64(d_jobs, n_chains, grid, (int)vec_bytes, smem, s)
                                : gfmc::launch_team_f32(d_jobs, n_chains, grid, (int)vec_bytes, smem, s,
-                                                       chains[0]->P.comp != 0);
+                                                       chains[0]->P.comp != 0, common_nv(jobs));
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "launching the batch");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(nullptr, e, "batch execution");
     gfmc_status result = GFMC_OK;
@@ -1426,16 +1462,14 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
             groups.push_back(g);
         }
     } else {
-        const size_t vsz = prec == GFMC_PREC_FP64 ? sizeof(double2) : sizeof(float2);
         int work = 0;
         for (int c = 0; c < n_chains; ++c) work = std::max(work, gfmc::engine_smem_bytes(chains[c]->K));
-        const int reserve = 20 * 1024;
+        const int reserve = 24 * 1024;
         size_t vec_bytes = 0;
         std::vector<int> resident(n_chains, 0);
         for (int c = 0; c < n_chains; ++c) {
-            const int nvc = chains[c]->recursion == GFMC_RECURSION_PROPOSAL ? 2 : gfmc::kVec;
-            const size_t vb = 2 * (size_t)nvc * chains[c]->N * vsz;
-            if (ctas[c] <= 1 && vb + work + reserve <= (size_t)dev_smem) {
+            const size_t vb = team_vec_bytes(chains[c], std::max(ctas[c], 1));
+            if (vb != SIZE_MAX && vb + work + reserve <= (size_t)dev_smem) {
                 resident[c] = 1;
                 vec_bytes = std::max(vec_bytes, (vb + 255) & ~(size_t)255);
             }
@@ -1461,7 +1495,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
             P.tile_start = h->d_team_tiles;
             P.nbr_ptr = h->d_team_nptr;
             P.nbr_idx = h->d_team_nidx;
-            P.nv = h->recursion == GFMC_RECURSION_PROPOSAL ? 2 : gfmc::kVec;
+            P.nv = team_nv(h);
             gfmc::TeamJob j{};
             j.p = P;
             if (ctas[c] > 0) {
@@ -1511,7 +1545,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
     if (ce == cudaSuccess && !clusters) {
         ce = prec == GFMC_PREC_FP64 ? gfmc::launch_team_ex_f64(p->d_jobs, nj, team_grid, team_vec, team_smem, cs)
                                     : gfmc::launch_team_ex_f32(p->d_jobs, nj, team_grid, team_vec, team_smem, cs,
-                                                               chains[0]->P.comp != 0);
+                                                               chains[0]->P.comp != 0, common_nv(jobs));
     } else if (ce == cudaSuccess) {
         cudaEvent_t fork = nullptr;
         ce = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
@@ -1774,7 +1808,7 @@ gfmc_status gfmc_server_submit(gfmc_server_t s, int slot, gfmc_t h, int64_t n_up
     P.n_mag = h->d_nmag;
     P.budget = h->budget;
     P.stall = 0;
-    P.nv = h->recursion == GFMC_RECURSION_PROPOSAL ? 2 : gfmc::kVec;
+    P.nv = h->recursion == GFMC_RECURSION_PROPOSAL ? 2 : gfmc::kVec;  // a served job runs the recursion its chain names
     // Clear the chain's control words and post the job with copies only: a
     // memset kernel could wait for an SM the running server occupies.
     static const unsigned zeros[256] = {};

@@ -1,6 +1,8 @@
 // FP32-mixed instantiations of the GFMC engines: FP32 recursion vectors and
 // stencil, Gram dot products summed in FP32 within a warp (plain, or
 // compensated when comp is set) and in FP64 above.
+#include <algorithm>
+
 #include "gfmc_engine.cuh"
 
 namespace gfmc {
@@ -47,15 +49,15 @@ cudaError_t engine_max_ctas_f32(int K, int* out)
     return e;
 }
 
-template <bool COMP>
+template <int NV, bool COMP>
 static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
                                bool ex)
 {
-    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<float, COMP>);
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<float, NV, COMP>);
     if (e != cudaSuccess) return e;
     if (!ex) {
         void* args[] = {(void*)&d_jobs, (void*)&njobs, (void*)&vec_bytes};
-        return cudaLaunchCooperativeKernel((void*)gfmc_team_engine<float, COMP>, dim3(grid), dim3(kThreads), args,
+        return cudaLaunchCooperativeKernel((void*)gfmc_team_engine<float, NV, COMP>, dim3(grid), dim3(kThreads), args,
                                            (size_t)smem, s);
     }
     // the same launch through cudaLaunchKernelEx with the cooperative attribute,
@@ -70,37 +72,47 @@ static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int v
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<float, COMP>, d_jobs, njobs, vec_bytes);
+    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<float, NV, COMP>, d_jobs, njobs, vec_bytes);
+}
+
+static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
+                               bool comp, int nv, bool ex)
+{
+    if (comp) return team_launch<0, true>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
+    if (nv == 2) return team_launch<2, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
+    if (nv == kVec) return team_launch<kVec, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
+    return team_launch<0, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
 }
 
 cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
-                            bool comp)
+                            bool comp, int nv)
 {
-    return comp ? team_launch<true>(d_jobs, njobs, grid, vec_bytes, smem, s, false)
-                : team_launch<false>(d_jobs, njobs, grid, vec_bytes, smem, s, false);
+    return team_launch(d_jobs, njobs, grid, vec_bytes, smem, s, comp, nv, false);
 }
 
 cudaError_t launch_team_ex_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
-                               bool comp)
+                               bool comp, int nv)
 {
-    return comp ? team_launch<true>(d_jobs, njobs, grid, vec_bytes, smem, s, true)
-                : team_launch<false>(d_jobs, njobs, grid, vec_bytes, smem, s, true);
+    return team_launch(d_jobs, njobs, grid, vec_bytes, smem, s, comp, nv, true);
 }
 
-template <bool COMP>
+template <int NV, bool COMP>
 static cudaError_t team_occupancy(int smem, int* out)
 {
-    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<float, COMP>);
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<float, NV, COMP>);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, gfmc_team_engine<float, COMP>, kThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, gfmc_team_engine<float, NV, COMP>, kThreads, smem);
 }
 
+// of the kernel that holds the fewest, so that a batch fits whichever it runs
 cudaError_t team_max_ctas_f32(int smem, int* out)
 {
-    int a = 0, b = 0;
-    cudaError_t e = team_occupancy<false>(smem, &a);
-    if (e == cudaSuccess) e = team_occupancy<true>(smem, &b);
-    if (e == cudaSuccess) *out = a < b ? a : b;
+    int n[4] = {};
+    cudaError_t e = team_occupancy<0, false>(smem, &n[0]);
+    if (e == cudaSuccess) e = team_occupancy<0, true>(smem, &n[1]);
+    if (e == cudaSuccess) e = team_occupancy<2, false>(smem, &n[2]);
+    if (e == cudaSuccess) e = team_occupancy<kVec, false>(smem, &n[3]);
+    if (e == cudaSuccess) *out = std::min(std::min(n[0], n[1]), std::min(n[2], n[3]));
     return e;
 }
 

@@ -56,17 +56,17 @@ namespace gfmc {
 
 cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s)
 {
-    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double>);
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double, 0>);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&d_jobs, (void*)&njobs, (void*)&vec_bytes};
-    return cudaLaunchCooperativeKernel((void*)gfmc_team_engine<double>, dim3(grid), dim3(kThreads), args, (size_t)smem, s);
+    return cudaLaunchCooperativeKernel((void*)gfmc_team_engine<double, 0>, dim3(grid), dim3(kThreads), args, (size_t)smem, s);
 }
 
 // The same launch through cudaLaunchKernelEx with the cooperative attribute,
 // the form a CUDA graph captures as a cooperative kernel node.
 cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s)
 {
-    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double>);
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double, 0>);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -78,14 +78,14 @@ cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int v
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<double>, d_jobs, njobs, vec_bytes);
+    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<double, 0>, d_jobs, njobs, vec_bytes);
 }
 
 cudaError_t team_max_ctas_f64(int smem, int* out)
 {
-    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double>);
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double, 0>);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, gfmc_team_engine<double>, kThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, gfmc_team_engine<double, 0>, kThreads, smem);
 }
 
 }  // namespace gfmc

@@ -97,3 +97,35 @@ def test_packed_grid_wait_runs_out(G):
         assert e.value.status == G.GFMC_ETIMEOUT
         a.set_wait_budget(4_000_000_000)
         assert np.array_equal(a.updates(n)["d_omega"], b.updates(n)["d_omega"])
+
+
+@pytest.mark.parametrize("precision,tol,tie", [
+    ("fp64", lambda r: 1e-10 * abs(r) + 1e-13 * A, 1e-9),
+    ("fp32_mixed", lambda r: 2e-5, 1e-3),
+])
+def test_teams_match_oracle(G, precision, tol, tie):
+    """Chains on teams of CTAs, both recursions: one CTA of 1, 2, 3 and 4 sites per
+    thread and more; tiles of a plane and more with the planes beside them in
+    shared memory (the whole lattice, tiles all edge, tiles with an interior,
+    tiles of unequal size) and tiles below a plane; odd lattices; chains on two
+    and on seven vectors sharing a CTA.  nsteps of 7, 8, 9 and 15 around the
+    groups of eight steps."""
+    # (L, team size, M, recursion, engine)
+    specs = [(4, 1, 16, "unit_vectors", "auto"), (6, 0, 32, "unit_vectors", "auto"),
+             (5, 0, 16, "unit_vectors", "auto"), (6, 0, 16, "unit_vectors", "grid"),
+             (8, 0, 16, "unit_vectors", "auto"), (8, 1, 64, "proposal", "auto"), (10, 1, 32, "unit_vectors", "auto"),
+             (12, 1, 16, "proposal", "auto"), (4, 2, 32, "unit_vectors", "auto"), (6, 3, 32, "proposal", "auto"),
+             (8, 3, 16, "unit_vectors", "auto"), (8, 20, 16, "unit_vectors", "auto"),
+             (10, 7, 32, "proposal", "auto"), (12, 5, 16, "unit_vectors", "auto"),
+             (14, 3, 32, "unit_vectors", "auto"), (7, 2, 16, "unit_vectors", "auto")]
+    n = 14
+    chains, sps = [], []
+    for c, (L, _, M, rec, eng) in enumerate(specs):
+        sps.append(inputs.uniform_sphere(L, 70 + c))
+        chains.append(G.Chain(L, sps[c], M=M, beta=12.0, mu=-2.0, seed=5, chain_id=c, precision=precision,
+                              recursion=rec, engine=eng))
+    outs = G.run_batch(chains, n, team_ctas=[s[1] for s in specs])
+    for c, (L, _, M, _, _) in enumerate(specs):
+        replay(L, sps[c], M, 0, c, outs[c], tol, tie)
+    for ch in chains:
+        ch.close()
