@@ -34,7 +34,7 @@ struct gfmc_ctx {
     // the engine, and the CTAs of a single chain, were left to the library
     bool auto_engine = false, auto_ctas = false;
     // even lattices on the automatic engine: Delta Omega calls run the packed
-    // recursion on one cluster (1) or on the whole grid (2); 0: another engine
+    // recursion on one cluster (1), the whole grid (2) or one CTA (3); 0: another engine
     int pk = 0, pk_engine = 0, pk_ctas = 0, pk_cy = 0, pk_cz = 0, pk_smem = 0;
     size_t pk_inbox_bytes = 0;
     Params P{};
@@ -230,7 +230,8 @@ int team_nv(const gfmc_ctx* h)
 }
 
 // Shared memory a team CTA of chain h needs for its vectors, or SIZE_MAX when
-// they stay in global memory.  Even lattices on the proposal's vectors: the packed
+// they stay in global memory.  Even lattices on the proposal's vectors: small one-CTA
+// chains the packed vector and the ring of the steps' sums, others the packed
 // vector on the CTA's sites and the planes beside them (a tile of a plane at least:
 // the planes' values then come from the CTAs it waits for); else one-CTA teams
 // only, every vector on the whole lattice.
@@ -239,18 +240,24 @@ size_t team_vec_bytes(const gfmc_ctx* h, int tc)
     const size_t vsz = h->precision == GFMC_PREC_FP64 ? sizeof(double2) : sizeof(float2);
     const int nv = team_nv(h), LL = h->L * h->L;
     if (nv == 2 && h->L % 2 == 0 && !h->P.comp) {
+        const bool fp64 = h->precision == GFMC_PREC_FP64;
+        if (tc == 1 && h->N <= (fp64 ? gfmc::one_cta_sites<double>(gfmc::kThreads) : gfmc::one_cta_sites<float>(gfmc::kThreads)))
+            return fp64 ? gfmc::one_cta_bytes<double>(h->N, gfmc::kThreads) : gfmc::one_cta_bytes<float>(h->N, gfmc::kThreads);
         if (tc > 1 && h->N / tc < LL) return SIZE_MAX;
         return 2 * (size_t)std::min(h->N, (h->N + tc - 1) / tc + 2 * LL) * vsz;
     }
     return tc <= 1 ? 2 * (size_t)nv * h->N * vsz : SIZE_MAX;
 }
 
-// the vectors of every job's recursion, 0 when they differ
-int common_nv(const std::vector<gfmc::TeamJob>& jobs)
+// the vectors of every job's recursion, 0 when they differ; 1: all on the packed one
+int common_nv(const gfmc::TeamJob* jobs, size_t n)
 {
-    for (const auto& j : jobs)
-        if (j.p.nv != jobs[0].p.nv) return 0;
-    return jobs[0].p.nv;
+    bool packed = true;
+    for (size_t j = 0; j < n; ++j) {
+        if (jobs[j].p.nv != jobs[0].p.nv) return 0;
+        packed = packed && jobs[j].p.nv == 2 && jobs[j].p.L % 2 == 0 && !jobs[j].p.comp;
+    }
+    return packed ? 1 : jobs[0].p.nv;
 }
 
 // Run one engine launch and wait for it; translate the device error word.
@@ -269,13 +276,15 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
     const int nv = P.mode != gfmc::MODE_MOMENTS &&
                            (h->recursion == GFMC_RECURSION_PROPOSAL || (h->auto_engine && h->auto_ctas && !h->vcl))
                        ? 2 : gfmc::kVec;
-    // a cluster of the packed engine has no flags to withhold: the stall hook runs the grid engine
-    const bool packed = h->pk != 0 && P.mode != gfmc::MODE_MOMENTS && !(P.stall && h->pk == 1);
+    // one CTA or a cluster of the packed engine has no flags to withhold: the stall hook runs the grid engine
+    const bool packed = h->pk != 0 && P.mode != gfmc::MODE_MOMENTS && !(P.stall && h->pk != 2);
     if (packed) {
         P.ncta = h->pk_ctas;
         P.pk_cy = h->pk_cy;
         P.pk_cz = h->pk_cz;
-        if (h->pk == 1) {
+        if (h->pk == 3) {
+            e = gfmc::launch_one_cta(h->precision, P, h->pk_smem, h->stream);
+        } else if (h->pk == 1) {
             e = gfmc::launch_packed_single(h->pk_engine, P, h->pk_smem, h->stream);
         } else {
             // the tags of the face values count from a cleared inbox
@@ -293,7 +302,8 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
             return cuda_fail(h, e, "uploading the job");
         const int smem = gfmc::engine_smem_bytes(P.K);
         e = h->precision == GFMC_PREC_FP64 ? gfmc::launch_team_f64(h->d_job, 1, P.ncta, 0, smem, h->stream)
-                                            : gfmc::launch_team_f32(h->d_job, 1, P.ncta, 0, smem, h->stream, P.comp != 0, nv);
+                                            : gfmc::launch_team_f32(h->d_job, 1, P.ncta, 0, smem, h->stream, P.comp != 0,
+                                                                    common_nv(&job, 1));
     } else {
         if (h->vcl && nv == gfmc::kVec)
             e = gfmc::launch_vcluster_f32(P, h->stream);
@@ -400,11 +410,13 @@ gfmc_status use_team_plan(gfmc_ctx* h, int tc)
 
 // The packed engine of a chain's Delta Omega calls (automatic engine, even L,
 // plain sums), if one takes it.  Measured, us per update at M = 1024:
-//   FP32-mixed, one cluster of C CTAs: L = 4: 276 on 1, 331-342 on 2-16; L = 8:
-//   326 on 1, 333-348 on 2-16; L = 16: 1173 on 1, 443 on 4, 353 on 16; L = 24: 628 on
-//   8, 446 on 16.  So one CTA up to 512 sites, else the most CTAs that split the
-//   lattice.  L = 32 stays on the seven vector clusters (767; one packed cluster
-//   643), whose moments without the doubling are twice as accurate in FP32.
+//   One CTA (gfmc_team.cuh) up to 512 sites in FP32, 256 in FP64: FP32-mixed L = 4: 156,
+//   on a cluster of 1 to 16 CTAs 276-342; L = 8: 246, on clusters 326-348.  FP64
+//   L = 4: 173, L = 6: 332; L = 8, one site per thread of 512, 669 and on 16 CTAs 425.
+//   FP32-mixed, one cluster of C CTAs: L = 16: 1173 on 1, 443 on 4, 353 on 16; L = 24:
+//   628 on 8, 446 on 16.  So the most CTAs that split the lattice.  L = 32 stays on the
+//   seven vector clusters (767; one packed cluster 643), whose moments without the
+//   doubling are twice as accurate in FP32.
 //   FP64: the cluster of the most CTAs up to L = 16 (L = 8: 418 on 16, 668 on the
 //   grid; L = 16: 614 and 651), where a CTA still has at most 256 sites, one per
 //   thread; the whole grid above.
@@ -415,10 +427,23 @@ gfmc_status plan_packed(gfmc_ctx* h)
     int dev_smem = 0, st = 0;
     cudaError_t e;
     const int engine = fp32 ? 1 : 2;
+    if (h->N <= (fp32 ? 2 : 1) * gfmc::kThreads) {
+        const int prec = h->precision;
+        const int NT = gfmc::one_cta_threads(prec, h->N);
+        // the tail's four sequences at once where they fit in a third of the SM's shared memory
+        const int vec = fp32 ? gfmc::one_cta_bytes<float>(h->N, NT) : gfmc::kOneCtaHist * 16 * h->N;
+        const int bytes = std::max({vec, 8 * h->K, std::min(32 * h->K, 72 * 1024)});
+        if (gfmc::one_cta_fits(prec, h->N, bytes)) {
+            h->pk = 3;
+            h->pk_ctas = h->pk_cy = h->pk_cz = 1;
+            h->pk_smem = bytes;
+            return GFMC_OK;
+        }
+    }
     if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device)) != cudaSuccess ||
         (e = gfmc::packed_static_smem(engine, &st)) != cudaSuccess)
         return cuda_fail(h, e, "querying shared memory");
-    for (int C = fp32 && h->N <= 512 ? 1 : 16; C >= 1; --C) {
+    for (int C = 16; C >= 1; --C) {
         int cy = 0, bytes = 0, active = 0;
         if (!gfmc::pk_split(h->L, C, h->K, fp32, &cy, &bytes)) continue;
         if (!fp32) {
@@ -963,7 +988,7 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
         return cuda_fail(nullptr, e, "uploading the job table");
     e = prec == GFMC_PREC_FP64 ? gfmc::launch_team_f64(d_jobs, n_chains, grid, (int)vec_bytes, smem, s)
                                : gfmc::launch_team_f32(d_jobs, n_chains, grid, (int)vec_bytes, smem, s,
-                                                       chains[0]->P.comp != 0, common_nv(jobs));
+                                                       chains[0]->P.comp != 0, common_nv(jobs.data(), jobs.size()));
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "launching the batch");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(nullptr, e, "batch execution");
     gfmc_status result = GFMC_OK;
@@ -1545,7 +1570,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
     if (ce == cudaSuccess && !clusters) {
         ce = prec == GFMC_PREC_FP64 ? gfmc::launch_team_ex_f64(p->d_jobs, nj, team_grid, team_vec, team_smem, cs)
                                     : gfmc::launch_team_ex_f32(p->d_jobs, nj, team_grid, team_vec, team_smem, cs,
-                                                               chains[0]->P.comp != 0, common_nv(jobs));
+                                                               chains[0]->P.comp != 0, common_nv(jobs.data(), jobs.size()));
     } else if (ce == cudaSuccess) {
         cudaEvent_t fork = nullptr;
         ce = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);

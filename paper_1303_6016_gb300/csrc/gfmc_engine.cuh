@@ -1552,337 +1552,6 @@ __device__ bool team_steps2(const Params& p, int cta, unsigned phase, typename C
 }
 
 // ---------------------------------------------------------------------------
-// team CTAs on an even lattice: one vector S = r^o + r^v
-// ---------------------------------------------------------------------------
-// On an even periodic lattice Htilde joins only sites of opposite parity, so
-// r_m^o lives on the sites of parity(o) + m (class A) and r_m^v on the others
-// (class B): S_m = r_m^o + r_m^v holds both in one vector, and S_{m+1} = 2 Htilde S_m
-// - S_{m-1} advances both at once.  The products parity leaves are |r_m^o|^2 and
-// <r_m^o|r_{m+1}^v> over class A and |r_m^v|^2 over class B.
-//
-// The sums of kSumRing steps by step, warp and value; those of a group of
-// kSumGroup steps are added over the warps while the next group's are written.
-constexpr int kSumGroup = 8, kSumRing = 2 * kSumGroup;
-template <class R> struct StepSums {
-    R w[kSumRing][kWarps][4];
-};
-
-// Butterfly reduce-scatter of 4 values: lanes 8j .. 8j + 7 return the warp's sum of value j.
-template <class R> __device__ __forceinline__ R warp_reduce_scatter4(const R (&v)[4], int lane)
-{
-    const bool hi = lane & 16, up = lane & 8;
-    const R a = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
-    const R b = (hi ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
-    R s = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 8);
-    s += __shfl_xor_sync(0xffffffffu, s, 4);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    return s;
-}
-
-// Add the sums of the steps f0 .. f1 (one group at most) over the warps.
-template <class R>
-__device__ __forceinline__ void add_step_sums(const Params& p, const StepSums<R>& sums, int f0, int f1)
-{
-    const int f = f0 + (int)(threadIdx.x >> 2), v = threadIdx.x & 3;
-    if (f <= f1) {
-        double sum = 0.0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) sum += (double)sums.w[f & (kSumRing - 1)][w][v];
-        gram_add(p, f, v < 2 ? v : v + 4, sum);
-    }
-}
-
-// What a site adds to the sums: cur = S_m and nxt = S_{m+1} there.
-template <class R, class R2>
-__device__ __forceinline__ void add_site(R (&acc)[4], bool class_a, R2 cur, R2 nxt)
-{
-    const R2 a = class_a ? cur : c_make<R2>(0, 0), b = class_a ? c_make<R2>(0, 0) : cur;
-    acc[0] = fma(a.x, a.x, fma(a.y, a.y, acc[0]));
-    acc[1] = fma(b.x, b.x, fma(b.y, b.y, acc[1]));
-    acc[2] = fma(a.x, nxt.x, fma(a.y, nxt.y, acc[2]));
-    acc[3] = fma(a.x, nxt.y, fma(-a.y, nxt.x, acc[3]));
-}
-
-// S_0 = e_o + v and S_1 = Htilde S_0 at site i.
-template <class R2>
-__device__ __forceinline__ void first_vectors(const Params& p, const R2* hop, const int* s_loc, const R2 (&cv6)[6],
-                                              int i, R2& r0, R2& r1)
-{
-    int nb[6];
-    site_nbrs(i, p.L, p.divL, p.divLL, nb);
-    r0 = c_make<R2>(i == s_loc[0] ? 1 : 0, 0);
-    r1 = c_make<R2>(0, 0);
-#pragma unroll
-    for (int k = 0; k < 6; ++k)
-        if (i == s_loc[k + 1]) {
-            r0.x += cv6[k].x;
-            r0.y += cv6[k].y;
-        }
-#pragma unroll
-    for (int d = 0; d < 6; ++d) {
-        bool hit = false;
-#pragma unroll
-        for (int k = 0; k < kVec; ++k) hit |= nb[d] == s_loc[k];
-        if (hit) {
-            const R2 h = hop_of(hop, p.N, i, d, nb[d]);
-            if (nb[d] == s_loc[0]) {
-                r1.x += h.x;
-                r1.y += h.y;
-            }
-#pragma unroll
-            for (int k = 0; k < 6; ++k)
-                if (nb[d] == s_loc[k + 1]) c_fma(r1, h, cv6[k]);
-        }
-    }
-}
-
-template <class R> __device__ __forceinline__ const typename Cx<R>::T* hop_table(const Params& p)
-{
-    if constexpr (sizeof(R) == 8) return (const double2*)p.hop64;
-    else return (const float2*)p.hop32;
-}
-
-// A one-CTA team of at most KR kThreads sites, the lattice in shared memory:
-// each thread keeps its sites' bonds, S_m and S_{m-1} in registers.  The step
-// is one CTA barrier and a chain of latencies (six shared loads, the FMAs, a
-// store, the warp sums), so nothing else is left in it.
-template <class R, int KR>
-__device__ __noinline__ void one_cta_steps(const Params& p, typename Cx<R>::T* buf, const int* s_loc, const double2* s_c,
-                              StepSums<R>& sums)
-{
-    using R2 = typename Cx<R>::T;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int N = p.N, L = p.L;
-    const R2* hop = hop_table<R>(p);
-    R2 cv6[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) cv6[k] = c_make<R2>((R)s_c[k + 1].x, (R)s_c[k + 1].y);
-    const int lo = s_loc[0];
-    const int par_o = (lo % L + (lo / L) % L + lo / (L * L)) & 1;
-    R2 h[KR][6], cur[KR], prv[KR];
-    int nb[KR][6], par[KR];
-#pragma unroll
-    for (int k = 0; k < KR; ++k) {
-        const int i = tid + k * kThreads;
-        const bool on = i < N;
-        const int g = on ? i : 0;
-        site_nbrs(g, L, p.divL, p.divLL, nb[k]);
-        const int r = (int)__umulhi((unsigned)g, p.divL), z = (int)__umulhi((unsigned)g, p.divLL);
-        par[k] = (g - r * L + r - z * L + z + par_o) & 1;
-        first_vectors(p, hop, s_loc, cv6, g, prv[k], cur[k]);
-        if (!on) prv[k] = cur[k] = c_make<R2>(0, 0);
-#pragma unroll
-        for (int d = 0; d < 6; ++d) {
-            const R2 q = hop_of(hop, N, g, d, nb[k][d]);
-            h[k][d] = on ? c_make<R2>(2 * q.x, 2 * q.y) : c_make<R2>(0, 0);  // 2 Htilde, exact
-        }
-        if (on) buf[N + i] = cur[k];
-    }
-    __syncthreads();
-    for (int m = 1; m <= p.nsteps; ++m) {
-        const R2* rd = buf + ((m & 1) ? N : 0);
-        R2* wr = buf + ((m & 1) ? 0 : N);
-        R acc[4] = {0, 0, 0, 0};
-        R2 nv[KR][6];
-#pragma unroll
-        for (int k = 0; k < KR; ++k)
-#pragma unroll
-            for (int d = 0; d < 6; ++d) nv[k][d] = rd[nb[k][d]];
-        if ((m & (kSumGroup - 1)) == 1 && m > kSumGroup) add_step_sums<R>(p, sums, m - kSumGroup, m - 1);
-#pragma unroll
-        for (int k = 0; k < KR; ++k) {
-            const R2 s = bond_sum6(h[k], nv[k]);
-            const R2 nx = c_make<R2>(s.x - prv[k].x, s.y - prv[k].y);
-            if (tid + k * kThreads < N) wr[tid + k * kThreads] = nx;
-            add_site(acc, ((par[k] + m) & 1) == 0, cur[k], nx);
-            prv[k] = cur[k];
-            cur[k] = nx;
-        }
-        const R s = warp_reduce_scatter4(acc, lane);
-        if ((lane & 7) == 0) sums.w[m & (kSumRing - 1)][warp][lane >> 3] = s;
-        __syncthreads();
-    }
-    add_step_sums<R>(p, sums, (p.nsteps - 1) / kSumGroup * kSumGroup + 1, p.nsteps);
-}
-
-// A team CTA of any number of sites.
-// WIN: S_m and S_{m-1} of the CTA's sites and of the planes before and after
-// them stand in shared memory (buf: two buffers of W sites); only those planes
-// -- 2 L^2 sites -- come from the other CTAs' stores each step.  The sites
-// within a plane of the tile's ends go first and are published before the
-// others are computed, so the neighbours' wait overlaps the rest of the step.
-// Without WIN (tiles below a plane, or too large for shared memory) all values
-// are read from global memory.
-template <class R, bool WIN, bool WIDE>
-__device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigned phase, typename Cx<R>::T* buf,
-                                  const int* s_loc, const double2* s_c, StepSums<R>& sums)
-{
-    using R2 = typename Cx<R>::T;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int N = p.N, L = p.L, LL = L * L;
-    const int s0 = p.tile_start[cta], s1 = p.tile_start[cta + 1], T = s1 - s0;
-    const R2* hop = hop_table<R>(p);
-    R2 cv6[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) cv6[k] = c_make<R2>((R)s_c[k + 1].x, (R)s_c[k + 1].y);
-    const int lo = s_loc[0];
-    const int par_o = (lo % L + (lo / L) % L + lo / LL) & 1;
-    // whole: the buffers hold the lattice, site i at i; else site s0 - L^2 + w (mod N) at w
-    const bool whole = !WIN || T + 2 * LL >= N;
-    const int W = whole ? N : T + 2 * LL, base = whole ? 0 : s0 - LL;
-    R2* g0 = (R2*)p.rbuf;
-    R2* g1 = g0 + N;
-    R2* b0 = WIN ? buf : g0;
-    R2* b1 = WIN ? buf + W : g1;
-    auto wrap = [&](int i) { return i < 0 ? i + N : i >= N ? i - N : i; };
-
-    const int n0 = WIN ? W : T, f0 = WIN ? base : s0;
-    for (int w = tid; w < n0; w += kThreads) {
-        R2 r0, r1;
-        first_vectors(p, hop, s_loc, cv6, wrap(f0 + w), r0, r1);
-        if constexpr (WIN) {
-            b0[w] = r0;
-            b1[w] = r1;
-        } else {
-            stcg2(b0 + s0 + w, r0);
-            stcg2(b1 + s0 + w, r1);
-        }
-    }
-    if constexpr (WIN) __syncthreads();
-    else publish(p, cta, phase + 1);
-
-    // sites of the tile within a plane of its ends: [0, e0) and [e1, T)
-    const int e0 = (WIN && p.ncta > 1 && T > 2 * LL) ? LL : T, e1 = e0 < T ? T - LL : T;
-    const int halo = whole ? N - T : 2 * LL;
-    for (int m = 1; m <= p.nsteps; ++m) {
-        const R2* rd = (m & 1) ? b1 : b0;
-        R2* wr = (m & 1) ? b0 : b1;
-        R2* gw = (m & 1) ? g0 : g1;
-        if (!WIN || (p.ncta > 1 && m > 1)) {
-            if (!wait_neighbours(p, cta, phase + (unsigned)m, 100 + m)) return false;
-        }
-        if constexpr (WIN) {
-            if (p.ncta > 1 && m > 1) {
-                const R2* gr = (m & 1) ? g1 : g0;
-                R2* dst = (m & 1) ? b1 : b0;
-                for (int k = tid; k < halo; k += kThreads) {
-                    // k-th site after the tile, or (k >= L^2) before it
-                    const int i = whole || k < LL ? wrap(s1 + k) : wrap(s0 - 2 * LL + k);
-                    const int w = whole ? i : k < LL ? LL + T + k : k - LL;
-                    dst[w] = ldcg2(gr + i);
-                }
-                __syncthreads();
-            }
-        }
-        R acc[4] = {0, 0, 0, 0};
-        struct Ops {
-            R2 h[6], nv[6], cur, pv;
-            int i, w, odd;
-        };
-        auto ld = [&](const R2* a) {
-            if constexpr (WIN) return *a;
-            else return ldcg2(a);
-        };
-        auto load = [&](int k, Ops& q) {
-            const int i = s0 + k;
-            const int z = (int)__umulhi((unsigned)i, p.divLL), r = (int)__umulhi((unsigned)i, p.divL);
-            const int x = i - r * L, y = r - z * L;
-            q.i = i;
-            q.w = whole ? i : k + LL;
-            q.odd = x + y + z;
-            const int xp = x == L - 1 ? 1 - L : 1, xm = x == 0 ? L - 1 : -1;
-            const int yp = y == L - 1 ? L - LL : L, ym = y == 0 ? LL - L : -L;
-            const int zm = z == 0 ? N - LL : -LL;
-            const int wzp = whole && z == L - 1 ? LL - N : LL, wzm = whole ? zm : -LL;
-            const R2* c = rd + q.w;
-            q.h[0] = ldcg2(hop + i);
-            q.h[1] = ldcg2(hop + (i + xm));
-            q.h[2] = ldcg2(hop + (N + i));
-            q.h[3] = ldcg2(hop + (N + i + ym));
-            q.h[4] = ldcg2(hop + (2 * N + i));
-            q.h[5] = ldcg2(hop + (2 * N + i + zm));
-            q.nv[0] = ld(c + xp);
-            q.nv[1] = ld(c + xm);
-            q.nv[2] = ld(c + yp);
-            q.nv[3] = ld(c + ym);
-            q.nv[4] = ld(c + wzp);
-            q.nv[5] = ld(c + wzm);
-            q.cur = ld(c);
-            q.pv = ld(wr + q.w);
-        };
-        auto step = [&](Ops& q, bool edge) {
-            q.h[1].y = -q.h[1].y;  // backward bonds: the conjugates
-            q.h[3].y = -q.h[3].y;
-            q.h[5].y = -q.h[5].y;
-            const R2 s = bond_sum6(q.h, q.nv);
-            const R2 nx = c_make<R2>(fma((R)2, s.x, -q.pv.x), fma((R)2, s.y, -q.pv.y));
-            if (m < p.nsteps) {
-                if constexpr (WIN) wr[q.w] = nx;
-                if (!WIN || edge) stcg2(gw + q.i, nx);
-            }
-            add_site(acc, ((q.odd + par_o + m) & 1) == 0, q.cur, nx);
-        };
-        // sites [0, n) of a list: k < j0 at k, the others at k + j1 - j0
-        auto sites = [&](int n, int j0, int j1, bool edge) {
-            auto at = [&](int k) { return k < j0 ? k : k + (j1 - j0); };
-            if constexpr (WIDE && sizeof(R) == 4) {
-                // two sites per pass, both sites' loads issued before the first use
-                for (int k = tid; k < n; k += 2 * kThreads) {
-                    Ops qa, qb;
-                    load(at(k), qa);
-                    if (k + kThreads < n) load(at(k + kThreads), qb);
-                    step(qa, edge);
-                    if (k + kThreads < n) step(qb, edge);
-                }
-            } else {
-                for (int k = tid; k < n; k += kThreads) {
-                    Ops q;
-                    load(at(k), q);
-                    step(q, edge);
-                }
-            }
-        };
-        // the tile's ends, read by the other CTAs, then the sites between
-        sites(e0 + T - e1, e0, e1, p.ncta > 1);
-        publish(p, cta, phase + (unsigned)m + 1u);
-        if (e0 < e1) sites(e1 - e0, 0, e0, false);
-        const R s = warp_reduce_scatter4(acc, lane);
-        if ((lane & 7) == 0) sums.w[m & (kSumRing - 1)][warp][lane >> 3] = s;
-        if ((m & (kSumGroup - 1)) == 0 || m == p.nsteps) {
-            __syncthreads();
-            add_step_sums<R>(p, sums, (m - 1) / kSumGroup * kSumGroup + 1, m);
-        }
-    }
-    return true;
-}
-
-// The steps of one update of a team CTA on an even lattice, plain sums.
-template <class R, bool WIDE>
-__device__ bool team_even_steps(const Params& p, int cta, unsigned phase, typename Cx<R>::T* vec_smem,
-                                const int* s_loc, const double2* s_c, StepSums<R>& sums)
-{
-    if constexpr (WIDE) {
-        if (vec_smem) {
-            if (p.ncta == 1 && p.N <= kThreads) {
-                one_cta_steps<R, 1>(p, vec_smem, s_loc, s_c, sums);
-                return true;
-            }
-            if (p.ncta == 1 && p.N <= 2 * kThreads) {
-                one_cta_steps<R, 2>(p, vec_smem, s_loc, s_c, sums);
-                return true;
-            }
-            if (sizeof(R) == 4 && p.ncta == 1 && p.N <= 4 * kThreads) {
-                if constexpr (sizeof(R) == 4) one_cta_steps<R, 4>(p, vec_smem, s_loc, s_c, sums);
-                return true;
-            }
-            return team_packed_steps<R, true, WIDE>(p, cta, phase, vec_smem, s_loc, s_c, sums);
-        }
-    }
-    return team_packed_steps<R, false, WIDE>(p, cta, phase, nullptr, s_loc, s_c, sums);
-}
-
-// ---------------------------------------------------------------------------
 // distributed shared memory of a cluster (explicit shared::cluster accesses)
 // ---------------------------------------------------------------------------
 
@@ -3290,16 +2959,7 @@ __device__ __forceinline__ void run_chain(const Params& p, const int cta, double
         } else if constexpr (VARIANT == 2) {
             cluster_steps2<R, NT, COMP>(p, cta, vec_smem, s_loc, s_c);
         } else if constexpr (NV == 2) {
-            // the steps' sums stand where the tail's work space is
-            static_assert(sizeof(StepSums<R>) <= sizeof(red), "the sums fit the work space");
-            bool even = false;
-            if constexpr (!COMP) {
-                even = L % 2 == 0;
-                if (even && !team_even_steps<R, WIDE>(p, cta, phase, vec_smem, s_loc, s_c, *(StepSums<R>*)&red[0][0]))
-                    return;
-            }
-            if (even) {
-            } else if (vec_smem) {
+            if (vec_smem) {
                 if (!team_steps2<R, SmemVec, WIDE, COMP>(p, cta, phase, buf0, buf1, s_loc, s_c, red, SmemVec{})) return;
             } else {
                 if (!team_steps2<R, GlobalVec, WIDE, COMP>(p, cta, phase, buf0, buf1, s_loc, s_c, red, GlobalVec{}))
@@ -3491,56 +3151,6 @@ __global__ void __launch_bounds__(engine_threads<R, NV>(), 1) gfmc_engine(const 
 {
     extern __shared__ double2 dyn[];
     run_chain<R, 0, NV, engine_threads<R, NV>(), true, COMP, SPLIT>(p, blockIdx.x, dyn, nullptr);
-}
-
-// A batch of chains, each on its own team of CTAs (jobs sorted by cta0).
-// The dynamic shared memory holds [vector area of vec_bytes][work area].
-// NV: the recursion of all chains, 0 when they differ.  With both recursions in one
-// kernel the FP32 steps on seven vectors spill (moments of L = 40: 866 us, alone 720).
-template <class R, int NV, bool COMP = false>
-__global__ void __launch_bounds__(kThreads, 1) gfmc_team_engine(const TeamJob* __restrict__ jobs, int njobs,
-                                                                 int vec_bytes)
-{
-    extern __shared__ double2 dyn_all[];
-    __shared__ Params sp;
-    __shared__ int s_job, s_cta, s_vs;
-    if (threadIdx.x == 0) {
-        int j = 0;
-        while (j + 1 < njobs && jobs[j + 1].cta0 <= (int)blockIdx.x) ++j;
-        // several one-CTA chains may share this CTA (same cta0): start at the first
-        while (j > 0 && jobs[j - 1].cta0 == jobs[j].cta0) --j;
-        s_job = j;
-    }
-    __syncthreads();
-    using R2 = typename Cx<R>::T;
-    // the chains of this CTA's team, one after another: one chain unless the
-    // team is a shared one-CTA team
-    auto load = [&]() {
-        if (threadIdx.x == 0) {
-            const int j = s_job;
-            s_cta = (int)blockIdx.x - jobs[j].cta0;
-            s_vs = jobs[j].vec_smem;
-            sp = jobs[j].p;
-        }
-        __syncthreads();
-    };
-    auto next = [&]() -> bool {
-        __syncthreads();  // every thread is done with sp and the shared memory
-        if (threadIdx.x == 0) {
-            const int j = s_job + 1;
-            s_job = (j < njobs && jobs[j].cta0 == jobs[j - 1].cta0) ? j : -1;
-        }
-        __syncthreads();
-        return s_job >= 0;
-    };
-    do {
-        load();
-        double2* work = dyn_all + vec_bytes / (int)sizeof(double2);
-        R2* vec = s_vs ? (R2*)dyn_all : nullptr;
-        if constexpr (NV != 0) run_chain<R, 1, NV, kThreads, true, COMP>(sp, s_cta, work, vec);
-        else if (sp.nv == 2) run_chain<R, 1, 2, kThreads, true, COMP>(sp, s_cta, work, vec);
-        else run_chain<R, 1, kVec, kThreads, true, COMP>(sp, s_cta, work, vec);
-    } while (next());
 }
 
 // A batch of chains, one thread-block cluster per chain (cluster size C = the

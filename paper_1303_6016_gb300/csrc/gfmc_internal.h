@@ -202,6 +202,20 @@ inline bool pk_grid_split(int L, int K, int max_ctas, int smem, int* cy, int* cz
     return best >= 0;
 }
 
+// One-CTA chains of a few sites per thread (gfmc_team.cuh): the most sites a CTA of nt
+// threads takes (FP32: 4 per thread, FP64 in fixed point: 2), the ring items per
+// step, and the shared memory of vectors and ring.
+template <class R> __host__ __device__ constexpr int one_cta_sites(int nt) { return sizeof(R) == 4 ? 4 * nt : 2 * nt; }
+__host__ __device__ inline int one_cta_items(int N, int nt) { return N < nt ? (N + 31) / 32 * 32 : nt; }
+template <class R> __host__ __device__ inline int one_cta_bytes(int N, int nt)
+{
+    return 4 * (int)sizeof(R) * N + 16 * one_cta_items(N, nt) * (sizeof(R) == 4 ? 16 : 8);
+}
+// An FP64 chain alone on a CTA: threads per site.  Two (the real and the imaginary part)
+// while that is one warp per sub-partition: L = 4 0.30 us per step, with one thread 0.40;
+// L = 6 0.69 with two, 0.61 with one.
+__host__ __device__ inline int one_cta_parts(int N) { return 2 * N <= 128 ? 2 : 1; }
+
 // One chain of a batch launch: its parameters (ncta = its team size, tile plan
 // for that team) and its CTAs [cta0, cta0 + p.ncta) of the grid.
 struct TeamJob {
@@ -237,7 +251,7 @@ cudaError_t launch_engine_f32(const Params& p, cudaStream_t s);
 cudaError_t launch_engine_f64(const Params& p, int nv, cudaStream_t s);
 cudaError_t launch_engine_f32(const Params& p, int nv, cudaStream_t s);
 cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s);
-// nv: the vectors of every job's recursion (p.nv), 0 when they differ
+// nv: the vectors of every job's recursion (p.nv), 0 when they differ; 1: even lattices on two vectors only
 cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
                             bool comp, int nv);
 cudaError_t team_max_ctas(int precision, int smem, int* out);
@@ -257,6 +271,12 @@ cudaError_t launch_packed(int engine, const TeamJob* d_jobs, int njobs, int C, i
 cudaError_t launch_packed_single(int engine, const Params& p, int smem, cudaStream_t s);
 cudaError_t packed_max_active(int engine, int C, int smem, int* out);
 cudaError_t packed_static_smem(int engine, int* out);
+// a single chain on one CTA: even L, at most kThreads sites (FP32: 2 kThreads)
+// (FP64: at most kThreads that advance the sites, and eight warps for the sums)
+inline int one_cta_threads(int precision, int N) { return precision != 0 && N <= kThreads ? kThreads : 2 * kThreads; }
+constexpr int kOneCtaHist = 32;  // vectors an FP64 chain keeps in shared memory
+cudaError_t launch_one_cta(int precision, const Params& p, int smem, cudaStream_t s);
+bool one_cta_fits(int precision, int N, int smem);
 // a single FP64 chain on p.ncta CTAs of a cooperative grid
 cudaError_t launch_packed64_grid(const Params& p, int smem, cudaStream_t s);
 cudaError_t packed64_grid_max_ctas(int smem, int* out);

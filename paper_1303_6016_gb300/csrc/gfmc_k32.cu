@@ -3,7 +3,7 @@
 // compensated when comp is set) and in FP64 above.
 #include <algorithm>
 
-#include "gfmc_engine.cuh"
+#include "gfmc_team.cuh"
 
 namespace gfmc {
 
@@ -79,6 +79,7 @@ static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int v
                                bool comp, int nv, bool ex)
 {
     if (comp) return team_launch<0, true>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
+    if (nv == 1) return team_launch<1, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
     if (nv == 2) return team_launch<2, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
     if (nv == kVec) return team_launch<kVec, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
     return team_launch<0, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
@@ -107,12 +108,13 @@ static cudaError_t team_occupancy(int smem, int* out)
 // of the kernel that holds the fewest, so that a batch fits whichever it runs
 cudaError_t team_max_ctas_f32(int smem, int* out)
 {
-    int n[4] = {};
+    int n[5] = {};
     cudaError_t e = team_occupancy<0, false>(smem, &n[0]);
     if (e == cudaSuccess) e = team_occupancy<0, true>(smem, &n[1]);
     if (e == cudaSuccess) e = team_occupancy<2, false>(smem, &n[2]);
     if (e == cudaSuccess) e = team_occupancy<kVec, false>(smem, &n[3]);
-    if (e == cudaSuccess) *out = std::min(std::min(n[0], n[1]), std::min(n[2], n[3]));
+    if (e == cudaSuccess) e = team_occupancy<1, false>(smem, &n[4]);
+    if (e == cudaSuccess) *out = *std::min_element(n, n + 5);
     return e;
 }
 

@@ -1,5 +1,5 @@
 // FP64 instantiation of the persistent GFMC engine.
-#include "gfmc_engine.cuh"
+#include "gfmc_team.cuh"
 
 namespace gfmc {
 

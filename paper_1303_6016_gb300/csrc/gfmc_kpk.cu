@@ -1,6 +1,8 @@
 // Launch of the packed engines: clusters FP32-mixed and FP64 (gfmc_packed.cuh),
-// FP64 small tiles on a cluster or on the whole grid (gfmc_packed64.cuh).
+// FP64 small tiles on a cluster or on the whole grid (gfmc_packed64.cuh), chains on
+// one CTA (gfmc_team.cuh).
 #include "gfmc_packed64.cuh"
+#include "gfmc_team.cuh"
 
 namespace gfmc {
 
@@ -95,6 +97,32 @@ cudaError_t packed64_grid_max_ctas(int smem, int* out)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     *out = per_sm > 0 ? sms : 0;  // one CTA per SM
     return e;
+}
+
+using OneCtaKernel = void (*)(const Params, int);
+static OneCtaKernel one_cta_kernel(int precision, int N)
+{
+    if (precision == 0) return gfmc_one_cta<double, 2 * kThreads>;
+    return one_cta_threads(precision, N) == kThreads ? gfmc_one_cta<float, kThreads> : gfmc_one_cta<float, 2 * kThreads>;
+}
+
+cudaError_t launch_one_cta(int precision, const Params& p, int smem, cudaStream_t s)
+{
+    const OneCtaKernel fn = one_cta_kernel(precision, p.N);
+    const cudaError_t e = allow_dynamic_smem((const void*)fn);
+    if (e != cudaSuccess) return e;
+    fn<<<1, one_cta_threads(precision, p.N), smem, s>>>(p, smem / (int)sizeof(double2));
+    return cudaGetLastError();
+}
+
+bool one_cta_fits(int precision, int N, int smem)
+{
+    const OneCtaKernel fn = one_cta_kernel(precision, N);
+    int n = 0;
+    const bool ok = allow_dynamic_smem((const void*)fn) == cudaSuccess &&
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, one_cta_threads(precision, N), smem) == cudaSuccess && n > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
 }
 
 }  // namespace gfmc

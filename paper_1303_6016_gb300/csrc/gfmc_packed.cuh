@@ -55,7 +55,7 @@ __device__ __forceinline__ long long fixed60(float x, bool& ok)
 
 // Values kept apart by the lane groups of 8 of a warp: on return lanes 8 v .. 8 v + 7
 // hold the warp's sum of value v (v < 4).
-template <class T> __device__ __forceinline__ T warp_reduce_scatter4(T (&v)[4], int lane)
+template <class T> __device__ __forceinline__ T warp_reduce_scatter4(const T (&v)[4], int lane)
 {
     const bool u16 = lane & 16, u8 = lane & 8;
     const T a = u16 ? v[2] : v[0], b = u16 ? v[3] : v[1];
@@ -217,6 +217,27 @@ __device__ __forceinline__ void pk_wait(int C)
 {
     if (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     else __syncthreads();
+}
+
+__device__ __forceinline__ int4 lds4(unsigned a)
+{
+    int4 v;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ int2 lds2(unsigned a)
+{
+    int2 v;
+    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts2(unsigned a, int2 v)
+{
+    asm volatile("st.shared.v2.s32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts4(unsigned a, int4 v)
+{
+    asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
 // the limbs of two fixed-point values: value = high 2^30 + low, the low limb in [-2^29, 2^29)

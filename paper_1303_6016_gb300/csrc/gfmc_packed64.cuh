@@ -31,27 +31,6 @@ struct __align__(8) PkRec {
     unsigned char fl;              // 1: y = 0, 2: y = PY - 1, 4: z = 0, 8: z = PZ - 1, 16: odd parity
 };
 
-__device__ __forceinline__ int4 lds4(unsigned a)
-{
-    int4 v;
-    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ int2 lds2(unsigned a)
-{
-    int2 v;
-    asm volatile("ld.shared.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ void sts2(unsigned a, int2 v)
-{
-    asm volatile("st.shared.v2.s32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
-}
-__device__ __forceinline__ void sts4(unsigned a, int4 v)
-{
-    asm volatile("st.shared.v4.s32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
 // Face values over distributed shared memory.  mb: this CTA's two mbarriers,
 // barrier m & 1 for the faces of S_m; each phase takes one arrival that states
 // the bytes of the faces (bytes).  The re-arming for S_{m+2} may come after some of its
@@ -362,16 +341,11 @@ __device__ __forceinline__ void pk64_records(const PkTile& t, PkRec* tab)
     }
 }
 
-// One main thread's part of a site.  SPL = 1: the whole site.  SPL = 2: lane bit 0
+// A thread's part of a site.  SPL = 1: the whole site.  SPL = 2: lane bit 0
 // the real (0) or the imaginary (1) part.  SPL = 4: also lane bit 1 the forward (0)
 // or backward (1) bonds.  A part is the sum over the bonds of X re + Y im with
 // re: (X, Y) = (Re h, -Im h), im: (Im h, Re h), h conjugated for a backward bond;
 // a whole site holds (Re h, Im h).
-template <int SPL> struct Pk64Lane {
-    static constexpr int ND = SPL == 4 ? 3 : 6;
-    unsigned off[ND];  // ring byte offsets of the neighbours
-    int X[ND][2], Y[ND][2];
-};
 __device__ __forceinline__ unsigned pk64_nbr(const PkTile& t, const PkRec& r, int d)
 {
     const unsigned a = 16u * r.at;

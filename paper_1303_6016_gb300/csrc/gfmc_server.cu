@@ -24,7 +24,7 @@
 // exits regardless, so every wait stays bounded.  A posted job that the
 // kernel did not take before the exit is taken by the next launch (each
 // launch starts from the done words).
-#include "gfmc_engine.cuh"
+#include "gfmc_team.cuh"
 
 namespace gfmc {
 
@@ -105,7 +105,10 @@ __global__ void __launch_bounds__(kThreads, 1) gfmc_server_kernel(ServerArgs a)
         const unsigned cmd = s_cmd;
         if (cmd == kExit) return;
         last = cmd;
-        if (s_prec == 0) {
+        if (sp.nv == 2 && sp.L % 2 == 0) {
+            if (s_prec == 0) pk_team_chain<double, kThreads, kServer>(sp, s_cta, (char*)work, sp.K, false);
+            else pk_team_chain<float, kThreads, kServer>(sp, s_cta, (char*)work, sp.K, false);
+        } else if (s_prec == 0) {
             if (sp.nv == 2) run_chain<double, 1, 2, kThreads, false>(sp, s_cta, work, nullptr);
             else run_chain<double, 1, kVec, kThreads, false>(sp, s_cta, work, nullptr);
         } else {

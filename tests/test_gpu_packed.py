@@ -129,3 +129,16 @@ def test_teams_match_oracle(G, precision, tol, tie):
         replay(L, sps[c], M, 0, c, outs[c], tol, tie)
     for ch in chains:
         ch.close()
+
+
+@pytest.mark.parametrize("L,M,nodes,n", [(4, 16, 0, 70), (4, 64, 128, 10), (6, 32, 0, 10), (8, 64, 0, 10),
+                                         (10, 32, 64, 6)])
+def test_fp32_single_chains_match_oracle(G, L, M, nodes, n):
+    """FP32-mixed chains on the automatic engine: one CTA of fewer sites than threads, of
+    a site per thread of 256 and of 512 threads, a full sweep at L = 4, and the first
+    size on a cluster."""
+    sp = inputs.von_mises_fisher(L, 2.0, L)
+    with G.Chain(L, sp, M=M, beta=12.0, mu=-2.0, seed=5, chain_id=3, precision="fp32_mixed", nodes=nodes) as ch:
+        out = ch.updates(n)
+        replay(L, sp, M, nodes, 3, out, lambda r: 2e-5, 1e-3)
+        assert out["magnetization"].size == n // L ** 3
