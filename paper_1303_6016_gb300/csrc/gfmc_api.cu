@@ -37,6 +37,8 @@ struct gfmc_ctx {
     // recursion on one cluster (1), the whole grid (2) or one CTA (3); 0: another engine
     int pk = 0, pk_engine = 0, pk_ctas = 0, pk_cy = 0, pk_cz = 0, pk_smem = 0;
     size_t pk_inbox_bytes = 0;
+    // the clusters of its moments calls (0: another engine)
+    int mom_ctas = 0, mom_cy = 0, mom_cz = 0, mom_smem = 0;
     Params P{};
     std::vector<void*> allocs;
     uint64_t alloc_bytes = 0;
@@ -278,7 +280,12 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
                        ? 2 : gfmc::kVec;
     // one CTA or a cluster of the packed engine has no flags to withhold: the stall hook runs the grid engine
     const bool packed = h->pk != 0 && P.mode != gfmc::MODE_MOMENTS && !(P.stall && h->pk != 2);
-    if (packed) {
+    if (P.mode == gfmc::MODE_MOMENTS && h->mom_ctas != 0 && !P.stall) {
+        P.ncta = h->mom_ctas;
+        P.pk_cy = h->mom_cy;
+        P.pk_cz = h->mom_cz;
+        e = gfmc::launch_packed64_moments(P, h->mom_smem, h->stream);
+    } else if (packed) {
         P.ncta = h->pk_ctas;
         P.pk_cy = h->pk_cy;
         P.pk_cz = h->pk_cz;
@@ -426,7 +433,34 @@ gfmc_status plan_packed(gfmc_ctx* h)
     if (h->L % 2 != 0 || h->vcl) return GFMC_OK;
     int dev_smem = 0, st = 0;
     cudaError_t e;
-    const int engine = fp32 ? 1 : 2;
+    if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device)) != cudaSuccess ||
+        (e = gfmc::packed_static_smem(fp32 ? 1 : 2, &st)) != cudaSuccess)
+        return cuda_fail(h, e, "querying shared memory");
+    // the cluster of the most CTAs that takes the chain (FP64: a site per thread)
+    auto cluster = [&](bool f32, int* ctas, int* cy, int* bytes) {
+        for (int C = 16; C >= 1; --C) {
+            int active = 0;
+            if (!gfmc::pk_split(h->L, C, h->K, f32, cy, bytes)) continue;
+            if (!f32) {
+                if (h->N / C > 256) break;
+                *bytes = gfmc::pk64_smem_bytes(h->L, h->L / *cy, h->L / (C / *cy), h->K);
+            }
+            if (*bytes + st > dev_smem) continue;
+            if (gfmc::packed_max_active(f32 ? 1 : 2, C, *bytes, &active) != cudaSuccess || active < 1) {
+                cudaGetLastError();
+                continue;
+            }
+            *ctas = C;
+            return true;
+        }
+        return false;
+    };
+    if (cluster(false, &h->mom_ctas, &h->mom_cy, &h->mom_smem)) h->mom_cz = h->mom_ctas / h->mom_cy;
+    if (cluster(fp32, &h->pk_ctas, &h->pk_cy, &h->pk_smem)) {
+        h->pk = 1;
+        h->pk_engine = fp32 ? 1 : 2;
+        h->pk_cz = h->pk_ctas / h->pk_cy;
+    }
     if (h->N <= (fp32 ? 2 : 1) * gfmc::kThreads) {
         const int prec = h->precision;
         const int NT = gfmc::one_cta_threads(prec, h->N);
@@ -440,30 +474,7 @@ gfmc_status plan_packed(gfmc_ctx* h)
             return GFMC_OK;
         }
     }
-    if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device)) != cudaSuccess ||
-        (e = gfmc::packed_static_smem(engine, &st)) != cudaSuccess)
-        return cuda_fail(h, e, "querying shared memory");
-    for (int C = 16; C >= 1; --C) {
-        int cy = 0, bytes = 0, active = 0;
-        if (!gfmc::pk_split(h->L, C, h->K, fp32, &cy, &bytes)) continue;
-        if (!fp32) {
-            if (h->N / C > 256) break;
-            bytes = gfmc::pk64_smem_bytes(h->L, h->L / cy, h->L / (C / cy), h->K);
-        }
-        if (bytes + st > dev_smem) continue;
-        if (gfmc::packed_max_active(engine, C, bytes, &active) != cudaSuccess || active < 1) {
-            cudaGetLastError();
-            continue;
-        }
-        h->pk = 1;
-        h->pk_engine = engine;
-        h->pk_ctas = C;
-        h->pk_cy = cy;
-        h->pk_cz = C / cy;
-        h->pk_smem = bytes;
-        return GFMC_OK;
-    }
-    if (fp32) return GFMC_OK;
+    if (fp32 || h->pk != 0) return GFMC_OK;
     int max_ctas = 0;
     if ((e = gfmc::packed64_grid_max_ctas(0, &max_ctas)) != cudaSuccess) return cuda_fail(h, e, "querying grid occupancy");
     if (gfmc::pk_grid_split(h->L, h->K, max_ctas, dev_smem - st, &h->pk_cy, &h->pk_cz, &h->pk_smem)) {
@@ -915,7 +926,7 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
     int dev_smem = 0;
     if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
         return cuda_fail(nullptr, e, "querying shared memory");
-    const int reserve = 24 * 1024;  // static shared memory of the kernel and the parameter copy
+    const int reserve = 28 * 1024;  // static shared memory of the kernel and the parameter copy
     size_t vec_bytes = 0;
     std::vector<int> resident(n_chains, 0);
     for (int c = 0; c < n_chains; ++c) {
@@ -1489,7 +1500,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
     } else {
         int work = 0;
         for (int c = 0; c < n_chains; ++c) work = std::max(work, gfmc::engine_smem_bytes(chains[c]->K));
-        const int reserve = 24 * 1024;
+        const int reserve = 28 * 1024;
         size_t vec_bytes = 0;
         std::vector<int> resident(n_chains, 0);
         for (int c = 0; c < n_chains; ++c) {

@@ -269,6 +269,7 @@ cudaError_t cluster_max_active(int precision, int C, int smem, int* out);
 // cluster of C CTAs per job; 2 FP64 with small tiles (pk64_smem_bytes)
 cudaError_t launch_packed(int engine, const TeamJob* d_jobs, int njobs, int C, int smem, cudaStream_t s);
 cudaError_t launch_packed_single(int engine, const Params& p, int smem, cudaStream_t s);
+cudaError_t launch_packed64_moments(const Params& p, int smem, cudaStream_t s);
 cudaError_t packed_max_active(int engine, int C, int smem, int* out);
 cudaError_t packed_static_smem(int engine, int* out);
 // a single chain on one CTA: even L, at most kThreads sites (FP32: 2 kThreads)

@@ -61,6 +61,19 @@ cudaError_t launch_packed_single(int engine, const Params& p, int smem, cudaStre
     return cudaLaunchKernelEx(&cfg, fn, p);
 }
 
+// six clusters of p.ncta CTAs
+cudaError_t launch_packed64_moments(const Params& p, int smem, cudaStream_t s)
+{
+    cudaError_t e = allow_dynamic_smem((const void*)gfmc_packed64_moments);
+    if (e == cudaSuccess && p.ncta > 8)
+        e = cudaFuncSetAttribute((const void*)gfmc_packed64_moments, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg;
+    if (e == cudaSuccess) e = pk_config(2, 6, p.ncta, smem, s, &cfg, attr);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchKernelEx(&cfg, gfmc_packed64_moments, p);
+}
+
 cudaError_t packed_max_active(int engine, int C, int smem, int* out)
 {
     cudaLaunchAttribute attr[1];

@@ -848,6 +848,8 @@ struct PkHead {
     double2 c[kVec], hop[kVec];  // Delta~ |o> and Htilde_{o, l_k} at the local sites
     double chi[8][3];            // spinors of the local sites and of the proposal
     int loc[kVec];
+    int mom[kVec];               // moments calls: the local sites, and where their values go
+    unsigned row[2][kVec];
     double draw[3];
     double vv0;                  // <v|v>
     double2 ov1;                 // <o|Htilde|v>

@@ -387,11 +387,14 @@ __device__ __forceinline__ void pk64_xy(unsigned bonds, const PkTile& t, const P
 // KI = 0: whole sites s, s + 256, ... with bonds and S_{m-1} from shared memory.
 // Not inlined: with the tail in one function the registers that live across it
 // went to local memory inside the step loop.
-template <class Ex, int SPL, int KI>
+// MOM: no sums; instead the values at the local sites of a moments call, limbs as they
+// are, go to head.mom (pk64_moments), S_m to place m of the sites' rows.
+template <class Ex, int SPL, int KI, bool MOM = false>
 __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, const PkRec* tab, const PkHead& head,
                                           PkSums<double, kPk64Threads / 32>& sums, unsigned mb, unsigned ph,
                                           volatile int* s_fail)
 {
+    static_assert(!MOM || KI == 1, "one site per thread");
     static_assert(KI == 1 || SPL == 1, "one part of a site per thread");
     constexpr int NT = kPk64Threads, NW = NT / 32, ND = SPL == 4 ? 3 : 6, KR = KI > 0 ? KI : 1;
     const PkTile t = tile;
@@ -428,6 +431,20 @@ __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, c
         return store(t.ring + 16u * r.at + 8u * c, 0, 0, ex.target(r, c), __double2ll_rn((c ? v.y : v.x) * 0x1p60),
                      __double2ll_rn(v.y * 0x1p60));
     };
+    // MOM: byte offsets of place 0 of the rows that take this site's S_m, m even and odd; ~0u: none
+    [[maybe_unused]] unsigned row[2] = {~0u, ~0u};
+    [[maybe_unused]] auto sample = [&](int m, int4 v) {
+        const unsigned r = row[m & 1];
+        char* a = (char*)p.mom_out + r + 16u * (unsigned)m;
+        if constexpr (SPL == 1)
+            asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0xffffffff;\n @p st.global.v4.s32 [%0], {%1, %2, %3, %4};\n}" ::"l"(a),
+                         "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(r)
+                         : "memory");
+        else
+            asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %3, 0xffffffff;\n @p st.global.v2.s32 [%0], {%1, %2};\n}" ::"l"(a), "r"(v.x),
+                         "r"(v.y), "r"(r)
+                         : "memory");
+    };
     if constexpr (KI > 0) {
 #pragma unroll
         for (int k = 0; k < KI; ++k) {
@@ -439,6 +456,15 @@ __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, c
                 own[k] = t.ring + 16u * r.at + 8u * c;
                 tgt[k] = ex.target(r, c);
                 odd[k] = (r.fl >> 4) != 0;
+                if constexpr (MOM) {
+                    const int od = r.col >= t.half ? 1 : 0, x = 2 * (r.col - od * t.half) + od;
+                    const int i = x + t.L * (t.y0 + r.y + t.L * (t.z0 + r.z));
+                    for (int j = 0; j < kVec; ++j)
+                        if (i == head.mom[j] && hf == 0)
+                            for (int b = 0; b < 2; ++b)
+                                if (head.row[b][j] != ~0u) row[b] = head.row[b][j] + 8u * (unsigned)c;
+                    sample(0, cur[k]);
+                }
 #pragma unroll
                 for (int d = 0; d < ND; ++d) {
                     const int e = SPL == 4 ? 2 * d + hf : d;
@@ -519,7 +545,8 @@ __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, c
 #pragma unroll
             for (int k = 0; k < KI; ++k) {
                 if (tid + k * NT < T) {
-                    acc.add(cur[k], nx[k], odd[k] == oddA);
+                    if constexpr (MOM) sample(m + 1, nx[k]);
+                    else acc.add(cur[k], nx[k], odd[k] == oddA);
                     prv[k] = cur[k];
                     cur[k] = nx[k];
                 }
@@ -552,7 +579,9 @@ __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, c
             if (m == 0) s = (s + 1) >> 1;
             if (on) {
                 const int4 nx = store(own[0], b1, m + 1, tgt[0], s, 0);
-                if (hf == 0) {
+                if constexpr (MOM) {
+                    sample(m + 1, nx);
+                } else if (hf == 0) {
                     if (odd[0] == oddA) {
                         acc.square<0>(cur[0].x, cur[0].y);
                         pk_mac(acc.RA, acc.RB, cur[0].x, cur[0].y, nx.x, nx.y);
@@ -569,16 +598,16 @@ __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, c
                 cur[0] = nx;
             }
         }
-        if (m > 0) {
+        if (!MOM && m > 0) {
             acc.put();
             const long long w = warp_reduce_scatter4(acc.v, lane);
             if ((lane & 7) == 0) sums.w[m & (kPkRing - 1)][warp][lane >> 3] = w;
         }
         // warps take turns (a barrier lies between the sums of the flushed steps and this)
-        if ((m & (kPkGroup - 1)) == 1) pk_flush_due<double, NW>(p, sums, m, warp ^ ((m >> 3) & (NW - 1)), lane);
+        if (!MOM && (m & (kPkGroup - 1)) == 1) pk_flush_due<double, NW>(p, sums, m, warp ^ ((m >> 3) & (NW - 1)), lane);
     }
     __syncthreads();
-    pk_flush_rest<double, NW>(p, sums, nsteps, warp, lane);
+    if (!MOM) pk_flush_rest<double, NW>(p, sums, nsteps, warp, lane);
     return true;
 }
 
@@ -683,6 +712,86 @@ template <bool GRID> __device__ __forceinline__ void pk64_run_chain(const Params
         }
         sync(0);  // no CTA leaves while another may still write into its shared memory
     }
+}
+
+// All moments <l_j|T_n(Htilde)|l_k>, n < M, of the seven local sites of p.site, by six
+// clusters, each on its own vector through M - 1 steps: cluster v > 0 on l_{v+1}, cluster 0 on
+// o + l_1 (opposite parities).  The values at the local sites are the moments, so a step
+// has no sums and the clusters do not meet; against the recursion on seven vectors to
+// M/2 with the sums of 28 pairs of products (a grid of flags), L = 12, M = 512:
+// 1346 -> 362 us per call, bound by the latency of a step (0.57 us).  Up to L = 16, a site
+// per thread; FP32-mixed chains take it as well, with the FP64 bonds.
+__global__ void __launch_bounds__(kPk64Threads, 1) gfmc_packed64_moments(const Params q)
+{
+    extern __shared__ double2 dyn_all[];
+    __shared__ Params p;
+    __shared__ PkSums<double, kPk64Threads / 32> sums;
+    __shared__ PkHead head;
+    __shared__ PkTile t;
+    __shared__ int s_fail;
+    __shared__ __align__(8) unsigned long long s_mb[2];
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int tid = threadIdx.x, rank = (int)cl.block_rank(), C = (int)cl.dim_blocks().x, v = (int)blockIdx.x / C;
+    const int kcol = v + 1, M = q.M;  // the column of the cluster's l
+    if (tid == 0) {
+        p = q;
+        p.nsteps = M - 2;  // S_{M-1} is the last vector
+        t = pk_tile<double>(p, rank, (char*)dyn_all);
+        s_fail = 0;
+        const int o = (int)p.site;
+        for (int j = 0; j < kVec; ++j) {
+            head.mom[j] = j == 0 ? o : nbr_site(o, j - 1, p.L);
+            // row (j, k) of the moment matrix, j <= k
+            const unsigned rj = 16u * (unsigned)(M * (kVec * j + kcol));
+            for (int b = 0; b < 2; ++b) head.row[b][j] = v > 0 && j <= kcol ? rj : ~0u;
+            head.loc[j] = -1;
+            head.c[j] = make_double2(1.0, 0.0);
+        }
+        if (v == 0) {
+            // at o: T_m|o> for even m, T_m|l_1> for odd m; at l_1: T_m|l_1> for even m
+            head.row[0][0] = 0u;
+            head.row[1][0] = 16u * (unsigned)M;
+            head.row[0][1] = 16u * (unsigned)(M * (kVec + 1));
+            head.row[1][1] = ~0u;
+            head.loc[0] = o;
+            head.loc[1] = head.mom[1];
+        } else {
+            head.loc[0] = head.mom[kcol];
+        }
+    }
+    __syncthreads();
+    PkRec* tab = (PkRec*)(t.bonds + (size_t)t.bond_rows() * t.rowB);
+    pk64_records(t, tab);
+    if (tid == 0) PkAsyncEx(t, p, smem_u32(s_mb), 0).init();
+    pk_load_bonds<double, kPk64Threads>(p, t);
+    cl.sync();  // every CTA has initialised its barriers before any remote store
+    const int T = t.L * t.PY * t.PZ;
+    const unsigned mb = smem_u32(s_mb);
+    constexpr int NT = kPk64Threads;
+    if (4 * T <= NT) pk64_advance<PkAsyncEx, 4, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
+    else if (2 * T <= NT) pk64_advance<PkAsyncEx, 2, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
+    else pk64_advance<PkAsyncEx, 1, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
+    if (s_fail) {  // values still in flight land before any CTA leaves
+        const long long t0 = clock64();
+        while (clock64() - t0 < (1ll << 21)) __nanosleep(256);
+    }
+    __threadfence();
+    cl.sync();
+    // limbs to values, and the conjugates below the diagonal
+    for (int k = v == 0 ? 0 : kcol; k <= kcol; ++k)
+        for (int e = rank * NT + tid; e < (k + 1) * M; e += C * NT) {
+            const int j = e / M, n = e - j * M;
+            double2* a = p.mom_out + (size_t)(kVec * j + k) * M + n;
+            const bool live = ((n + (j > 0 ? 1 : 0) + (k > 0 ? 1 : 0)) & 1) == 0;
+            double2 m = make_double2(0.0, 0.0);
+            if (live) {
+                const int4 w = __ldcg((const int4*)a);
+                m = make_double2((double)pk_join(w.x, w.y) * 0x1p-60, (double)pk_join(w.z, w.w) * 0x1p-60);
+            }
+            if (j == k) m.y = 0.0;
+            __stcg(a, m);
+            if (j < k) __stcg(p.mom_out + (size_t)(kVec * k + j) * M + n, make_double2(m.x, -m.y));
+        }
 }
 
 __global__ void __launch_bounds__(kPk64Threads, 1) gfmc_packed64_cluster(const TeamJob* __restrict__ jobs)

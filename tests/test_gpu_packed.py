@@ -142,3 +142,18 @@ def test_fp32_single_chains_match_oracle(G, L, M, nodes, n):
         out = ch.updates(n)
         replay(L, sp, M, nodes, 3, out, lambda r: 2e-5, 1e-3)
         assert out["magnetization"].size == n // L ** 3
+
+
+@pytest.mark.parametrize("L,M", [(4, 16), (4, 64), (6, 64), (8, 32), (10, 32), (12, 16), (14, 16), (16, 64)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32_mixed"])
+def test_moments_on_clusters_match_oracle(G, L, M, precision):
+    """Moments read off six vectors on clusters: 1/4 of a site, half a site and a
+    whole site per thread, sites on every face of the lattice.  Tolerance: 2^-60 per
+    step and site, and the oracle's doubling, 1e-13 for values <= 1."""
+    sp = inputs.von_mises_fisher(L, 2.0, L)
+    with G.Chain(L, sp, M=M, precision=precision) as ch:
+        for o in (0, L ** 3 - 1, L ** 3 // 2 + 3):
+            mu = ch.moments(o)
+            assert np.abs(mu - O.moments(L, sp, o, M)).max() <= 1e-13
+            assert np.array_equal(mu, mu.transpose(1, 0, 2).conj())
+        assert np.array_equal(mu, ch.moments(o))
