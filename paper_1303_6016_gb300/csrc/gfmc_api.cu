@@ -251,15 +251,66 @@ size_t team_vec_bytes(const gfmc_ctx* h, int tc)
     return tc <= 1 ? 2 * (size_t)nv * h->N * vsz : SIZE_MAX;
 }
 
-// the vectors of every job's recursion, 0 when they differ; 1: all on the packed one
-int common_nv(const gfmc::TeamJob* jobs, size_t n)
+bool team_packed(const gfmc_ctx* h) { return team_nv(h) == 2 && h->L % 2 == 0 && !h->P.comp; }
+
+// the vectors of every chain's recursion on a team, 0 when they differ; 1: all on the packed one
+int common_nv(gfmc_ctx* const* chains, int n)
 {
     bool packed = true;
-    for (size_t j = 0; j < n; ++j) {
-        if (jobs[j].p.nv != jobs[0].p.nv) return 0;
-        packed = packed && jobs[j].p.nv == 2 && jobs[j].p.L % 2 == 0 && !jobs[j].p.comp;
+    for (int c = 0; c < n; ++c) {
+        if (team_nv(chains[c]) != team_nv(chains[0])) return 0;
+        packed = packed && team_packed(chains[c]);
     }
-    return packed ? 1 : jobs[0].p.nv;
+    return packed ? 1 : team_nv(chains[0]);
+}
+
+// Dynamic shared memory of a launch of teams: the vector area of the chains that
+// keep their vectors there and the work area of the largest chain (none where every
+// chain is packed and resident: its work area is then the vectors').  What is left
+// holds bonds of the packed chains of more sites than registers take.
+struct TeamSmem {
+    std::vector<int> resident;
+    int vec_bytes = 0, smem = 0, nv = 0;
+};
+gfmc_status plan_team_smem(gfmc_ctx* const* chains, int n, const int* ctas, TeamSmem* out)
+{
+    const bool comp = chains[0]->P.comp != 0;
+    const int prec = chains[0]->precision;
+    const int vsz = prec == GFMC_PREC_FP64 ? (int)sizeof(double2) : (int)sizeof(float2);
+    cudaError_t e;
+    int dev_smem = 0, stat = 0;
+    // the FP64 and the compensated kernel hold every recursion
+    out->nv = prec == GFMC_PREC_FP32_MIXED && !comp ? common_nv(chains, n) : 0;
+    if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, chains[0]->device)) != cudaSuccess ||
+        (e = gfmc::team_static_smem(prec, comp, out->nv, &stat)) != cudaSuccess)
+        return cuda_fail(nullptr, e, "querying shared memory");
+    int K = 0, work = 0;
+    for (int c = 0; c < n; ++c) K = std::max(K, chains[c]->K);
+    work = out->nv == 1 ? K * (int)sizeof(double2) : gfmc::engine_smem_bytes(K);
+    size_t vec = 0, want = 0;
+    bool all = true;
+    out->resident.assign(n, 0);
+    for (int c = 0; c < n; ++c) {
+        const gfmc_ctx* h = chains[c];
+        const int tc = std::max(ctas ? ctas[c] : 1, 1);
+        const size_t vb = team_vec_bytes(h, tc);
+        if (vb == SIZE_MAX || vb + work + stat > (size_t)dev_smem) {
+            all = false;
+            continue;
+        }
+        out->resident[c] = 1;
+        vec = std::max(vec, vb);
+        if (team_packed(h)) want = std::max(want, vb + 3 * (size_t)vsz * ((h->N + tc - 1) / tc) + (size_t)vsz * h->L * h->L);
+    }
+    if (out->nv == 1 && vec > 0) {
+        vec = std::max(vec, (size_t)work);
+        if (all) work = 0;
+    }
+    if (vec > 0) vec = std::max(vec, std::min(want, (size_t)(dev_smem - stat - work)));
+    out->vec_bytes = (int)((vec + 15) & ~(size_t)15);
+    if (out->vec_bytes + work + stat > dev_smem) out->vec_bytes -= 16;
+    out->smem = out->vec_bytes + work;
+    return GFMC_OK;
 }
 
 // Run one engine launch and wait for it; translate the device error word.
@@ -290,7 +341,7 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
         P.pk_cy = h->pk_cy;
         P.pk_cz = h->pk_cz;
         if (h->pk == 3) {
-            e = gfmc::launch_one_cta(h->precision, P, h->pk_smem, h->stream);
+            e = gfmc::launch_one_cta(h->pk_engine, P, h->pk_smem, h->stream);
         } else if (h->pk == 1) {
             e = gfmc::launch_packed_single(h->pk_engine, P, h->pk_smem, h->stream);
         } else {
@@ -310,7 +361,7 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
         const int smem = gfmc::engine_smem_bytes(P.K);
         e = h->precision == GFMC_PREC_FP64 ? gfmc::launch_team_f64(h->d_job, 1, P.ncta, 0, smem, h->stream)
                                             : gfmc::launch_team_f32(h->d_job, 1, P.ncta, 0, smem, h->stream, P.comp != 0,
-                                                                    common_nv(&job, 1));
+                                                                    (P.nv == 2 && h->L % 2 == 0 && !P.comp) ? 1 : P.nv);
     } else {
         if (h->vcl && nv == gfmc::kVec)
             e = gfmc::launch_vcluster_f32(P, h->stream);
@@ -417,9 +468,9 @@ gfmc_status use_team_plan(gfmc_ctx* h, int tc)
 
 // The packed engine of a chain's Delta Omega calls (automatic engine, even L,
 // plain sums), if one takes it.  Measured, us per update at M = 1024:
-//   One CTA (gfmc_team.cuh) up to 512 sites in FP32, 256 in FP64: FP32-mixed L = 4: 156,
-//   on a cluster of 1 to 16 CTAs 276-342; L = 8: 246, on clusters 326-348.  FP64
-//   L = 4: 173, L = 6: 332; L = 8, one site per thread of 512, 669 and on 16 CTAs 425.
+//   One CTA (gfmc_team.cuh) up to 512 sites in FP32, 256 in FP64: FP32-mixed L = 8: 246,
+//   on clusters 326-348; L = 4: 156, on a cluster 276-342 (kOneCtaExact: 173 in fixed
+//   point).  FP64 L = 4: 173, L = 6: 332; L = 8, one site per thread of 512, 669 and on 16 CTAs 425.
 //   FP32-mixed, one cluster of C CTAs: L = 16: 1173 on 1, 443 on 4, 353 on 16; L = 24:
 //   628 on 8, 446 on 16.  So the most CTAs that split the lattice.  L = 32 stays on the
 //   seven vector clusters (767; one packed cluster 643), whose moments without the
@@ -462,13 +513,14 @@ gfmc_status plan_packed(gfmc_ctx* h)
         h->pk_cz = h->pk_ctas / h->pk_cy;
     }
     if (h->N <= (fp32 ? 2 : 1) * gfmc::kThreads) {
-        const int prec = h->precision;
+        const int prec = h->N <= gfmc::kOneCtaExact ? GFMC_PREC_FP64 : h->precision;
         const int NT = gfmc::one_cta_threads(prec, h->N);
         // the tail's four sequences at once where they fit in a third of the SM's shared memory
-        const int vec = fp32 ? gfmc::one_cta_bytes<float>(h->N, NT) : gfmc::kOneCtaHist * 16 * h->N;
+        const int vec = prec != GFMC_PREC_FP64 ? gfmc::one_cta_bytes<float>(h->N, NT) : gfmc::kOneCtaHist * 16 * h->N;
         const int bytes = std::max({vec, 8 * h->K, std::min(32 * h->K, 72 * 1024)});
         if (gfmc::one_cta_fits(prec, h->N, bytes)) {
             h->pk = 3;
+            h->pk_engine = prec;
             h->pk_ctas = h->pk_cy = h->pk_cz = 1;
             h->pk_smem = bytes;
             return GFMC_OK;
@@ -590,7 +642,7 @@ gfmc_status gfmc_create(int L, const double* spins, double t, double mu, double 
     if ((e = gfmc::engine_max_ctas(h->precision, K, &maxc)) != cudaSuccess)
         return bail(cuda_fail(h, e, "querying engine occupancy"));
     int maxt = 0;
-    if ((e = gfmc::team_max_ctas(h->precision, gfmc::engine_smem_bytes(K), &maxt)) != cudaSuccess)
+    if ((e = gfmc::team_max_ctas(h->precision, gfmc::engine_smem_bytes(K), opt.compensated != 0, -1, &maxt)) != cudaSuccess)
         return bail(cuda_fail(h, e, "querying team occupancy"));
     maxc = std::min(maxc, maxt);
     if (opt.engine != GFMC_ENGINE_GRID && h->precision == GFMC_PREC_FP32_MIXED && L == gfmc::kVcLattice) {
@@ -920,28 +972,15 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e;
     if ((e = cudaSetDevice(dev)) != cudaSuccess) return cuda_fail(nullptr, e, "cudaSetDevice");
-    // Shared memory: the largest resident lattice plus the work area of the largest M.
-    int work = 0;
-    for (int c = 0; c < n_chains; ++c) work = std::max(work, gfmc::engine_smem_bytes(chains[c]->K));
-    int dev_smem = 0;
-    if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
-        return cuda_fail(nullptr, e, "querying shared memory");
-    const int reserve = 28 * 1024;  // static shared memory of the kernel and the parameter copy
-    size_t vec_bytes = 0;
-    std::vector<int> resident(n_chains, 0);
-    for (int c = 0; c < n_chains; ++c) {
-        const int tc = team_ctas ? team_ctas[c] : 1;
-        const size_t vb = team_vec_bytes(chains[c], std::max(tc, 1));
-        if (vb != SIZE_MAX && vb + work + reserve <= (size_t)dev_smem) {
-            resident[c] = 1;
-            vec_bytes = std::max(vec_bytes, (vb + 255) & ~(size_t)255);
-        }
-    }
-    const int smem = (int)vec_bytes + work;
+    TeamSmem tm;
+    if (const gfmc_status st = plan_team_smem(chains, n_chains, team_ctas, &tm); st != GFMC_OK) return st;
+    const int smem = tm.smem, vec_bytes = tm.vec_bytes;
+    const std::vector<int>& resident = tm.resident;
     int grid = 0;
     for (int c = 0; c < n_chains; ++c) grid += team_ctas ? team_ctas[c] : 1;
     int maxc = 0;
-    if ((e = gfmc::team_max_ctas(prec, smem, &maxc)) != cudaSuccess) return cuda_fail(nullptr, e, "team occupancy");
+    if ((e = gfmc::team_max_ctas(prec, smem, chains[0]->P.comp != 0, tm.nv, &maxc)) != cudaSuccess)
+        return cuda_fail(nullptr, e, "team occupancy");
     if (grid > maxc)
         return fail(nullptr, GFMC_EINVAL, "the batch needs %d co-resident CTAs, the device holds %d at %d B of "
                     "shared memory; run it in smaller parts", grid, maxc, smem);
@@ -999,7 +1038,7 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
         return cuda_fail(nullptr, e, "uploading the job table");
     e = prec == GFMC_PREC_FP64 ? gfmc::launch_team_f64(d_jobs, n_chains, grid, (int)vec_bytes, smem, s)
                                : gfmc::launch_team_f32(d_jobs, n_chains, grid, (int)vec_bytes, smem, s,
-                                                       chains[0]->P.comp != 0, common_nv(jobs.data(), jobs.size()));
+                                                       chains[0]->P.comp != 0, tm.nv);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "launching the batch");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(nullptr, e, "batch execution");
     gfmc_status result = GFMC_OK;
@@ -1439,6 +1478,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
         return P;
     };
     int team_grid = 0, team_smem = 0, team_vec = 0;
+    TeamSmem tplan;
     if (clusters) {
         int static_smem[2] = {0, 0};
         if ((e = gfmc::cluster_static_smem(GFMC_PREC_FP64, &static_smem[0])) != cudaSuccess ||
@@ -1498,23 +1538,13 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
             groups.push_back(g);
         }
     } else {
-        int work = 0;
-        for (int c = 0; c < n_chains; ++c) work = std::max(work, gfmc::engine_smem_bytes(chains[c]->K));
-        const int reserve = 28 * 1024;
-        size_t vec_bytes = 0;
-        std::vector<int> resident(n_chains, 0);
-        for (int c = 0; c < n_chains; ++c) {
-            const size_t vb = team_vec_bytes(chains[c], std::max(ctas[c], 1));
-            if (vb != SIZE_MAX && vb + work + reserve <= (size_t)dev_smem) {
-                resident[c] = 1;
-                vec_bytes = std::max(vec_bytes, (vb + 255) & ~(size_t)255);
-            }
-        }
-        team_vec = (int)vec_bytes;
-        team_smem = (int)vec_bytes + work;
+        if (const gfmc_status st = plan_team_smem(chains, n_chains, ctas, &tplan); st != GFMC_OK) return bail(st);
+        const std::vector<int>& resident = tplan.resident;
+        team_vec = tplan.vec_bytes;
+        team_smem = tplan.smem;
         for (int c = 0; c < n_chains; ++c) team_grid += ctas[c];
         int maxc = 0;
-        if ((e = gfmc::team_max_ctas(prec, team_smem, &maxc)) != cudaSuccess)
+        if ((e = gfmc::team_max_ctas(prec, team_smem, chains[0]->P.comp != 0, tplan.nv, &maxc)) != cudaSuccess)
             return bail(cuda_fail(nullptr, e, "team occupancy"));
         if (team_grid > maxc)
             return bail(fail(nullptr, GFMC_EINVAL, "the batch needs %d co-resident CTAs, the device holds %d", team_grid,
@@ -1581,7 +1611,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
     if (ce == cudaSuccess && !clusters) {
         ce = prec == GFMC_PREC_FP64 ? gfmc::launch_team_ex_f64(p->d_jobs, nj, team_grid, team_vec, team_smem, cs)
                                     : gfmc::launch_team_ex_f32(p->d_jobs, nj, team_grid, team_vec, team_smem, cs,
-                                                               chains[0]->P.comp != 0, common_nv(jobs.data(), jobs.size()));
+                                                               chains[0]->P.comp != 0, tplan.nv);
     } else if (ce == cudaSuccess) {
         cudaEvent_t fork = nullptr;
         ce = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);

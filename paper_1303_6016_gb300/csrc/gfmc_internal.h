@@ -254,7 +254,10 @@ cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_
 // nv: the vectors of every job's recursion (p.nv), 0 when they differ; 1: even lattices on two vectors only
 cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
                             bool comp, int nv);
-cudaError_t team_max_ctas(int precision, int smem, int* out);
+// co-resident CTAs of the kernel launch_team_* takes for comp and nv, and its static shared memory
+// (bytes); nv < 0: the fewest of any
+cudaError_t team_max_ctas(int precision, int smem, bool comp, int nv, int* out);
+cudaError_t team_static_smem(int precision, bool comp, int nv, int* out);
 // launch_team_* through cudaLaunchKernelEx with the cooperative attribute (capturable in a CUDA graph)
 cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s);
 cudaError_t launch_team_ex_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
@@ -275,6 +278,10 @@ cudaError_t packed_static_smem(int engine, int* out);
 // a single chain on one CTA: even L, at most kThreads sites (FP32: 2 kThreads)
 // (FP64: at most kThreads that advance the sites, and eight warps for the sums)
 inline int one_cta_threads(int precision, int N) { return precision != 0 && N <= kThreads ? kThreads : 2 * kThreads; }
+// FP32-mixed chains on one CTA up to this size (L = 4) run the FP64 chains' fixed point: their
+// few levels stand apart at the resolution of a large M, which magnifies the rounding of FP32
+// vectors to 1e-6 t (L = 4, M = 1024; L = 6: 2e-7), and the steps are bound by latency either way.
+constexpr int kOneCtaExact = 64;
 constexpr int kOneCtaHist = 32;  // vectors an FP64 chain keeps in shared memory
 cudaError_t launch_one_cta(int precision, const Params& p, int smem, cudaStream_t s);
 bool one_cta_fits(int precision, int N, int smem);

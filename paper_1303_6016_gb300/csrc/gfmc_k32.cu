@@ -105,16 +105,35 @@ static cudaError_t team_occupancy(int smem, int* out)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, gfmc_team_engine<float, NV, COMP>, kThreads, smem);
 }
 
-// of the kernel that holds the fewest, so that a batch fits whichever it runs
-cudaError_t team_max_ctas_f32(int smem, int* out)
+cudaError_t team_max_ctas_f32(int smem, bool comp, int nv, int* out)
 {
-    int n[5] = {};
-    cudaError_t e = team_occupancy<0, false>(smem, &n[0]);
-    if (e == cudaSuccess) e = team_occupancy<0, true>(smem, &n[1]);
-    if (e == cudaSuccess) e = team_occupancy<2, false>(smem, &n[2]);
-    if (e == cudaSuccess) e = team_occupancy<kVec, false>(smem, &n[3]);
-    if (e == cudaSuccess) e = team_occupancy<1, false>(smem, &n[4]);
-    if (e == cudaSuccess) *out = *std::min_element(n, n + 5);
+    if (nv < 0) {  // of the kernel that holds the fewest
+        *out = 1 << 30;
+        for (int k = 0; k < 5; ++k) {
+            const int kinds[5] = {0, 1, 2, kVec, 0};
+            int n = 0;
+            const cudaError_t e = team_max_ctas_f32(smem, k == 4, kinds[k], &n);
+            if (e != cudaSuccess) return e;
+            *out = std::min(*out, n);
+        }
+        return cudaSuccess;
+    }
+    if (comp) return team_occupancy<0, true>(smem, out);
+    if (nv == 1) return team_occupancy<1, false>(smem, out);
+    if (nv == 2) return team_occupancy<2, false>(smem, out);
+    if (nv == kVec) return team_occupancy<kVec, false>(smem, out);
+    return team_occupancy<0, false>(smem, out);
+}
+
+cudaError_t team_static_smem_f32(bool comp, int nv, int* out)
+{
+    cudaFuncAttributes a;
+    const cudaError_t e = comp ? cudaFuncGetAttributes(&a, gfmc_team_engine<float, 0, true>)
+                          : nv == 1 ? cudaFuncGetAttributes(&a, gfmc_team_engine<float, 1, false>)
+                          : nv == 2 ? cudaFuncGetAttributes(&a, gfmc_team_engine<float, 2, false>)
+                          : nv == kVec ? cudaFuncGetAttributes(&a, gfmc_team_engine<float, kVec, false>)
+                                       : cudaFuncGetAttributes(&a, gfmc_team_engine<float, 0, false>);
+    if (e == cudaSuccess) *out = (int)a.sharedSizeBytes;
     return e;
 }
 

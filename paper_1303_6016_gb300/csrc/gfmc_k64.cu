@@ -81,6 +81,14 @@ cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int v
     return cudaLaunchKernelEx(&cfg, gfmc_team_engine<double, 0>, d_jobs, njobs, vec_bytes);
 }
 
+cudaError_t team_static_smem_f64(int* out)
+{
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, gfmc_team_engine<double, 0>);
+    if (e == cudaSuccess) *out = (int)a.sharedSizeBytes;
+    return e;
+}
+
 cudaError_t team_max_ctas_f64(int smem, int* out)
 {
     cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double, 0>);

@@ -106,8 +106,8 @@ __global__ void __launch_bounds__(kThreads, 1) gfmc_server_kernel(ServerArgs a)
         if (cmd == kExit) return;
         last = cmd;
         if (sp.nv == 2 && sp.L % 2 == 0) {
-            if (s_prec == 0) pk_team_chain<double, kThreads, kServer>(sp, s_cta, (char*)work, sp.K, false);
-            else pk_team_chain<float, kThreads, kServer>(sp, s_cta, (char*)work, sp.K, false);
+            if (s_prec == 0) pk_team_chain<double, kThreads, kServer>(sp, s_cta, (char*)work, sp.K, 0);
+            else pk_team_chain<float, kThreads, kServer>(sp, s_cta, (char*)work, sp.K, 0);
         } else if (s_prec == 0) {
             if (sp.nv == 2) run_chain<double, 1, 2, kThreads, false>(sp, s_cta, work, nullptr);
             else run_chain<double, 1, kVec, kThreads, false>(sp, s_cta, work, nullptr);

@@ -11,12 +11,19 @@ namespace gfmc {
 cudaError_t engine_max_ctas_f64(int K, int* out);
 cudaError_t engine_max_ctas_f32(int K, int* out);
 cudaError_t team_max_ctas_f64(int smem, int* out);
-cudaError_t team_max_ctas_f32(int smem, int* out);
+cudaError_t team_max_ctas_f32(int smem, bool comp, int nv, int* out);
+cudaError_t team_static_smem_f64(int* out);
+cudaError_t team_static_smem_f32(bool comp, int nv, int* out);
 
-cudaError_t team_max_ctas(int precision, int smem, int* out)
+cudaError_t team_static_smem(int precision, bool comp, int nv, int* out)
+{
+    return precision == 0 ? team_static_smem_f64(out) : team_static_smem_f32(comp, nv, out);
+}
+
+cudaError_t team_max_ctas(int precision, int smem, bool comp, int nv, int* out)
 {
     int per_sm = 0;
-    cudaError_t e = precision == 0 ? team_max_ctas_f64(smem, &per_sm) : team_max_ctas_f32(smem, &per_sm);
+    cudaError_t e = precision == 0 ? team_max_ctas_f64(smem, &per_sm) : team_max_ctas_f32(smem, comp, nv, &per_sm);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -6,9 +6,14 @@
 // vectors stay in registers, a step's products are formed under the next step's
 // loads, and they are added over the threads by the eight steps, not by a warp
 // reduction in each.  us per step (a default chain, before the packed recursion on one
-// CTA and now): FP32 on a team of one CTA, L = 4 0.77 -> 0.27, L = 8 0.97 -> 0.43; FP64
+// CTA and now): FP32 on a team of one CTA, L = 8 0.97 -> 0.40, L = 4 0.77 -> 0.27 (0.62 in the
+// fixed point it takes for its accuracy); FP64
 // alone, L = 4 0.82 (a cluster) -> 0.30; the tail of a team's update 49 -> 29 us.
-// Larger tiles by their bonds' and vectors' loads: L = 32 on 5 CTAs 11.4 us.
+// Larger tiles by the latency of their loads and index arithmetic, two warps per
+// sub-partition: with the bonds in shared memory L = 16 on one CTA 5.6 -> 4.3 us, L = 24
+// on three 7.9 -> 6.8, L = 32 on eight 8.2 -> 7.3.  Sixteen warps would add a chain's FP32
+// sums in another order than a launch that also holds odd lattices; four sites per
+// pass spill (5.5 us).
 #pragma once
 
 #include "gfmc_packed.cuh"
@@ -407,15 +412,17 @@ template <class R> __device__ __forceinline__ const typename Cx<R>::T* hop_table
 
 // A team CTA of any number of sites.
 // WIN: S_m and S_{m-1} of the CTA's sites and of the planes before and after
-// them stand in shared memory (buf: two buffers of W sites); only those planes
-// -- 2 L^2 sites -- come from the other CTAs' stores each step.  The sites
+// them stand in shared memory (buf: two buffers of W sites; behind them, in what is
+// left of `bytes`, the forward bonds of the tile's first Tb sites and the z bonds of
+// the plane before it); only those planes -- 2 L^2 sites -- come from the other
+// CTAs' stores each step.  The sites
 // within a plane of the tile's ends go first and are published before the
 // others are computed, so the neighbours' wait overlaps the rest of the step.
 // Without WIN (tiles below a plane, or too large for shared memory) all values
 // are read from global memory.
 template <class R, bool WIN, bool WIDE>
-__device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigned phase, unsigned buf, const PkHead& head,
-                                               StepSums<R>& sums)
+__device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigned phase, unsigned buf, int bytes,
+                                               const PkHead& head, StepSums<R>& sums)
 {
     using R2 = typename Cx<R>::T;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -436,6 +443,21 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
     constexpr unsigned kB = sizeof(R2);
     const unsigned b0 = buf, b1 = buf + kB * (unsigned)W;  // WIN
     auto wrap = [&](int i) { return i < 0 ? i + N : i >= N ? i - N : i; };
+
+    // bonds in shared memory: x and y of sites k < Tb at k, z of site k at LLw + k
+    const int LLw = whole ? 0 : LL;
+    const int Tb = WIN && (!whole || p.ncta == 1)
+                       ? max(0, min(T, (bytes - (int)kB * (2 * W + LLw)) / (3 * (int)kB))) : 0;
+    const unsigned hx = b0 + 2u * kB * (unsigned)W, hy = hx + kB * (unsigned)Tb, hz = hy + kB * (unsigned)Tb;
+    if constexpr (WIN) {
+        for (int k = tid; k < Tb; k += kThreads) {
+            sts_v(hx + kB * k, ldcg2(hop + (s0 + k)));
+            sts_v(hy + kB * k, ldcg2(hop + (N + s0 + k)));
+            sts_v(hz + kB * (LLw + k), ldcg2(hop + (2 * N + s0 + k)));
+        }
+        if (Tb > 0)
+            for (int k = tid; k < LLw; k += kThreads) sts_v(hz + kB * k, ldcg2(hop + (2 * N + wrap(s0 - LL + k))));
+    }
 
     const int n0 = WIN ? W : T, f0 = WIN ? base : s0;
     for (int w = tid; w < n0; w += kThreads) {
@@ -494,12 +516,22 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
             const int yp = y == L - 1 ? L - LL : L, ym = y == 0 ? LL - L : -L;
             const int zm = z == 0 ? N - LL : -LL;
             const int wzp = whole && z == L - 1 ? LL - N : LL, wzm = whole ? zm : -LL;
-            q.h[0] = ldcg2(hop + i);
-            q.h[1] = ldcg2(hop + (i + xm));
-            q.h[2] = ldcg2(hop + (N + i));
-            q.h[3] = ldcg2(hop + (N + i + ym));
-            q.h[4] = ldcg2(hop + (2 * N + i));
-            q.h[5] = ldcg2(hop + (2 * N + i + zm));
+            const int kz = whole ? k + zm : k;  // place of the lower z bond
+            if (WIN && k < Tb && (unsigned)(k + xm) < (unsigned)Tb && (unsigned)(k + ym) < (unsigned)Tb && kz < LLw + Tb) {
+                q.h[0] = lds_v(hx + kB * (unsigned)k, R2());
+                q.h[1] = lds_v(hx + kB * (unsigned)(k + xm), R2());
+                q.h[2] = lds_v(hy + kB * (unsigned)k, R2());
+                q.h[3] = lds_v(hy + kB * (unsigned)(k + ym), R2());
+                q.h[4] = lds_v(hz + kB * (unsigned)(LLw + k), R2());
+                q.h[5] = lds_v(hz + kB * (unsigned)kz, R2());
+            } else {
+                q.h[0] = ldcg2(hop + i);
+                q.h[1] = ldcg2(hop + (i + xm));
+                q.h[2] = ldcg2(hop + (N + i));
+                q.h[3] = ldcg2(hop + (N + i + ym));
+                q.h[4] = ldcg2(hop + (2 * N + i));
+                q.h[5] = ldcg2(hop + (2 * N + i + zm));
+            }
             q.nv[0] = ld(i, q.w, xp);
             q.nv[1] = ld(i, q.w, xm);
             q.nv[2] = ld(i, q.w, yp);
@@ -561,12 +593,12 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
 // one chain
 // ---------------------------------------------------------------------------
 // A chain on the p.ncta CTAs of a team, this one its CTA `cta`.  smem: room for
-// work_n double2 at least; vec: the vectors stand there too (team_vec_bytes), the
-// tail's work space in their place after the steps.  USE: kTeam all paths, kOne a chain
+// work_n double2 at least; bytes > 0: the vectors stand there too (`bytes`, at least
+// team_vec_bytes), the tail's work space in their place after the steps.  USE: kTeam all paths, kOne a chain
 // of at most NT sites on one CTA, kServer no vectors in shared memory.
 enum { kTeam, kOne, kServer };
 template <class R, int NT, int USE>
-__device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, char* smem, int work_n, bool vec)
+__device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, char* smem, int work_n, int bytes)
 {
     __shared__ PkHead head;
     [[maybe_unused]] __shared__ StepSums<R> sums;
@@ -588,7 +620,7 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
         __syncthreads();
         bool done = false;
         if constexpr (USE != kServer) {
-            if (USE == kOne || (vec && C == 1 && N <= one_cta_sites<R>(NT))) {
+            if (USE == kOne || (bytes > 0 && C == 1 && N <= one_cta_sites<R>(NT))) {
                 const unsigned ring = buf + 2u * (unsigned)(sizeof(typename OneCta<R>::V) * N);
                 const int ntr = one_cta_items(N, NT);
                 if constexpr (USE == kOne && sizeof(R) == 8) {
@@ -599,6 +631,9 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
                     } else if (tid < nt) {
                         one_cta_products(p, head, buf, (tid - nm) >> 5, nt);
                     }
+                } else if (sizeof(R) == 4 && USE == kTeam && N <= kOneCtaExact) {
+                    // FP32-mixed chains of the smallest lattice in fixed point as well
+                    one_cta_steps<double, NT, 1>(p, head, buf, buf + 32u * (unsigned)N, ntr);
                 } else if (USE == kOne || N <= NT) {
                     one_cta_steps<R, NT, 1>(p, head, buf, ring, ntr);
                 }
@@ -613,13 +648,13 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
             }
         }
         if constexpr (USE == kTeam) {
-            if (!done && vec) {
-                if (!team_packed_steps<R, true, true>(p, cta, phase, buf, head, sums)) return;
+            if (!done && bytes > 0) {
+                if (!team_packed_steps<R, true, true>(p, cta, phase, buf, bytes, head, sums)) return;
                 done = true;
             }
         }
         if constexpr (USE != kOne) {
-            if (!done && !team_packed_steps<R, false, USE == kTeam>(p, cta, phase, buf, head, sums)) return;
+            if (!done && !team_packed_steps<R, false, USE == kTeam>(p, cta, phase, buf, 0, head, sums)) return;
         }
         phase += (unsigned)p.nsteps + 1u;
         if (!sync(1)) return;
@@ -655,11 +690,11 @@ __global__ void __launch_bounds__(NT, 1) gfmc_one_cta(const Params p, int work_n
     __shared__ Params sp;
     if (threadIdx.x == 0) sp = p;
     __syncthreads();
-    pk_team_chain<R, NT, kOne>(sp, 0, (char*)dyn_all, work_n, true);
+    pk_team_chain<R, NT, kOne>(sp, 0, (char*)dyn_all, work_n, 1);
 }
 
 // A batch of chains, each on its own team of CTAs (jobs sorted by cta0).
-// The dynamic shared memory holds [vector area of vec_bytes][work area].
+// The dynamic shared memory holds [vector area of vec_bytes][work area] (plan_team_smem).
 // NV: the recursion of all chains, 0 when they differ; 1: all on the packed recursion.
 // With several recursions in one kernel the FP32 steps spill (seven vectors, moments
 // of L = 40: 866 us, alone 720; packed, one-CTA chain of L = 8: 0.94 us per step, alone 0.45).
@@ -705,9 +740,10 @@ __global__ void __launch_bounds__(kThreads, 1) gfmc_team_engine(const TeamJob* _
         [[maybe_unused]] R2* vec = s_vs ? (R2*)dyn_all : nullptr;
         if constexpr (!COMP && NV != kVec) {
             if (NV == 1 || (sp.nv == 2 && sp.L % 2 == 0)) {
-                // work space: K double2 behind the vector area, which belongs to it when the vectors stand there
-                const int room = s_vs ? vec_bytes / (int)sizeof(double2) + sp.K : sp.K;
-                pk_team_chain<R, kThreads, kTeam>(sp, s_cta, (char*)(s_vs ? dyn_all : work), room, s_vs != 0);
+                // work space: K double2 behind the vector area, which belongs to it when the vectors
+                // stand there (and with packed chains only is large enough for it alone)
+                const int room = s_vs ? vec_bytes / (int)sizeof(double2) + (NV == 1 ? 0 : sp.K) : sp.K;
+                pk_team_chain<R, kThreads, kTeam>(sp, s_cta, (char*)(s_vs ? dyn_all : work), room, s_vs ? vec_bytes : 0);
                 continue;
             }
         }
