@@ -54,8 +54,13 @@ FLOP_PER_SITE_STEP_PROPOSAL = 2 * 52 + 8 * 3 + 8
 #   Gram     7 real diagonals x 3 + 15 pairs among the neighbours x 6
 #            + 6 products <r_m^o|r_m+1^k> x 6                              = 147 flop
 #   sums     49 nonzero real entries                                          = 49 flop
-# i.e. 280 flop per site and step: the work the FP64 engine does on even L.
+# i.e. 280 flop per site and step: the work of the FP64 grid engine on even L.
+# Delta Omega alone needs the four moment sequences of o and v, packed into one
+# vector on even L: 6 complex multiply-adds onto -r_prev, 48 flop, and, over the pair
+# of sites, |r^o|^2, |r^v|^2 and <r_m^o|r_m+1^v>, 16 flop with their sums: 56 per site and
+# step, the work of the FP64 chain's default engine (in fixed point).
 FLOP_PER_SITE_STEP_BIPARTITE = (364 + 147 + 49) / 2
+FLOP_PER_SITE_STEP_PACKED = 48 + 16 / 2
 
 
 # Bytes of one site in one step of the doubling: read r_m and r_{m-1}, write
@@ -75,9 +80,9 @@ def update_work(L: int, M: int, real_bytes: int, nv: int = 7):
 
 
 def update_flop_nonzero(L: int, M: int) -> float:
-    """Flop of one update of the FP64 engine without the terms that vanish by
-    parity (L even; the full count for odd L)."""
-    per = FLOP_PER_SITE_STEP_BIPARTITE if L % 2 == 0 else FLOP_PER_SITE_STEP
+    """Flop of one update of the FP64 chain's default engine: the packed vector
+    (L even), or the two vectors o and v (odd L)."""
+    per = FLOP_PER_SITE_STEP_PACKED if L % 2 == 0 else FLOP_PER_SITE_STEP_PROPOSAL
     return (M // 2 - 1) * L ** 3 * per
 
 
@@ -89,7 +94,7 @@ def update_flop_nonzero(L: int, M: int) -> float:
 # sources is unchanged and the launch has that many updates, and null
 # otherwise.
 TRAFFIC_SOURCES = ("gfmc_engine.cuh", "gfmc_k64.cu", "gfmc_k32.cu", "gfmc_internal.h", "gfmc_vcluster.cuh",
-                   "gfmc_kvc.cu")
+                   "gfmc_kvc.cu", "gfmc_packed.cuh", "gfmc_packed64.cuh", "gfmc_kpk.cu")
 TRAFFIC_HASH = "f1314c5534c2c5a7"
 TRAFFIC_PER_LAUNCH = {"fp64": (16, 6818304 + 2359296), "fp32_mixed": (64, 1485312 + 26880)}
 
@@ -599,9 +604,11 @@ def main():
                      "frac": achieved_tf / peak_tf, "traffic": traffic_per_launch("fp64", U),
                      "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
                      "flop_per_update": flop_nz,
-                     "flop_note": "flop of the update without the terms that vanish by parity on the bipartite "
-                                  "lattice (280 per site and step of the M/2-1 doubling steps at even L; the "
-                                  "count with them, 791, gives flop_full_per_update)",
+                     "flop_note": "flop of the recursion that runs: |o> + |v| as one vector (56 per site and step "
+                                  "of the M/2-1 doubling steps at even L), done in fixed point on the integer "
+                                  "multiplier; peak is the FP64 pipe's, which it replaces.  The seven unit "
+                                  "vectors of the grid engine (280; 791 with the terms that vanish by parity) "
+                                  "give flop_full_per_update and stencil_gbs",
                      "flop_full_per_update": flop_u,
                      "peak_source": "measured in this run: gfmc_measure_fma_peak (own kernel, 16 independent "
                                     "double fma chains per thread, one CTA of 256 on every SM, best of 3, CUDA "
@@ -611,8 +618,8 @@ def main():
                      "peak_derived_source": "152 SMs x max SM clock x 2 FP64 FMA lanes per SM x 2 flop",
                      "flop_s8d_per_update": (M // 2) * L ** 3 * 830,
                      "frac_s8d": U * (M // 2) * L ** 3 * 830 / launch_s / 1e12 / peak_tf,
-                     "s8d_note": "the survey's per-update count (M/2) N 830 counts the products that vanish by "
-                                 "parity, which this engine does not execute; against it the fraction exceeds 1",
+                     "s8d_note": "the per-update count (M/2) N 830 of the seven-vector algorithm, most of which this "
+                                 "engine does not execute; against it the fraction exceeds 1",
                      "fp64_issue": issue},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
         "gpu_launches": args.steps,
