@@ -71,7 +71,8 @@ enum { GFMC_RECURSION_UNIT_VECTORS = 0, GFMC_RECURSION_PROPOSAL = 1 };
  *                    the proposal's vectors o and v, which live on opposite
  *                    parities, as one vector on one thread-block cluster or on
  *                    the whole GPU; FP64 chains hold it in 62-bit fixed point
- *                    (|value| <= 1, 60 fraction bits), and so, in both
+ *                    (|value| <= 1, 60 fraction bits; FP32-mixed chains of
+ *                    L = 4 on one CTA as well), and so, in both
  *                    precisions, do the moments of even L up to 16, read off
  *                    T_n e_k without the doubling.  Else VECTOR_CLUSTERS
  *                    where it applies, else GRID.  The two below run the
