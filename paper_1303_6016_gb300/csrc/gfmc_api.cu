@@ -50,7 +50,8 @@ struct gfmc_ctx {
     double* d_mag = nullptr;
     unsigned long long* d_nacc = nullptr;
     long long* d_nmag = nullptr;
-    // CTAs the per-CTA buffers (flags, phase sums) are sized for
+    // CTAs the per-CTA buffers (flags, phase sums) are sized for, never below those of the
+    // chain's own launches
     int cap_ncta = 0;
     // more sites than threads of the chain's CTAs: single-chain calls run the
     // team variant of the engine (several sites per thread) as a one-job launch
@@ -337,6 +338,8 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
         P.pk_cz = h->mom_cz;
         e = gfmc::launch_packed64_moments(P, h->mom_smem, h->stream);
     } else if (packed) {
+        if (h->pk_ctas > h->cap_ncta)
+            return fail(h, GFMC_ECUDA, "per-CTA buffers for %d CTAs, the engine runs %d", h->cap_ncta, h->pk_ctas);
         P.ncta = h->pk_ctas;
         P.pk_cy = h->pk_cy;
         P.pk_cz = h->pk_cz;
@@ -723,6 +726,8 @@ gfmc_status gfmc_create(int L, const double* spins, double t, double mu, double 
     const size_t vbytes = h->precision == GFMC_PREC_FP64 ? sizeof(double2) : sizeof(float2);
     int *d_ts = nullptr, *d_np = nullptr, *d_ni = nullptr;
     void* rb = nullptr;
+    // the most CTAs of any of the chain's own launches: the grid engine, a vector cluster, the packed engine
+    const int cap = std::max({ncta, 16, h->pk_ctas});
     if ((e = dalloc(h, &P.spins, 2 * (size_t)N)) != cudaSuccess ||
         (e = dalloc(h, &P.hop64, 3 * (size_t)N)) != cudaSuccess ||
         (e = dalloc(h, &P.hop32, 3 * (size_t)N)) != cudaSuccess ||
@@ -733,14 +738,14 @@ gfmc_status gfmc_create(int L, const double* spins, double t, double mu, double 
         (e = dalloc(h, &P.gram, (size_t)P.nsteps * gfmc::kEntries)) != cudaSuccess ||
         (e = dalloc(h, &P.fftin, 4 * (size_t)M)) != cudaSuccess ||
         (e = dalloc(h, &P.gnode, 4 * (size_t)K)) != cudaSuccess ||
-        (e = dalloc(h, &P.qpart, 2 * (size_t)std::max({ncta, 16, h->pk_ctas}))) != cudaSuccess ||
-        (e = dalloc(h, &P.magpart, 3 * (size_t)std::max({ncta, 16, h->pk_ctas}))) != cudaSuccess ||
+        (e = dalloc(h, &P.qpart, 2 * (size_t)cap)) != cudaSuccess ||
+        (e = dalloc(h, &P.magpart, 3 * (size_t)cap)) != cudaSuccess ||
         (h->pk == 2 && (e = dalloc(h, (char**)&P.pk_inbox, h->pk_inbox_bytes)) != cudaSuccess) ||
         (h->vcl && (e = dalloc(h, &P.mom32, 49 * (size_t)M)) != cudaSuccess) ||
         (e = dalloc(h, &P.mom_out, 49 * (size_t)M)) != cudaSuccess ||
         (e = dalloc(h, &d_ts, tstart.size())) != cudaSuccess || (e = dalloc(h, &d_np, nptr.size())) != cudaSuccess ||
         (e = dalloc(h, &d_ni, nidx.size() + 1)) != cudaSuccess ||
-        (e = dalloc(h, &P.flags, (size_t)ncta)) != cudaSuccess || (e = dalloc(h, &P.bar, 2)) != cudaSuccess ||
+        (e = dalloc(h, &P.flags, (size_t)cap)) != cudaSuccess || (e = dalloc(h, &P.bar, 2)) != cudaSuccess ||
         (e = dalloc(h, &P.err, 4)) != cudaSuccess || (e = dalloc(h, &h->d_nacc, 1)) != cudaSuccess ||
         (e = dalloc(h, &h->d_nmag, 1)) != cudaSuccess)
         return bail(cuda_fail(h, e, "allocating chain state"));
@@ -761,7 +766,7 @@ gfmc_status gfmc_create(int L, const double* spins, double t, double mu, double 
         P.prefetch = 1;
     }
     P.rbuf = rb;
-    h->cap_ncta = ncta;
+    h->cap_ncta = cap;
     P.tile_start = d_ts;
     P.nbr_ptr = d_np;
     P.nbr_idx = d_ni;
