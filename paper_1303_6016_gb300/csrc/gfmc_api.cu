@@ -330,9 +330,11 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
     const int nv = P.mode != gfmc::MODE_MOMENTS &&
                            (h->recursion == GFMC_RECURSION_PROPOSAL || (h->auto_engine && h->auto_ctas && !h->vcl))
                        ? 2 : gfmc::kVec;
-    // one CTA or a cluster of the packed engine has no flags to withhold: the stall hook runs the grid engine
-    const bool packed = h->pk != 0 && P.mode != gfmc::MODE_MOMENTS && !(P.stall && h->pk != 2);
-    if (P.mode == gfmc::MODE_MOMENTS && h->mom_ctas != 0 && !P.stall) {
+    // one CTA, and an FP32 cluster (hardware barriers only), wait for nothing that could be withheld:
+    // the stall hook runs the grid engine
+    const bool no_wait = h->pk_ctas == 1 || h->pk_engine == 1;
+    const bool packed = h->pk != 0 && P.mode != gfmc::MODE_MOMENTS && !(P.stall && h->pk != 2 && no_wait);
+    if (P.mode == gfmc::MODE_MOMENTS && h->mom_ctas != 0 && !(P.stall && h->mom_ctas == 1)) {
         P.ncta = h->mom_ctas;
         P.pk_cy = h->mom_cy;
         P.pk_cz = h->mom_cz;
@@ -1321,7 +1323,8 @@ gfmc_status gfmc_run_clusters(gfmc_t* chains, int n_chains, const int64_t* n_upd
         if (err[0] != 0) {
             clear_gram(h, s);
             if (result == GFMC_OK) {
-                result = err[0] == gfmc::ERR_NUMERIC ? GFMC_ENUMERIC : GFMC_ECUDA;
+                result = err[0] == gfmc::ERR_TIMEOUT ? GFMC_ETIMEOUT
+                         : err[0] == gfmc::ERR_NUMERIC ? GFMC_ENUMERIC : GFMC_ECUDA;
                 fail(nullptr, result, "chain %d: device error %d at stage %d", c, err[0], err[1]);
             }
             continue;

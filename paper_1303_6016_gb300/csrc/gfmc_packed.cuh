@@ -854,6 +854,7 @@ struct PkHead {
     double vv0;                  // <v|v>
     double2 ov1;                 // <o|Htilde|v>
     int acc;
+    int stop;                    // a CTA marked the update as failed
 };
 
 // Local sites, proposal and Delta~ by warp 0, one sincos per lane (lane k the
@@ -911,8 +912,8 @@ __device__ __forceinline__ void pk_setup(const Params& p, PkHead& h, int o, unsi
     }
 }
 
-// Delta Omega from the CTAs' phase sums (added in one order by every CTA) and
-// the Metropolis decision, by warp 0; the caller's barrier follows.
+// Delta Omega from the CTAs' phase sums (added in one order by every CTA; an infinite
+// increment marks a failed update) and the Metropolis decision, by warp 0; the caller's barrier follows.
 __device__ __forceinline__ void pk_decide(const Params& p, PkHead& h, int rank, long long q)
 {
     if (threadIdx.x >= 32) return;
@@ -932,6 +933,7 @@ __device__ __forceinline__ void pk_decide(const Params& p, PkHead& h, int rank, 
         int acc = 0;
         if (p.mode == MODE_SWEEP) acc = exp(-p.beta * dom) > h.draw[2];
         h.acc = acc;
+        h.stop = isinf(mx);
         if (rank == 0) {
             const long long slot = (p.mode == MODE_SWEEP) ? q : 0;
             p.domega_out[slot] = dom;

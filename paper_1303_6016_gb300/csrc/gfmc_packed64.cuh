@@ -23,6 +23,7 @@
 namespace gfmc {
 
 constexpr int kPk64Threads = 256;
+constexpr int kNoFail = 1 << 30;
 
 // a site of the tile
 struct __align__(8) PkRec {
@@ -37,8 +38,11 @@ struct __align__(8) PkRec {
 // data: the phase cannot complete before the arrival.  A neighbour sends
 // S_{m+2} only after it received S_{m+1} from this CTA, which was sent after
 // the phase of S_m completed here.
-// A wait that runs out records the error; the CTA then neither waits nor sends
-// but runs the same sequence of barriers as the others to the end of the launch.
+// A wait that runs out records the error.  The thread then neither waits, sends nor
+// arms again -- its next wait on the same barrier would be for a phase after the one that
+// did not complete, and try_wait reports such a phase as passed -- and so does its
+// CTA from the next step = 7 mod 8 on.  The CTA runs the same sequence of barriers as
+// the others to the end of the update, where the cluster leaves the launch together.
 struct PkAsyncEx {
     static constexpr bool kAbort = false;
     const PkTile& t;
@@ -47,6 +51,7 @@ struct PkAsyncEx {
     unsigned bytes, yB, zB;
     int last;  // the last step whose values are sent
     unsigned ph;  // values sent before this update (an even number)
+    unsigned faces;  // the faces that are sent: none from CTA 0 under the stall hook
     bool dead = false;
     __device__ __forceinline__ PkAsyncEx(const PkTile& t_, const Params& p_, unsigned mb_, unsigned ph_)
         : t(t_), p(p_), mb(mb_), ph(ph_)
@@ -57,6 +62,7 @@ struct PkAsyncEx {
         m_zp = cluster_addr(mb, t.cy + ((t.cz + 1) % t.Cz) * t.Cy);
         bytes = t.rowB * (unsigned)((t.Cy > 1 ? 2 * t.PZ : 0) + (t.Cz > 1 ? 2 * t.PY : 0));
         last = p.nsteps;
+        faces = p.stall && bytes && t.rank == 0 ? 0u : 15u;
         yB = t.rowB * (unsigned)t.PY;
         zB = t.rowB * (unsigned)(t.zstr * t.PZ);
     }
@@ -79,7 +85,7 @@ struct PkAsyncEx {
     struct Target {
         unsigned fl, o;
     };
-    __device__ __forceinline__ Target target(const PkRec& r, int c) const { return {r.fl & 15u, 16u * r.at + 8u * (unsigned)c}; }
+    __device__ __forceinline__ Target target(const PkRec& r, int c) const { return {r.fl & faces, 16u * r.at + 8u * (unsigned)c}; }
     static __device__ __forceinline__ void send(unsigned on, unsigned a, int2 v, unsigned m)
     {
         asm volatile(
@@ -138,7 +144,10 @@ struct PkAsyncEx {
     {
         if (!bytes || dead) return true;
         const bool ok = vc_wait(mb + 8u * (unsigned)(m & 1), ((ph + (unsigned)m) >> 1) & 1u, p.budget);
-        if (!ok) set_error(p, ERR_TIMEOUT, 400, m);
+        if (!ok) {
+            set_error(p, ERR_TIMEOUT, 400, m);
+            dead = true;
+        }
         return ok;
     }
     // ok: this thread's wait for S_m ended, so the phase is complete and takes the next arrival
@@ -181,7 +190,7 @@ template <int NP, int NF> struct PkGridEx {
     unsigned half;             // words of a phase's half of an inbox (4 faces)
     unsigned ring, ph;         // ph: first phase of the update
     int L, last;
-    bool mute, dead = false;
+    bool mute;
     unsigned nb[4];            // word offsets of the neighbours' faces this CTA writes
     unsigned src[NP], dst[NP]; // word offset from inbox in phase 0's half, and ring byte offset; src ~0u: none
     __device__ __forceinline__ PkGridEx(const PkTile& t, const Params& p_, unsigned, unsigned ph_) : p(p_), ph(ph_)
@@ -387,12 +396,14 @@ __device__ __forceinline__ void pk64_xy(unsigned bonds, const PkTile& t, const P
 // KI = 0: whole sites s, s + 256, ... with bonds and S_{m-1} from shared memory.
 // Not inlined: with the tail in one function the registers that live across it
 // went to local memory inside the step loop.
+// s_fail: the first step whose wait ran out (before it, kNoFail).  False (in every
+// thread): a wait of the CTA ran out.
 // MOM: no sums; instead the values at the local sites of a moments call, limbs as they
 // are, go to head.mom (pk64_moments), S_m to place m of the sites' rows.
 template <class Ex, int SPL, int KI, bool MOM = false>
 __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, const PkRec* tab, const PkHead& head,
                                           PkSums<double, kPk64Threads / 32>& sums, unsigned mb, unsigned ph,
-                                          volatile int* s_fail)
+                                          int* s_fail)
 {
     static_assert(!MOM || KI == 1, "one site per thread");
     static_assert(KI == 1 || SPL == 1, "one part of a site per thread");
@@ -481,13 +492,14 @@ __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, c
     for (int m = 0; m <= nsteps; ++m) {
         const unsigned b0 = (m & 1) ? t.bufB : 0u, b1 = (m & 1) ? 0u : t.bufB;
         const bool ok = ex.receive(m, b0);
-        if (!ok) *s_fail = 1;
+        if (!ok) atomicMin(s_fail, m);
         __syncthreads();
         ex.received(m, ok);
-        // a wait that ran out: every thread of the CTA sees it after a barrier, a few steps on
-        if ((m & 7) == 7 && *s_fail) {
-            if (Ex::kAbort) return false;
-            ex.dead = true;
+        // a wait that ran out by step m: the same answer in every thread, as one that runs out
+        // in a later step (of a thread ahead of this one) records that step
+        if ((m & 7) == 7 && *(volatile int*)s_fail <= m) {
+            if constexpr (Ex::kAbort) return false;
+            else ex.dead = true;
         }
         const bool oddA = odd_o ^ ((m & 1) != 0);  // the parity that holds r_m^o
         Pk64Sums acc;
@@ -608,7 +620,7 @@ __device__ __noinline__ bool pk64_advance(const Params& p, const PkTile& tile, c
     }
     __syncthreads();
     if (!MOM) pk_flush_rest<double, NW>(p, sums, nsteps, warp, lane);
-    return true;
+    return *(volatile int*)s_fail > nsteps;
 }
 
 // ---------------------------------------------------------------------------
@@ -639,7 +651,8 @@ template <bool GRID> __device__ __forceinline__ void pk64_run_chain(const Params
     if constexpr (!GRID) {
         if (tid == 0) PkAsyncEx(t, p, smem_u32(s_mb), 0).init();
     }
-    if (tid == 0) s_fail = 0;
+    if (tid == 0) s_fail = kNoFail;
+    bool ok = true;  // no wait of the CTA has run out
     auto sync = [&](int where) -> bool {
         if constexpr (GRID) {
             return grid_barrier(p, where);
@@ -664,7 +677,6 @@ template <bool GRID> __device__ __forceinline__ void pk64_run_chain(const Params
         if (reload) pk_load_bonds<double, kPk64Threads>(p, t);
         reload = false;
         __syncthreads();
-        bool ok;
         const unsigned mb = smem_u32(s_mb), ph = (unsigned)(q * (long long)(p.nsteps + 1));
         constexpr int NT = kPk64Threads;
         const int faces = GRID ? 2 * (t.PY + t.PZ) * t.L : 0;
@@ -675,18 +687,21 @@ template <bool GRID> __device__ __forceinline__ void pk64_run_chain(const Params
         else if (T <= 2 * NT && faces <= 3 * NT && wide) ok = pk64_advance<Ex3, 1, 2>(p, t, tab, head, sums, mb, ph, &s_fail);
         else if (T <= 3 * NT && faces <= 3 * NT && wide) ok = pk64_advance<Ex3, 1, 3>(p, t, tab, head, sums, mb, ph, &s_fail);
         else ok = pk64_advance<ExN, 1, 0>(p, t, tab, head, sums, mb, ph, &s_fail);
-        if (!ok) return;
+        if (GRID && !ok) return;
         if (!sync(1)) return;
         pk_tail_fft<kPk64Threads>(p, rank, C, work, work_n, head.vv0, head.ov1);
         if (!sync(2)) return;
         pk_tail_clear<kPk64Threads>(p, rank, C);
         pk_tail_phase<kPk64Threads>(p, rank, C, (double*)work);
-        // after a wait that ran out on a cluster no CTA accepts the move
-        if (!GRID && s_fail && tid == 0) p.qpart[2 * rank] = CUDART_NAN;
+        // after a wait that ran out on a cluster no CTA accepts the move, and all leave
+        if (!GRID && !ok && tid == 0) {
+            p.qpart[2 * rank] = CUDART_NAN;
+            p.qpart[2 * rank + 1] = CUDART_INF;
+        }
         if (!sync(3)) return;
         pk_decide(p, head, rank, q);
         __syncthreads();
-        if (p.mode == MODE_DELTA) break;
+        if (p.mode == MODE_DELTA || (!GRID && head.stop)) break;
         if (head.acc) {
             ++nacc;
             // only the bonds of o change: pencils that do not hold or border its row keep theirs
@@ -706,7 +721,7 @@ template <bool GRID> __device__ __forceinline__ void pk64_run_chain(const Params
         *p.n_mag = nmag;
     }
     if constexpr (!GRID) {
-        if (s_fail) {  // values still in flight land before any CTA leaves
+        if (!ok) {  // values still in flight land before any CTA leaves
             const long long t0 = clock64();
             while (clock64() - t0 < (1ll << 21)) __nanosleep(256);
         }
@@ -737,7 +752,7 @@ __global__ void __launch_bounds__(kPk64Threads, 1) gfmc_packed64_moments(const P
         p = q;
         p.nsteps = M - 2;  // S_{M-1} is the last vector
         t = pk_tile<double>(p, rank, (char*)dyn_all);
-        s_fail = 0;
+        s_fail = kNoFail;
         const int o = (int)p.site;
         for (int j = 0; j < kVec; ++j) {
             head.mom[j] = j == 0 ? o : nbr_site(o, j - 1, p.L);
@@ -768,10 +783,11 @@ __global__ void __launch_bounds__(kPk64Threads, 1) gfmc_packed64_moments(const P
     const int T = t.L * t.PY * t.PZ;
     const unsigned mb = smem_u32(s_mb);
     constexpr int NT = kPk64Threads;
-    if (4 * T <= NT) pk64_advance<PkAsyncEx, 4, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
-    else if (2 * T <= NT) pk64_advance<PkAsyncEx, 2, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
-    else pk64_advance<PkAsyncEx, 1, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
-    if (s_fail) {  // values still in flight land before any CTA leaves
+    bool ok;
+    if (4 * T <= NT) ok = pk64_advance<PkAsyncEx, 4, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
+    else if (2 * T <= NT) ok = pk64_advance<PkAsyncEx, 2, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
+    else ok = pk64_advance<PkAsyncEx, 1, 1, true>(p, t, tab, head, sums, mb, 0, &s_fail);
+    if (!ok) {  // values still in flight land before any CTA leaves
         const long long t0 = clock64();
         while (clock64() - t0 < (1ll << 21)) __nanosleep(256);
     }

@@ -1,5 +1,7 @@
 """The packed engines beside the other calls of a chain, and where they end: a chain
-in a batch and then alone."""
+in a batch and then alone, waits that run out on a cluster."""
+import time
+
 import numpy as np
 import pytest
 
@@ -30,3 +32,39 @@ def test_chain_alone_after_a_team_smaller_than_its_engine(G, L, team, wide):
         ra, rb = a.updates(n), b.updates(n)
         assert np.array_equal(ra["d_omega"], rb["d_omega"])
         assert np.array_equal(ra["decisions"], rb["decisions"])
+
+
+def _times_out(G, ch, call):
+    """A stalled call ends with GFMC_ETIMEOUT in little more than one budget of 10 ms."""
+    ch.set_wait_budget(20_000_000)
+    ch.inject_stall(True)
+    t = time.perf_counter()
+    with pytest.raises(G.GfmcError) as e:
+        call()
+    assert e.value.status == G.GFMC_ETIMEOUT
+    assert time.perf_counter() - t < 1.0
+    ch.set_wait_budget(4_000_000_000)
+
+
+@pytest.mark.parametrize("L,M,n", [(8, 16, 300), (12, 64, 300), (16, 64, 300)])
+def test_cluster_wait_runs_out(G, L, M, n):
+    """An FP64 chain on one cluster (a quarter, half a site and a site per thread) whose CTA 0
+    sends no face values: the waits of the others run out once and the launch ends,
+    however many updates are left, and the chain runs on as if nothing had happened."""
+    sp = inputs.uniform_sphere(L, 1)
+    with G.Chain(L, sp, M=M, seed=3) as a, G.Chain(L, sp, M=M, seed=3) as b:
+        _times_out(G, a, lambda: a.updates(n))
+        assert a.counter == 0
+        assert np.array_equal(a.updates(20)["d_omega"], b.updates(20)["d_omega"])
+        _times_out(G, a, lambda: a.delta_omega(5, 1.0, 2.0))
+        assert a.delta_omega(5, 1.0, 2.0) == b.delta_omega(5, 1.0, 2.0)
+
+
+@pytest.mark.parametrize("L,M", [(4, 16), (8, 64), (16, 64)])
+def test_moments_wait_runs_out(G, L, M):
+    """The same on the six clusters of a moments call."""
+    sp = inputs.uniform_sphere(L, 1)
+    with G.Chain(L, sp, M=M) as ch:
+        ref = ch.moments(7)
+        _times_out(G, ch, lambda: ch.moments(7))
+        assert np.array_equal(ch.moments(7), ref)
