@@ -265,19 +265,18 @@ int common_nv(gfmc_ctx* const* chains, int n)
     return packed ? 1 : team_nv(chains[0]);
 }
 
-// Dynamic shared memory of a launch of teams: the vector area of the chains that
-// keep their vectors there and the work area of the largest chain (none where every
-// chain is packed and resident: its work area is then the vectors').  What is left
-// holds bonds of the packed chains of more sites than registers take.
+// Dynamic shared memory of a launch of teams and where each chain's vectors stand
+// (team_smem_bytes).  What is left holds bonds of the packed chains of more sites
+// than registers take.
 struct TeamSmem {
-    std::vector<int> resident;
-    int vec_bytes = 0, smem = 0, nv = 0;
+    std::vector<int> at;  // vec_smem of each chain's job
+    int smem = 0, nv = 0;
 };
 gfmc_status plan_team_smem(gfmc_ctx* const* chains, int n, const int* ctas, TeamSmem* out)
 {
     const bool comp = chains[0]->P.comp != 0;
     const int prec = chains[0]->precision;
-    const int vsz = prec == GFMC_PREC_FP64 ? (int)sizeof(double2) : (int)sizeof(float2);
+    const size_t vsz = prec == GFMC_PREC_FP64 ? sizeof(double2) : sizeof(float2);
     cudaError_t e;
     int dev_smem = 0, stat = 0;
     // the FP64 and the compensated kernel hold every recursion
@@ -285,32 +284,18 @@ gfmc_status plan_team_smem(gfmc_ctx* const* chains, int n, const int* ctas, Team
     if ((e = cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, chains[0]->device)) != cudaSuccess ||
         (e = gfmc::team_static_smem(prec, comp, out->nv, &stat)) != cudaSuccess)
         return cuda_fail(nullptr, e, "querying shared memory");
-    int K = 0, work = 0;
-    for (int c = 0; c < n; ++c) K = std::max(K, chains[c]->K);
-    work = out->nv == 1 ? K * (int)sizeof(double2) : gfmc::engine_smem_bytes(K);
-    size_t vec = 0, want = 0;
-    bool all = true;
-    out->resident.assign(n, 0);
+    std::vector<gfmc::TeamChainSmem> need(n);
     for (int c = 0; c < n; ++c) {
         const gfmc_ctx* h = chains[c];
         const int tc = std::max(ctas ? ctas[c] : 1, 1);
-        const size_t vb = team_vec_bytes(h, tc);
-        if (vb == SIZE_MAX || vb + work + stat > (size_t)dev_smem) {
-            all = false;
-            continue;
-        }
-        out->resident[c] = 1;
-        vec = std::max(vec, vb);
-        if (team_packed(h)) want = std::max(want, vb + 3 * (size_t)vsz * ((h->N + tc - 1) / tc) + (size_t)vsz * h->L * h->L);
+        gfmc::TeamChainSmem& q = need[c];
+        q.packed = team_packed(h);
+        q.vec = team_vec_bytes(h, tc);
+        q.work = q.packed ? h->K * sizeof(double2) : (size_t)gfmc::engine_smem_bytes(h->K);
+        q.want = q.vec == SIZE_MAX ? 0 : q.vec + 3 * vsz * ((h->N + tc - 1) / tc) + vsz * h->L * h->L;
     }
-    if (out->nv == 1 && vec > 0) {
-        vec = std::max(vec, (size_t)work);
-        if (all) work = 0;
-    }
-    if (vec > 0) vec = std::max(vec, std::min(want, (size_t)(dev_smem - stat - work)));
-    out->vec_bytes = (int)((vec + 15) & ~(size_t)15);
-    if (out->vec_bytes + work + stat > dev_smem) out->vec_bytes -= 16;
-    out->smem = out->vec_bytes + work;
+    out->smem = gfmc::team_smem_bytes(need.data(), n, (size_t)(dev_smem - stat));
+    for (const auto& q : need) out->at.push_back(q.at);
     return GFMC_OK;
 }
 
@@ -364,8 +349,8 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
         if ((e = cudaMemcpyAsync(h->d_job, &job, sizeof(job), cudaMemcpyHostToDevice, h->stream)) != cudaSuccess)
             return cuda_fail(h, e, "uploading the job");
         const int smem = gfmc::engine_smem_bytes(P.K);
-        e = h->precision == GFMC_PREC_FP64 ? gfmc::launch_team_f64(h->d_job, 1, P.ncta, 0, smem, h->stream)
-                                            : gfmc::launch_team_f32(h->d_job, 1, P.ncta, 0, smem, h->stream, P.comp != 0,
+        e = h->precision == GFMC_PREC_FP64 ? gfmc::launch_team_f64(h->d_job, 1, P.ncta, smem, h->stream)
+                                            : gfmc::launch_team_f32(h->d_job, 1, P.ncta, smem, h->stream, P.comp != 0,
                                                                     (P.nv == 2 && h->L % 2 == 0 && !P.comp) ? 1 : P.nv);
     } else {
         if (h->vcl && nv == gfmc::kVec)
@@ -981,8 +966,7 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
     if ((e = cudaSetDevice(dev)) != cudaSuccess) return cuda_fail(nullptr, e, "cudaSetDevice");
     TeamSmem tm;
     if (const gfmc_status st = plan_team_smem(chains, n_chains, team_ctas, &tm); st != GFMC_OK) return st;
-    const int smem = tm.smem, vec_bytes = tm.vec_bytes;
-    const std::vector<int>& resident = tm.resident;
+    const int smem = tm.smem;
     int grid = 0;
     for (int c = 0; c < n_chains; ++c) grid += team_ctas ? team_ctas[c] : 1;
     int maxc = 0;
@@ -1025,7 +1009,7 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
             cta0 += tc;
         }
         jobs[c].cta0 = last0;
-        jobs[c].vec_smem = resident[c];
+        jobs[c].vec_smem = tm.at[c];
         if ((e = cudaMemsetAsync(P.flags, 0, sizeof(unsigned) * tc, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(P.bar, 0, sizeof(unsigned) * 2, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(P.err, 0, sizeof(int) * 4, s)) != cudaSuccess ||
@@ -1043,9 +1027,8 @@ gfmc_status gfmc_run_batch(gfmc_t* chains, int n_chains, const int64_t* n_update
     if ((e = cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(gfmc::TeamJob) * n_chains, cudaMemcpyHostToDevice, s)) !=
         cudaSuccess)
         return cuda_fail(nullptr, e, "uploading the job table");
-    e = prec == GFMC_PREC_FP64 ? gfmc::launch_team_f64(d_jobs, n_chains, grid, (int)vec_bytes, smem, s)
-                               : gfmc::launch_team_f32(d_jobs, n_chains, grid, (int)vec_bytes, smem, s,
-                                                       chains[0]->P.comp != 0, tm.nv);
+    e = prec == GFMC_PREC_FP64 ? gfmc::launch_team_f64(d_jobs, n_chains, grid, smem, s)
+                               : gfmc::launch_team_f32(d_jobs, n_chains, grid, smem, s, chains[0]->P.comp != 0, tm.nv);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "launching the batch");
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(nullptr, e, "batch execution");
     gfmc_status result = GFMC_OK;
@@ -1485,7 +1468,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
         P.stall = 0;
         return P;
     };
-    int team_grid = 0, team_smem = 0, team_vec = 0;
+    int team_grid = 0, team_smem = 0;
     TeamSmem tplan;
     if (clusters) {
         int static_smem[2] = {0, 0};
@@ -1547,8 +1530,6 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
         }
     } else {
         if (const gfmc_status st = plan_team_smem(chains, n_chains, ctas, &tplan); st != GFMC_OK) return bail(st);
-        const std::vector<int>& resident = tplan.resident;
-        team_vec = tplan.vec_bytes;
         team_smem = tplan.smem;
         for (int c = 0; c < n_chains; ++c) team_grid += ctas[c];
         int maxc = 0;
@@ -1577,7 +1558,7 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
                 cta0 += tc;
             }
             j.cta0 = last0;
-            j.vec_smem = resident[c];
+            j.vec_smem = tplan.at[c];
             jobs.push_back(j);
             p->chains.push_back(h);
             p->caller.push_back(c);
@@ -1617,8 +1598,8 @@ gfmc_status gfmc_plan_create(gfmc_t* chains, int n_chains, const int64_t* n_upda
     gfmc::plan_prepare_kernel<<<nj, 128, 0, cs>>>(p->d_jobs, nj, p->d_counters, p->d_nupd);
     ce = cudaGetLastError();
     if (ce == cudaSuccess && !clusters) {
-        ce = prec == GFMC_PREC_FP64 ? gfmc::launch_team_ex_f64(p->d_jobs, nj, team_grid, team_vec, team_smem, cs)
-                                    : gfmc::launch_team_ex_f32(p->d_jobs, nj, team_grid, team_vec, team_smem, cs,
+        ce = prec == GFMC_PREC_FP64 ? gfmc::launch_team_ex_f64(p->d_jobs, nj, team_grid, team_smem, cs)
+                                    : gfmc::launch_team_ex_f32(p->d_jobs, nj, team_grid, team_smem, cs,
                                                                chains[0]->P.comp != 0, tplan.nv);
     } else if (ce == cudaSuccess) {
         cudaEvent_t fork = nullptr;

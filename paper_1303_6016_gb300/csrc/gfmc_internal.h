@@ -221,9 +221,37 @@ __host__ __device__ inline int one_cta_parts(int N) { return 2 * N <= 128 ? 2 : 
 struct TeamJob {
     Params p;
     int cta0;
-    int vec_smem;  // the chain's recursion vectors live in the CTA's shared memory
+    int vec_smem;  // bytes of the chain's recursion vectors in the CTA's shared memory, 0: in global memory
     int pad[2];
 };
+
+// Shared memory of a launch of teams.  Every CTA runs one chain at a time, which has
+// all of it: its vectors first, if they stand there, and the tail's work area behind
+// them -- on the packed recursion in their place.  So the launch takes the largest
+// need of any chain, and whether a chain's vectors stand there follows from its own
+// sizes and the room (the device's limit less the kernel's static part) alone.
+struct TeamChainSmem {
+    size_t vec;   // bytes of the vectors; SIZE_MAX: they stay in global memory
+    size_t work;  // bytes of the work area
+    size_t want;  // packed: bytes that more of the chain's data could use
+    bool packed;
+    int at;       // out: vec_smem of the chain's job
+};
+inline int team_smem_bytes(TeamChainSmem* c, int n, size_t room)
+{
+    size_t total = 0, want = 0;
+    for (int k = 0; k < n; ++k) {
+        const size_t vec = c[k].vec == SIZE_MAX ? 0 : (c[k].vec + 15) & ~(size_t)15;
+        const size_t need = c[k].packed ? (vec > c[k].work ? vec : c[k].work) : vec + c[k].work;
+        const bool resident = vec > 0 && need <= room;
+        c[k].at = resident ? (int)vec : 0;
+        const size_t use = resident ? need : c[k].work;
+        total = total > use ? total : use;
+        if (resident && c[k].packed && c[k].want > want) want = c[k].want;
+    }
+    want = (want < room ? want : room) & ~(size_t)15;
+    return (int)(total > want ? total : want);
+}
 
 // Mailbox of one slot of the serving loop (device memory).  The host writes
 // [prec, cta0, job] and then seq; the slot's CTA 0 relays seq through cmd.
@@ -250,18 +278,16 @@ cudaError_t launch_engine_f32(const Params& p, cudaStream_t s);
 // nv = 7: recursion on the 7 unit vectors; nv = 2: on the proposal's vectors o and v
 cudaError_t launch_engine_f64(const Params& p, int nv, cudaStream_t s);
 cudaError_t launch_engine_f32(const Params& p, int nv, cudaStream_t s);
-cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s);
+cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s);
 // nv: the vectors of every job's recursion (p.nv), 0 when they differ; 1: even lattices on two vectors only
-cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
-                            bool comp, int nv);
+cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s, bool comp, int nv);
 // co-resident CTAs of the kernel launch_team_* takes for comp and nv, and its static shared memory
 // (bytes); nv < 0: the fewest of any
 cudaError_t team_max_ctas(int precision, int smem, bool comp, int nv, int* out);
 cudaError_t team_static_smem(int precision, bool comp, int nv, int* out);
 // launch_team_* through cudaLaunchKernelEx with the cooperative attribute (capturable in a CUDA graph)
-cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s);
-cudaError_t launch_team_ex_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
-                               bool comp, int nv);
+cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s);
+cudaError_t launch_team_ex_f32(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s, bool comp, int nv);
 cudaError_t launch_server(const ServerArgs& a, int grid, int smem, cudaStream_t s);
 // one cluster of C CTAs per job (recursion on the proposal's vectors)
 cudaError_t launch_cluster_f64(const TeamJob* d_jobs, int njobs, int C, int vec_bytes, int smem, cudaStream_t s);

@@ -50,13 +50,13 @@ cudaError_t engine_max_ctas_f32(int K, int* out)
 }
 
 template <int NV, bool COMP>
-static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
+static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s,
                                bool ex)
 {
     cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<float, NV, COMP>);
     if (e != cudaSuccess) return e;
     if (!ex) {
-        void* args[] = {(void*)&d_jobs, (void*)&njobs, (void*)&vec_bytes};
+        void* args[] = {(void*)&d_jobs, (void*)&njobs, (void*)&smem};
         return cudaLaunchCooperativeKernel((void*)gfmc_team_engine<float, NV, COMP>, dim3(grid), dim3(kThreads), args,
                                            (size_t)smem, s);
     }
@@ -72,29 +72,29 @@ static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int v
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<float, NV, COMP>, d_jobs, njobs, vec_bytes);
+    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<float, NV, COMP>, d_jobs, njobs, smem);
 }
 
-static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
+static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s,
                                bool comp, int nv, bool ex)
 {
-    if (comp) return team_launch<0, true>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
-    if (nv == 1) return team_launch<1, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
-    if (nv == 2) return team_launch<2, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
-    if (nv == kVec) return team_launch<kVec, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
-    return team_launch<0, false>(d_jobs, njobs, grid, vec_bytes, smem, s, ex);
+    if (comp) return team_launch<0, true>(d_jobs, njobs, grid, smem, s, ex);
+    if (nv == 1) return team_launch<1, false>(d_jobs, njobs, grid, smem, s, ex);
+    if (nv == 2) return team_launch<2, false>(d_jobs, njobs, grid, smem, s, ex);
+    if (nv == kVec) return team_launch<kVec, false>(d_jobs, njobs, grid, smem, s, ex);
+    return team_launch<0, false>(d_jobs, njobs, grid, smem, s, ex);
 }
 
-cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
+cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s,
                             bool comp, int nv)
 {
-    return team_launch(d_jobs, njobs, grid, vec_bytes, smem, s, comp, nv, false);
+    return team_launch(d_jobs, njobs, grid, smem, s, comp, nv, false);
 }
 
-cudaError_t launch_team_ex_f32(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s,
+cudaError_t launch_team_ex_f32(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s,
                                bool comp, int nv)
 {
-    return team_launch(d_jobs, njobs, grid, vec_bytes, smem, s, comp, nv, true);
+    return team_launch(d_jobs, njobs, grid, smem, s, comp, nv, true);
 }
 
 template <int NV, bool COMP>

@@ -54,17 +54,17 @@ cudaError_t engine_max_ctas_f64(int K, int* out)
 
 namespace gfmc {
 
-cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s)
+cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s)
 {
     cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double, 0>);
     if (e != cudaSuccess) return e;
-    void* args[] = {(void*)&d_jobs, (void*)&njobs, (void*)&vec_bytes};
+    void* args[] = {(void*)&d_jobs, (void*)&njobs, (void*)&smem};
     return cudaLaunchCooperativeKernel((void*)gfmc_team_engine<double, 0>, dim3(grid), dim3(kThreads), args, (size_t)smem, s);
 }
 
 // The same launch through cudaLaunchKernelEx with the cooperative attribute,
 // the form a CUDA graph captures as a cooperative kernel node.
-cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int vec_bytes, int smem, cudaStream_t s)
+cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s)
 {
     cudaError_t e = allow_dynamic_smem((const void*)gfmc_team_engine<double, 0>);
     if (e != cudaSuccess) return e;
@@ -78,7 +78,7 @@ cudaError_t launch_team_ex_f64(const TeamJob* d_jobs, int njobs, int grid, int v
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<double, 0>, d_jobs, njobs, vec_bytes);
+    return cudaLaunchKernelEx(&cfg, gfmc_team_engine<double, 0>, d_jobs, njobs, smem);
 }
 
 cudaError_t team_static_smem_f64(int* out)

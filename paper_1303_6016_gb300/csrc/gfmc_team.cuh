@@ -694,13 +694,12 @@ __global__ void __launch_bounds__(NT, 1) gfmc_one_cta(const Params p, int work_n
 }
 
 // A batch of chains, each on its own team of CTAs (jobs sorted by cta0).
-// The dynamic shared memory holds [vector area of vec_bytes][work area] (plan_team_smem).
+// smem: bytes of dynamic shared memory, shared out chain by chain (team_smem_bytes).
 // NV: the recursion of all chains, 0 when they differ; 1: all on the packed recursion.
 // With several recursions in one kernel the FP32 steps spill (seven vectors, moments
 // of L = 40: 866 us, alone 720; packed, one-CTA chain of L = 8: 0.94 us per step, alone 0.45).
 template <class R, int NV, bool COMP = false>
-__global__ void __launch_bounds__(kThreads, 1) gfmc_team_engine(const TeamJob* __restrict__ jobs, int njobs,
-                                                                 int vec_bytes)
+__global__ void __launch_bounds__(kThreads, 1) gfmc_team_engine(const TeamJob* __restrict__ jobs, int njobs, int smem)
 {
     extern __shared__ double2 dyn_all[];
     __shared__ Params sp;
@@ -736,14 +735,11 @@ __global__ void __launch_bounds__(kThreads, 1) gfmc_team_engine(const TeamJob* _
     };
     do {
         load();
-        double2* work = dyn_all + vec_bytes / (int)sizeof(double2);
+        [[maybe_unused]] double2* work = dyn_all + s_vs / (int)sizeof(double2);
         [[maybe_unused]] R2* vec = s_vs ? (R2*)dyn_all : nullptr;
         if constexpr (!COMP && NV != kVec) {
             if (NV == 1 || (sp.nv == 2 && sp.L % 2 == 0)) {
-                // work space: K double2 behind the vector area, which belongs to it when the vectors
-                // stand there (and with packed chains only is large enough for it alone)
-                const int room = s_vs ? vec_bytes / (int)sizeof(double2) + (NV == 1 ? 0 : sp.K) : sp.K;
-                pk_team_chain<R, kThreads, kTeam>(sp, s_cta, (char*)(s_vs ? dyn_all : work), room, s_vs ? vec_bytes : 0);
+                pk_team_chain<R, kThreads, kTeam>(sp, s_cta, (char*)dyn_all, smem / (int)sizeof(double2), s_vs ? smem : 0);
                 continue;
             }
         }

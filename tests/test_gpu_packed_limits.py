@@ -1,5 +1,6 @@
 """The packed engines beside the other calls of a chain, and where they end: a chain
-in a batch and then alone, waits that run out on a cluster."""
+in a batch and then alone, waits that run out on a cluster,
+teams on as many nodes as the tail takes."""
 import time
 
 import numpy as np
@@ -68,3 +69,34 @@ def test_moments_wait_runs_out(G, L, M):
         ref = ch.moments(7)
         _times_out(G, ch, lambda: ch.moments(7))
         assert np.array_equal(ch.moments(7), ref)
+
+
+@pytest.mark.parametrize("small,large", [((8, 1), (24, 1)), ((6, 1), (8, 20))])
+def test_team_batch_on_8192_nodes(G, small, large):
+    """FP32 chains of M = 4096 on 2M nodes, whose tail alone takes 128 KB of a CTA's
+    shared memory: one with its vectors there beside one whose vectors stay in global
+    memory (a lattice too large, a tile below a plane) in one batch and in one plan, each
+    as in a batch of its own."""
+    specs = [small, large]
+    sps = [inputs.uniform_sphere(L, 5 + c) for c, (L, _) in enumerate(specs)]
+
+    def chains():
+        return [G.Chain(L, sps[c], M=4096, nodes=8192, seed=2, chain_id=c, precision="fp32_mixed")
+                for c, (L, _) in enumerate(specs)]
+
+    ref = []
+    for c, ch in enumerate(chains()):
+        ref.append(G.run_batch([ch], 2, team_ctas=[specs[c][1]])[0]["d_omega"])
+        ch.close()
+    both = chains()
+    for r, out in zip(ref, G.run_batch(both, 2, team_ctas=[tc for _, tc in specs])):
+        assert np.array_equal(out["d_omega"], r)
+    for ch in both:
+        ch.close()
+    both = chains()
+    with G.Plan(both, 2, [tc for _, tc in specs], schedule="teams") as plan:
+        plan.launch(1)
+        for r, out in zip(ref, plan.sync()):
+            assert np.array_equal(out["d_omega"], r)
+    for ch in both:
+        ch.close()
