@@ -419,7 +419,7 @@ template <class R> __device__ __forceinline__ const typename Cx<R>::T* hop_table
 // within a plane of the tile's ends go first and are published before the
 // others are computed, so the neighbours' wait overlaps the rest of the step.
 // Without WIN (tiles below a plane, or too large for shared memory) all values
-// are read from global memory.
+// are read from global memory, in the same order.
 template <class R, bool WIN, bool WIDE>
 __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigned phase, unsigned buf, int bytes,
                                                const PkHead& head, StepSums<R>& sums)
@@ -474,8 +474,9 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
     if constexpr (WIN) __syncthreads();
     else publish(p, cta, phase + 1);
 
-    // sites of the tile within a plane of its ends: [0, e0) and [e1, T)
-    const int e0 = (WIN && p.ncta > 1 && T > 2 * LL) ? LL : T, e1 = e0 < T ? T - LL : T;
+    // sites of the tile within a plane of its ends: [0, e0) and [e1, T).  Wherever the vectors
+    // stand (which the launch's other chains have a say in): the order of the sums follows it
+    const int e0 = (p.ncta > 1 && T > 2 * LL) ? LL : T, e1 = e0 < T ? T - LL : T;
     const int halo = whole ? N - T : 2 * LL;
     for (int m = 1; m <= p.nsteps; ++m) {
         const unsigned rd = (m & 1) ? b1 : b0, wr = (m & 1) ? b0 : b1;

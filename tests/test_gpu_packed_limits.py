@@ -1,6 +1,6 @@
 """The packed engines beside the other calls of a chain, and where they end: a chain
 in a batch and then alone, waits that run out on a cluster,
-teams on as many nodes as the tail takes."""
+teams on as many nodes as the tail takes, teams beside other chains."""
 import time
 
 import numpy as np
@@ -100,3 +100,22 @@ def test_team_batch_on_8192_nodes(G, small, large):
             assert np.array_equal(out["d_omega"], r)
     for ch in both:
         ch.close()
+
+
+@pytest.mark.parametrize("precision,L,team,other", [
+    ("fp32_mixed", 32, 3, dict(L=5)), ("fp32_mixed", 32, 3, dict(L=6, engine="grid")),
+    ("fp32_mixed", 32, 4, dict(L=6, engine="grid")), ("fp32_mixed", 12, 1, dict(L=4, M=4096, nodes=8192)),
+    ("fp32_mixed", 10, 1, dict(L=6, engine="grid", M=4096, nodes=8192)), ("fp64", 24, 8, dict(L=4, M=4096, nodes=8192)),
+    ("fp64", 8, 1, dict(L=5, M=4096, nodes=8192))])
+def test_team_results_do_not_depend_on_the_other_chains(G, precision, L, team, other):
+    """A chain on a team whose vectors fit in shared memory beside some chains and not
+    beside others (another kernel's static share, the tail of another chain): the same
+    bits in both launches."""
+    kw = dict(M=64, beta=12.0, mu=-2.0, seed=5, precision=precision)
+    sp = inputs.uniform_sphere(L, 3)
+    okw = {**kw, **{k: v for k, v in other.items() if k != "L"}}
+    with G.Chain(L, sp, **kw) as a, G.Chain(L, sp, **kw) as b, \
+            G.Chain(other["L"], inputs.uniform_sphere(other["L"], 4), **okw) as o:
+        ra = G.run_batch([a], 3, team_ctas=[team])[0]
+        rb = G.run_batch([b, o], 3, team_ctas=[team, 1])[0]
+        assert np.array_equal(ra["d_omega"], rb["d_omega"])
