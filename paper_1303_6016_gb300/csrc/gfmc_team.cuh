@@ -477,6 +477,7 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
     // sites of the tile within a plane of its ends: [0, e0) and [e1, T).  Wherever the vectors
     // stand (which the launch's other chains have a say in): the order of the sums follows it
     const int e0 = (p.ncta > 1 && T > 2 * LL) ? LL : T, e1 = e0 < T ? T - LL : T;
+    const int parts = e0 < e1 ? 2 : 1;
     const int halo = whole ? N - T : 2 * LL;
     for (int m = 1; m <= p.nsteps; ++m) {
         const unsigned rd = (m & 1) ? b1 : b0, wr = (m & 1) ? b0 : b1;
@@ -575,10 +576,19 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
                 }
             }
         };
-        // the tile's ends, read by the other CTAs, then the sites between
-        sites(e0 + T - e1, e0, e1, p.ncta > 1);
-        publish(p, cta, phase + (unsigned)m + 1u);
-        if (e0 < e1) sites(e1 - e0, 0, e0, false);
+        // the tile's ends, read by the other CTAs, then the sites between.  FP32: one loop;
+        // with its body twice in the function, one_cta_steps of the same kernel spilled in its steps
+        auto part = [&](bool ends) {
+            sites(ends ? e0 + T - e1 : e1 - e0, ends ? e0 : 0, ends ? e1 : e0, ends && p.ncta > 1);
+            if (ends) publish(p, cta, phase + (unsigned)m + 1u);
+        };
+        if constexpr (sizeof(R) == 4) {
+#pragma unroll 1
+            for (int k = 0; k < parts; ++k) part(k == 0);
+        } else {
+            part(true);
+            if (parts > 1) part(false);
+        }
         const R s = warp_reduce_scatter4(acc, lane);
         if ((lane & 7) == 0) sums.w[m & (kPkGroup - 1)][warp][lane >> 3] = s;
         if ((m & (kPkGroup - 1)) == 0 || m == p.nsteps) {
@@ -598,18 +608,65 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
 // team_vec_bytes), the tail's work space in their place after the steps.  USE: kTeam all paths, kOne a chain
 // of at most NT sites on one CTA, kServer no vectors in shared memory.
 enum { kTeam, kOne, kServer };
+__device__ __forceinline__ bool team_sync(const Params& p, int where)
+{
+    if (p.ncta > 1) return grid_barrier(p, where);
+    __syncthreads();
+    return true;
+}
+
+// What an update does besides its steps.  In the FP32 kernels that also hold the steps of
+// tiles it is called: inlined, its registers live across the steps and take theirs (us per
+// update at M = 1024 with both inlined and called: L = 10 on one CTA 481 and 366, L = 16 on one
+// 2306 and 2051, L = 32 on eight 3713 and 3450).
+template <int NT>
+__device__ __forceinline__ bool team_tail_body(const Params& p, PkHead& head, int cta, char* smem, int work_n, long long q)
+{
+    const int C = p.ncta;
+    if (!team_sync(p, 1)) return false;
+    pk_tail_fft<NT>(p, cta, C, (double2*)smem, work_n, head.vv0, head.ov1);
+    if (!team_sync(p, 2)) return false;
+    pk_tail_clear<NT>(p, cta, C);
+    pk_tail_phase<NT>(p, cta, C, (double*)smem);
+    if (!team_sync(p, 3)) return false;
+    pk_decide(p, head, cta, q);
+    __syncthreads();
+    return true;
+}
+// the accepted move, and the magnetisation after a sweep
+template <int NT>
+__device__ __forceinline__ bool team_accept_body(const Params& p, PkHead& head, int cta, int o, bool sweep_done, long long nmag)
+{
+    if (head.acc) {
+        if (cta == 0 && threadIdx.x < 7) patch_site(p, o, head.loc, head.draw[0], head.draw[1], (int)threadIdx.x);
+        if (!team_sync(p, 5)) return false;
+    }
+    auto sync = [&](int where) { return team_sync(p, where); };
+    return !sweep_done || pk_magnetisation<NT>(p, cta, nmag, sync);
+}
+template <int NT>
+__device__ __noinline__ bool team_tail(const Params& p, PkHead& head, int cta, char* smem, int work_n, long long q)
+{
+    return team_tail_body<NT>(p, head, cta, smem, work_n, q);
+}
+template <int NT>
+__device__ __noinline__ bool team_accept(const Params& p, PkHead& head, int cta, int o, bool sweep_done, long long nmag)
+{
+    return team_accept_body<NT>(p, head, cta, o, sweep_done, nmag);
+}
+static __device__ __noinline__ void team_setup(const Params& p, PkHead& head, int o, unsigned long long upd)
+{
+    pk_setup(p, head, o, upd);
+}
+
 template <class R, int NT, int USE>
 __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, char* smem, int work_n, int bytes)
 {
     __shared__ PkHead head;
     [[maybe_unused]] __shared__ StepSums<R> sums;
-    const int tid = threadIdx.x, N = p.N, C = p.ncta;
+    constexpr bool kCall = USE != kOne && sizeof(R) == 4;
+    const int tid = threadIdx.x, N = p.N;
     const unsigned buf = smem_u32(smem);
-    auto sync = [&](int where) -> bool {
-        if (C > 1) return grid_barrier(p, where);
-        __syncthreads();
-        return true;
-    };
     const long long nupd = (p.mode == MODE_SWEEP) ? p.n_updates : 1;
     long long nmag = 0;
     unsigned long long nacc = 0;
@@ -617,11 +674,12 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
     for (long long q = 0; q < nupd; ++q) {
         const unsigned long long upd = p.upd0 + (unsigned long long)q;
         const int o = (p.mode == MODE_SWEEP) ? (int)(upd % (unsigned long long)N) : (int)p.site;
-        pk_setup(p, head, o, upd);
+        if constexpr (!kCall) pk_setup(p, head, o, upd);
+        else team_setup(p, head, o, upd);
         __syncthreads();
         bool done = false;
         if constexpr (USE != kServer) {
-            if (USE == kOne || (bytes > 0 && C == 1 && N <= one_cta_sites<R>(NT))) {
+            if (USE == kOne || (bytes > 0 && p.ncta == 1 && N <= one_cta_sites<R>(NT))) {
                 const unsigned ring = buf + 2u * (unsigned)(sizeof(typename OneCta<R>::V) * N);
                 const int ntr = one_cta_items(N, NT);
                 if constexpr (USE == kOne && sizeof(R) == 8) {
@@ -658,23 +716,21 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
             if (!done && !team_packed_steps<R, false, USE == kTeam>(p, cta, phase, buf, 0, head, sums)) return;
         }
         phase += (unsigned)p.nsteps + 1u;
-        if (!sync(1)) return;
-        pk_tail_fft<NT>(p, cta, C, (double2*)smem, work_n, head.vv0, head.ov1);
-        if (!sync(2)) return;
-        pk_tail_clear<NT>(p, cta, C);
-        pk_tail_phase<NT>(p, cta, C, (double*)smem);
-        if (!sync(3)) return;
-        pk_decide(p, head, cta, q);
-        __syncthreads();
-        if (p.mode == MODE_DELTA) break;
-        if (head.acc) {
-            ++nacc;
-            if (cta == 0 && tid < 7) patch_site(p, o, head.loc, head.draw[0], head.draw[1], tid);
-            if (!sync(5)) return;
+        if constexpr (!kCall) {
+            if (!team_tail_body<NT>(p, head, cta, smem, work_n, q)) return;
+        } else {
+            if (!team_tail<NT>(p, head, cta, smem, work_n, q)) return;
         }
-        if ((upd + 1ull) % (unsigned long long)N == 0ull) {
-            if (!pk_magnetisation<NT>(p, cta, nmag, sync)) return;
-            ++nmag;
+        if (p.mode == MODE_DELTA) break;
+        const bool sweep_done = (upd + 1ull) % (unsigned long long)N == 0ull;
+        if (head.acc || sweep_done) {
+            nacc += head.acc;
+            if constexpr (!kCall) {
+                if (!team_accept_body<NT>(p, head, cta, o, sweep_done, nmag)) return;
+            } else {
+                if (!team_accept<NT>(p, head, cta, o, sweep_done, nmag)) return;
+            }
+            nmag += sweep_done;
         }
     }
     if (cta == 0 && tid == 0 && p.mode == MODE_SWEEP) {
