@@ -53,6 +53,27 @@ __device__ __forceinline__ long long fixed60(float x, bool& ok)
     return (b >> 31) ? -(long long)q : (long long)q;
 }
 
+// FP32 terms summed exactly, as integers: x = hi 2^-20 + lo 2^-41 to 2^-42, for |x| < 4 - 2^-20, by four
+// additions.  Adding 12 leaves x on the grid of the floats in [8, 16), whose bits count in
+// units of 2^-20; the remainder, at most 2^-21, goes the same way.  Sums of up to 2047
+// terms (|lo| <= 2^20 each) do not depend on their order.  bad collects the bits that a
+// term in range leaves zero.
+struct FixTerm {
+    int hi, lo;
+};
+constexpr unsigned kFixBad = 0xbe800000u;
+__device__ __forceinline__ FixTerm fix_term(float x, unsigned& bad)
+{
+    constexpr float kHi = 12.f, kLo = 0x1.8p-18f;
+    constexpr int kHiBits = 0x41400000, kLoBits = 0x36c00000;
+    const float t = __fadd_rn(x, kHi);
+    const float u = __fadd_rn(__fsub_rn(x, __fsub_rn(t, kHi)), kLo);
+    bad |= __float_as_uint(t);
+    return {__float_as_int(t) - kHiBits, __float_as_int(u) - kLoBits};
+}
+// the value of a sum of terms, in units of 2^-60
+__device__ __forceinline__ long long fix_value(int hi, int lo) { return ((long long)hi << 40) + ((long long)lo << 19); }
+
 // Values kept apart by the lane groups of 8 of a warp: on return lanes 8 v .. 8 v + 7
 // hold the warp's sum of value v (v < 4).
 template <class T> __device__ __forceinline__ T warp_reduce_scatter4(const T (&v)[4], int lane)

@@ -70,6 +70,48 @@ __device__ __forceinline__ void add_site(R (&acc)[4], bool class_a, R2 cur, R2 n
     acc[3] = fma(a.x, nxt.y, fma(-a.y, nxt.x, acc[3]));
 }
 
+// A thread's sums of a step, for tiles of any number of sites: FP64 terms in FP64; of
+// FP32, each site's terms (|S_m|^2, Re and Im of the product) as integers (fix_term), so
+// that neither the tile, nor the order of its sites, nor the warps change a bit of them.
+// Added in FP32 over a tile and a warp they cost more accuracy than the recursion: rms
+// error of Delta Omega at M = 256, uniform spins, L = 16 on two CTAs 2.4e-8, so 1.1e-8, L = 32
+// on four 2.2e-8 and 1.1e-8.  The twenty instructions per site cost 7 to 15 % of a step (us per
+// update at M = 1024: L = 16 on one CTA 2048 -> 2365, L = 32 on eight 3650 -> 3917).
+template <class R> struct SiteSums {
+    R v[4] = {0, 0, 0, 0};
+    __device__ __forceinline__ void add(bool class_a, double2 cur, double2 nxt) { add_site(v, class_a, cur, nxt); }
+    __device__ __forceinline__ R reduce(const Params&, int, int lane) const { return warp_reduce_scatter4(v, lane); }
+};
+template <> struct SiteSums<float> {
+    int hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+    unsigned bad = 0;
+    __device__ __forceinline__ void add(bool class_a, float2 cur, float2 nxt)
+    {
+        const float2 a = class_a ? cur : make_float2(0.f, 0.f);
+        const FixTerm u = fix_term(fmaf(cur.x, cur.x, __fmul_rn(cur.y, cur.y)), bad);
+        const FixTerm x = fix_term(fmaf(a.x, nxt.x, __fmul_rn(a.y, nxt.y)), bad);
+        const FixTerm y = fix_term(fmaf(a.x, nxt.y, -__fmul_rn(a.y, nxt.x)), bad);
+        if (class_a) {
+            hi[0] += u.hi;
+            lo[0] += u.lo;
+        } else {
+            hi[1] += u.hi;
+            lo[1] += u.lo;
+        }
+        hi[2] += x.hi;
+        lo[2] += x.lo;
+        hi[3] += y.hi;
+        lo[3] += y.lo;
+    }
+    __device__ __forceinline__ long long reduce(const Params& p, int m, int lane) const
+    {
+        if (bad & kFixBad) set_error(p, ERR_NUMERIC, 90, m);
+        const long long q[4] = {fix_value(hi[0], lo[0]), fix_value(hi[1], lo[1]), fix_value(hi[2], lo[2]),
+                                fix_value(hi[3], lo[3])};
+        return warp_reduce_scatter4(q, lane);
+    }
+};
+
 // ---------------------------------------------------------------------------
 // one CTA, a few sites per thread
 // ---------------------------------------------------------------------------
@@ -349,7 +391,7 @@ static __device__ __noinline__ void one_cta_products(const Params& p, const PkHe
 // The sums of a group of kPkGroup steps by step, warp and value; they are added over the
 // warps together, a warp per step.
 template <class R> struct StepSums {
-    R w[kPkGroup][kWarps][4];
+    std::conditional_t<sizeof(R) == 4, long long, R> w[kPkGroup][kWarps][4];
 };
 
 // Add the sums of the steps f0 .. f1 (one group at most) over the warps, in units of 2^-60.
@@ -358,13 +400,16 @@ __device__ __forceinline__ void add_step_sums(const Params& p, const StepSums<R>
 {
     const int f = f0 + warp;
     if (f > f1) return;
-    const R x = sums.w[f & (kPkGroup - 1)][lane & 7][lane >> 3];
-    bool ok;
+    const auto x = sums.w[f & (kPkGroup - 1)][lane & 7][lane >> 3];
     long long q;
-    if constexpr (sizeof(R) == 4) q = fixed60(x, ok);
-    else q = fixed58(4.0 * x, ok);
-    if (!ok) set_error(p, ERR_NUMERIC, 90, f);
-    q = ok ? q : 0;
+    if constexpr (sizeof(R) == 4) {
+        q = x;
+    } else {
+        bool ok;
+        q = fixed58(4.0 * x, ok);
+        if (!ok) set_error(p, ERR_NUMERIC, 90, f);
+        q = ok ? q : 0;
+    }
     q += __shfl_xor_sync(0xffffffffu, q, 4);
     q += __shfl_xor_sync(0xffffffffu, q, 2);
     q += __shfl_xor_sync(0xffffffffu, q, 1);
@@ -497,7 +542,7 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
                 __syncthreads();
             }
         }
-        R acc[4] = {0, 0, 0, 0};
+        SiteSums<R> acc;
         struct Ops {
             R2 h[6], nv[6], cur, pv;
             int i, w, odd;
@@ -554,7 +599,7 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
                 if constexpr (WIN) sts_v(wr + kB * (unsigned)q.w, nx);
                 if (!WIN || edge) stcg2(gw + q.i, nx);
             }
-            add_site(acc, ((q.odd + par_o + m) & 1) == 0, q.cur, nx);
+            acc.add(((q.odd + par_o + m) & 1) == 0, q.cur, nx);
         };
         // sites [0, n) of a list: k < j0 at k, the others at k + j1 - j0
         auto sites = [&](int n, int j0, int j1, bool edge) {
@@ -589,7 +634,7 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
             part(true);
             if (parts > 1) part(false);
         }
-        const R s = warp_reduce_scatter4(acc, lane);
+        const auto s = acc.reduce(p, m, lane);
         if ((lane & 7) == 0) sums.w[m & (kPkGroup - 1)][warp][lane >> 3] = s;
         if ((m & (kPkGroup - 1)) == 0 || m == p.nsteps) {
             __syncthreads();
