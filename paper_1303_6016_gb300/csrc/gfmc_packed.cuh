@@ -74,15 +74,19 @@ __device__ __forceinline__ FixTerm fix_term(float x, unsigned& bad)
 // the value of a sum of terms, in units of 2^-60
 __device__ __forceinline__ long long fix_value(int hi, int lo) { return ((long long)hi << 40) + ((long long)lo << 19); }
 
-// Values kept apart by the lane groups of 8 of a warp: on return lanes 8 v .. 8 v + 7
-// hold the warp's sum of value v (v < 4).
-template <class T> __device__ __forceinline__ T warp_reduce_scatter4(const T (&v)[4], int lane)
+// Values kept apart by the lane groups of 8 of a warp: on return lanes 8 v .. 8 v + 7 hold value
+// v (v < 4) over four lanes each (scatter), or the warp's sum of it.
+template <class T> __device__ __forceinline__ T warp_scatter4(const T (&v)[4], int lane)
 {
     const bool u16 = lane & 16, u8 = lane & 8;
     const T a = u16 ? v[2] : v[0], b = u16 ? v[3] : v[1];
     const T sa = u16 ? v[0] : v[2], sb = u16 ? v[1] : v[3];
     const T x = a + __shfl_xor_sync(0xffffffffu, sa, 16), y = b + __shfl_xor_sync(0xffffffffu, sb, 16);
-    T r = (u8 ? y : x) + __shfl_xor_sync(0xffffffffu, u8 ? x : y, 8);
+    return (u8 ? y : x) + __shfl_xor_sync(0xffffffffu, u8 ? x : y, 8);
+}
+template <class T> __device__ __forceinline__ T warp_reduce_scatter4(const T (&v)[4], int lane)
+{
+    T r = warp_scatter4(v, lane);
     r += __shfl_xor_sync(0xffffffffu, r, 4);
     r += __shfl_xor_sync(0xffffffffu, r, 2);
     r += __shfl_xor_sync(0xffffffffu, r, 1);
@@ -99,7 +103,7 @@ template <class T> __device__ __forceinline__ T warp_reduce_scatter4(const T (&v
 // cost 220-320 cycles of each.
 constexpr int kPkGroup = 8, kPkRing = 16;
 template <class R, int NW> struct PkSums {
-    std::conditional_t<sizeof(R) == 4, float, long long> w[kPkRing][NW][4];
+    long long w[kPkRing][NW][4];
 };
 
 // Add the warps' sums of step m (run by one warp) into the chain's fixed-point
@@ -112,23 +116,11 @@ __device__ __forceinline__ void pk_flush(const Params& p, const PkSums<R, NW>& s
 {
     const int v = lane >> 3;
     long long q = 0;
-    bool fine = true;
 #pragma unroll
-    for (int w = 0; w < NW; w += 8) {
-        const auto x = s.w[m & (kPkRing - 1)][w + (lane & 7)][v];
-        if constexpr (sizeof(R) == 4) {
-            bool ok;
-            const long long t = fixed60(x, ok);
-            fine = fine && ok;
-            q += ok ? t : 0;
-        } else {
-            q += x;
-        }
-    }
+    for (int w = 0; w < NW; w += 8) q += s.w[m & (kPkRing - 1)][w + (lane & 7)][v];
     q += __shfl_xor_sync(0xffffffffu, q, 4);
     q += __shfl_xor_sync(0xffffffffu, q, 2);
     q += __shfl_xor_sync(0xffffffffu, q, 1);
-    if (!fine) set_error(p, ERR_NUMERIC, 90, m);
     if ((lane & 7) == 0)
         atomicAdd(p.gram + (size_t)(m - 1) * kEntries + (v < 2 ? v : v + 4), (unsigned long long)q);
 }
@@ -334,21 +326,22 @@ __device__ __forceinline__ Pk32Bond pk_bond(const char* a)
     return {make_float2(b.x, b.y), make_float2(b.z, b.w)};
 }
 
+// sums of the positive terms (P, Q) and of the negative ones (S, W): re = P - S, im = Q - W
 struct Pk32Acc {
-    float2 P, Q, Sf, Wf, Sb, Wb;
+    float2 P = {0.f, 0.f}, Q = {0.f, 0.f}, S = {0.f, 0.f}, W = {0.f, 0.f};
     __device__ __forceinline__ void fwd(const Pk32Bond& h, float2 re, float2 im)
     {
         P = __ffma2_rn(h.re, re, P);
         Q = __ffma2_rn(h.re, im, Q);
-        Sf = __ffma2_rn(h.im, im, Sf);
-        Wf = __ffma2_rn(h.im, re, Wf);
+        S = __ffma2_rn(h.im, im, S);
+        Q = __ffma2_rn(h.im, re, Q);
     }
     __device__ __forceinline__ void bwd(const Pk32Bond& h, float2 re, float2 im)
     {
         P = __ffma2_rn(h.re, re, P);
         Q = __ffma2_rn(h.re, im, Q);
-        Sb = __ffma2_rn(h.im, im, Sb);
-        Wb = __ffma2_rn(h.im, re, Wb);
+        P = __ffma2_rn(h.im, im, P);
+        W = __ffma2_rn(h.im, re, W);
     }
 };
 
@@ -458,9 +451,6 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
                     zf = pk_bond(a_zf + k * sZz);
                 }
                 Pk32Acc a;
-                a.P = make_float2(-prv[k].x, -prv[k].y);
-                a.Q = make_float2(-prv[k].z, -prv[k].w);
-                a.Sf = a.Wf = a.Sb = a.Wb = make_float2(0.f, 0.f);
                 // even site: odd of the own pair; odd site: even of the own pair (conjugated bond)
                 a.fwd({make_float2(bin[k].x, bin[k].x), make_float2(bin[k].y, -bin[k].y)}, make_float2(c.y, c.x),
                       make_float2(c.w, c.z));
@@ -470,8 +460,12 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
                 a.fwd(hf, make_float2(yp.x, yp.y), make_float2(yp.z, yp.w));
                 a.bwd(hb, make_float2(ym.x, ym.y), make_float2(ym.z, ym.w));
                 const float2 m1 = make_float2(-1.f, -1.f);
-                float2 re = __fadd2_rn(__ffma2_rn(a.Sf, m1, a.P), a.Sb);
-                float2 im = __ffma2_rn(a.Wb, m1, __fadd2_rn(a.Q, a.Wf));
+                // the bonds first, S_{m-1} last: added onto -S_{m-1}, every term rounds at its magnitude
+                // (rms error of Delta Omega, L = 16 at M = 256: 2.6e-8 so, 2.2e-8 with the bonds first)
+                float2 re = __ffma2_rn(a.S, m1, a.P);
+                float2 im = __ffma2_rn(a.W, m1, a.Q);
+                re = __ffma2_rn(make_float2(prv[k].x, prv[k].y), m1, re);
+                im = __ffma2_rn(make_float2(prv[k].z, prv[k].w), m1, im);
                 if (m == 0) {  // S_1 = Htilde S_0
                     re = make_float2(0.5f * re.x, 0.5f * re.y);
                     im = make_float2(0.5f * im.x, 0.5f * im.y);
@@ -488,6 +482,7 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
                 prv[k] = nx;
             }
         }
+        int h = 0, l = 0;  // value lane >> 3 of the step's sums
         if (m > 0) {
             // class A: the sites of parity par_o + m; an even site has the parity of its row
             const bool ea = par_t == ((par_o + m) & 1);
@@ -496,12 +491,32 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
             v[1] = ea ? U[0].y + U[1].x : U[0].x + U[1].y;
             v[2] = ea ? Xr[0].x + Xr[1].y : Xr[0].y + Xr[1].x;
             v[3] = ea ? Xi[0].x + Xi[1].y : Xi[0].y + Xi[1].x;
-            const float s = warp_reduce_scatter4(v, lane);
-            if ((lane & 7) == 0) sums.w[m & (kPkRing - 1)][warp][lane >> 3] = s;
+            // a thread's sums (of up to four pairs) in FP32, the threads' as integers: over the warp
+            // in FP32 they cost more than the recursion's rounding (rms error of Delta Omega over 72
+            // updates, M = 256, uniform spins: L = 24 on 16 CTAs 2.4e-8, with the bonds first and this 1.3e-8)
+            unsigned bad = 0;
+            int hi[4], lo[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const FixTerm f = fix_term(v[k], bad);
+                hi[k] = f.hi;
+                lo[k] = f.lo;
+            }
+            if (bad & kFixBad) set_error(p, ERR_NUMERIC, 90, m);
+            h = warp_scatter4(hi, lane);
+            l = warp_scatter4(lo, lane);
         }
-        // the sums come before the arrival: its release waits for the remote stores
-        // to be acknowledged (400-560 cycles on a cluster), which the sums cover
+        // these come before the arrival, whose release waits for the remote stores to be
+        // acknowledged (400-560 cycles on a cluster); the rest of the sums before the wait
         pk_arrive(t.C);
+        if (m > 0) {
+#pragma unroll
+            for (int b = 4; b > 0; b >>= 1) {
+                h += __shfl_xor_sync(0xffffffffu, h, b);
+                l += __shfl_xor_sync(0xffffffffu, l, b);
+            }
+            if ((lane & 7) == 0) sums.w[m & (kPkRing - 1)][warp][lane >> 3] = fix_value(h, l);
+        }
         pk_flush_due<float, NW>(p, sums, m, warp, lane);
         pk_wait(t.C);
     };
