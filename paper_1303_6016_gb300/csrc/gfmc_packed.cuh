@@ -37,22 +37,6 @@ namespace gfmc {
 // sums
 // ---------------------------------------------------------------------------
 
-// round(x 2^60) from the bits of a float with integer operations only: the
-// value is mant 2^(ex - 150); ok: |x| <= 4
-__device__ __forceinline__ long long fixed60(float x, bool& ok)
-{
-    const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
-    ok = mag <= 0x40800000u;
-    const int ex = (int)(mag >> 23);
-    const unsigned long long mant = (mag & 0x7fffffu) | (ex ? 0x800000u : 0u);
-    const int sh = (ex ? ex : 1) - 90;  // <= 39 for |x| <= 4
-    unsigned long long q;
-    if (sh >= 0) q = mant << sh;
-    else if (sh <= -25) q = 0;
-    else q = (mant + (1ull << (-sh - 1))) >> -sh;
-    return (b >> 31) ? -(long long)q : (long long)q;
-}
-
 // FP32 terms summed exactly, as integers: x = hi 2^-20 + lo 2^-41 to 2^-42, for |x| < 4 - 2^-20, by four
 // additions.  Adding 12 leaves x on the grid of the floats in [8, 16), whose bits count in
 // units of 2^-20; the remainder, at most 2^-21, goes the same way.  Sums of up to 2047
@@ -73,6 +57,17 @@ __device__ __forceinline__ FixTerm fix_term(float x, unsigned& bad)
 }
 // the value of a sum of terms, in units of 2^-60
 __device__ __forceinline__ long long fix_value(int hi, int lo) { return ((long long)hi << 40) + ((long long)lo << 19); }
+// fix_term of x.x and x.y, by packed additions
+__device__ __forceinline__ void fix_terms(float2 x, FixTerm& a, FixTerm& b, unsigned& bad)
+{
+    constexpr float kHi = 12.f, kLo = 0x1.8p-18f;
+    constexpr int kHiBits = 0x41400000, kLoBits = 0x36c00000;
+    const float2 t = __fadd2_rn(x, make_float2(kHi, kHi)), w = __fadd2_rn(t, make_float2(-kHi, -kHi));
+    const float2 u = __fadd2_rn(__ffma2_rn(w, make_float2(-1.f, -1.f), x), make_float2(kLo, kLo));
+    bad |= __float_as_uint(t.x) | __float_as_uint(t.y);
+    a = {__float_as_int(t.x) - kHiBits, __float_as_int(u.x) - kLoBits};
+    b = {__float_as_int(t.y) - kHiBits, __float_as_int(u.y) - kLoBits};
+}
 
 // Values kept apart by the lane groups of 8 of a warp: on return lanes 8 v .. 8 v + 7 hold value
 // v (v < 4) over four lanes each (scatter), or the warp's sum of it.
@@ -497,10 +492,13 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
             unsigned bad = 0;
             int hi[4], lo[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const FixTerm f = fix_term(v[k], bad);
-                hi[k] = f.hi;
-                lo[k] = f.lo;
+            for (int k = 0; k < 4; k += 2) {
+                FixTerm a, b;
+                fix_terms(make_float2(v[k], v[k + 1]), a, b, bad);
+                hi[k] = a.hi;
+                lo[k] = a.lo;
+                hi[k + 1] = b.hi;
+                lo[k + 1] = b.lo;
             }
             if (bad & kFixBad) set_error(p, ERR_NUMERIC, 90, m);
             h = warp_scatter4(hi, lane);

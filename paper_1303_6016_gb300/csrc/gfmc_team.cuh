@@ -89,8 +89,8 @@ template <> struct SiteSums<float> {
     {
         const float2 a = class_a ? cur : make_float2(0.f, 0.f);
         const FixTerm u = fix_term(fmaf(cur.x, cur.x, __fmul_rn(cur.y, cur.y)), bad);
-        const FixTerm x = fix_term(fmaf(a.x, nxt.x, __fmul_rn(a.y, nxt.y)), bad);
-        const FixTerm y = fix_term(fmaf(a.x, nxt.y, -__fmul_rn(a.y, nxt.x)), bad);
+        FixTerm x, y;
+        fix_terms(make_float2(fmaf(a.x, nxt.x, __fmul_rn(a.y, nxt.y)), fmaf(a.x, nxt.y, -__fmul_rn(a.y, nxt.x))), x, y, bad);
         if (class_a) {
             hi[0] += u.hi;
             lo[0] += u.lo;
@@ -125,7 +125,9 @@ template <class R> struct OneCta {
     static constexpr int kItem = kFix ? 8 : 16;
 };
 
-// Add the sums of the steps f0 .. f1 (at most kPkGroup) over the threads, a warp per step.
+// Add the sums of the steps f0 .. f1 (at most kPkGroup) over the threads, a warp per step, as
+// integers (FP32: of each thread's up to four sites; eight threads' in FP32 first cost, rms error of
+// Delta Omega over 192 updates at L = 8, M = 256, uniform spins, 1.9e-8, now 1.1e-8).
 template <class R>
 __device__ __forceinline__ void one_cta_flush(const Params& p, unsigned ring, int ntr, int f0, int f1, int warp, int lane)
 {
@@ -134,14 +136,22 @@ __device__ __forceinline__ void one_cta_flush(const Params& p, unsigned ring, in
     const unsigned at = ring + (unsigned)OneCta<R>::kItem * (unsigned)((f & (kPkRing - 1)) * ntr + lane);
     long long q = 0;
     if constexpr (sizeof(R) == 4) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        int hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+        unsigned bad = 0;
         for (int j = 0; j < ntr; j += 32) {
             const float4 b = lds_v(at + 16u * j, float4());
-            a = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+            FixTerm t[4];
+            fix_terms(make_float2(b.x, b.y), t[0], t[1], bad);
+            fix_terms(make_float2(b.z, b.w), t[2], t[3], bad);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                hi[k] += t[k].hi;
+                lo[k] += t[k].lo;
+            }
         }
-        bool ok[4];
-        const long long s[4] = {fixed60(a.x, ok[0]), fixed60(a.y, ok[1]), fixed60(a.z, ok[2]), fixed60(a.w, ok[3])};
-        if (!(ok[0] && ok[1] && ok[2] && ok[3])) set_error(p, ERR_NUMERIC, 90, f);
+        if (bad & kFixBad) set_error(p, ERR_NUMERIC, 90, f);
+        const long long s[4] = {fix_value(hi[0], lo[0]), fix_value(hi[1], lo[1]), fix_value(hi[2], lo[2]),
+                                fix_value(hi[3], lo[3])};
         q = warp_reduce_scatter4(s, lane);
     } else {
         for (int j = 0; j < ntr; j += 32) {

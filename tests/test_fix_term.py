@@ -21,6 +21,10 @@ PRELUDE = r"""
 #define __forceinline__ inline
 static float __fadd_rn(float a, float b) { volatile float r = a + b; return r; }
 static float __fsub_rn(float a, float b) { volatile float r = a - b; return r; }
+struct float2 { float x, y; };
+static float2 make_float2(float x, float y) { return {x, y}; }
+static float2 __fadd2_rn(float2 a, float2 b) { return {__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y)}; }
+static float2 __ffma2_rn(float2 a, float2 b, float2 c) { return {std::fma(a.x, b.x, c.x), std::fma(a.y, b.y, c.y)}; }
 static int __float_as_int(float x) { int i; std::memcpy(&i, &x, 4); return i; }
 static unsigned __float_as_uint(float x) { unsigned i; std::memcpy(&i, &x, 4); return i; }
 """
@@ -31,6 +35,13 @@ static int check(float x)
     unsigned bad = 0;
     const FixTerm t = fix_term(x, bad);
     const long long q = fix_value(t.hi, t.lo);
+    FixTerm a, b;  // the packed form, in either place
+    unsigned bad2 = 0;
+    fix_terms(make_float2(x, 0.25f), a, b, bad2);
+    if (bad2 != (bad | 0x41440000u) || (!(bad & kFixBad) && (a.hi != t.hi || a.lo != t.lo || fix_value(b.hi, b.lo) != 1ll << 58))) return 1;
+    bad2 = 0;
+    fix_terms(make_float2(-1.f, x), a, b, bad2);
+    if (!(bad & kFixBad) && (b.hi != t.hi || b.lo != t.lo || fix_value(a.hi, a.lo) != -(1ll << 60) || (bad2 & kFixBad))) return 1;
     const bool ok = (bad & kFixBad) == 0;
     if (!(std::fabs(x) < 4.f - 0x1p-20f)) return std::fabs(x) < 4.1f ? 0 : ok;  // at the end of the range either is right
     if (!ok) return 1;
@@ -83,7 +94,7 @@ def test_fix_term(tmp_path):
         pytest.skip("no host C++ compiler")
     src = open(SRC).read()
     a = src.index("struct FixTerm {")
-    b = src.index("}\n", src.index("long long fix_value")) + 2
+    b = src.index("\n}\n", src.index("void fix_terms")) + 3
     f = tmp_path / "fix.cpp"
     f.write_text(PRELUDE + src[a:b] + DRIVER)
     exe = tmp_path / "fix"

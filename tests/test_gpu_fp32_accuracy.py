@@ -70,3 +70,13 @@ def test_packed_fp32_is_as_exact_as_two_vectors(G, reference, how, ctas):
     for L in SIZES:
         err += squares(G, L, exact[L], how, ctas.get(L), **kw)
     assert np.sqrt(np.mean(err)) <= 1.1 * two
+
+
+def test_one_cta_fp32_is_as_exact_as_seven_vectors(G):
+    """Sizes that one CTA takes with its sites in registers, alone (a site per thread) and as
+    a team of one CTA (two): threads' sums added as integers, so no worse than the seven
+    unit vectors on the grid engine (sums of a warp in FP32: 1.06 of them, so 0.65)."""
+    exact = run(G, 8, "single")
+    seven = squares(G, 8, exact, "single", engine="grid")
+    for how, ctas in (("single", None), ("team", 1)):
+        assert np.mean(squares(G, 8, exact, how, ctas)) <= np.mean(seven)
