@@ -663,9 +663,9 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
 // team_vec_bytes), the tail's work space in their place after the steps.  USE: kTeam all paths, kOne a chain
 // of at most NT sites on one CTA, kServer no vectors in shared memory.
 enum { kTeam, kOne, kServer };
-__device__ __forceinline__ bool team_sync(const Params& p, int where)
+template <bool ONE> __device__ __forceinline__ bool team_sync(const Params& p, int where)
 {
-    if (p.ncta > 1) return grid_barrier(p, where);
+    if (!ONE && p.ncta > 1) return grid_barrier(p, where);
     __syncthreads();
     return true;
 }
@@ -674,40 +674,40 @@ __device__ __forceinline__ bool team_sync(const Params& p, int where)
 // tiles it is called: inlined, its registers live across the steps and take theirs (us per
 // update at M = 1024 with both inlined and called: L = 10 on one CTA 481 and 366, L = 16 on one
 // 2306 and 2051, L = 32 on eight 3713 and 3450).
-template <int NT>
+template <int NT, bool ONE>
 __device__ __forceinline__ bool team_tail_body(const Params& p, PkHead& head, int cta, char* smem, int work_n, long long q)
 {
-    const int C = p.ncta;
-    if (!team_sync(p, 1)) return false;
+    const int C = ONE ? 1 : p.ncta;
+    if (!team_sync<ONE>(p, 1)) return false;
     pk_tail_fft<NT>(p, cta, C, (double2*)smem, work_n, head.vv0, head.ov1);
-    if (!team_sync(p, 2)) return false;
+    if (!team_sync<ONE>(p, 2)) return false;
     pk_tail_clear<NT>(p, cta, C);
     pk_tail_phase<NT>(p, cta, C, (double*)smem);
-    if (!team_sync(p, 3)) return false;
+    if (!team_sync<ONE>(p, 3)) return false;
     pk_decide(p, head, cta, q);
     __syncthreads();
     return true;
 }
 // the accepted move, and the magnetisation after a sweep
-template <int NT>
+template <int NT, bool ONE>
 __device__ __forceinline__ bool team_accept_body(const Params& p, PkHead& head, int cta, int o, bool sweep_done, long long nmag)
 {
     if (head.acc) {
         if (cta == 0 && threadIdx.x < 7) patch_site(p, o, head.loc, head.draw[0], head.draw[1], (int)threadIdx.x);
-        if (!team_sync(p, 5)) return false;
+        if (!team_sync<ONE>(p, 5)) return false;
     }
-    auto sync = [&](int where) { return team_sync(p, where); };
+    auto sync = [&](int where) { return team_sync<ONE>(p, where); };
     return !sweep_done || pk_magnetisation<NT>(p, cta, nmag, sync);
 }
 template <int NT>
 __device__ __noinline__ bool team_tail(const Params& p, PkHead& head, int cta, char* smem, int work_n, long long q)
 {
-    return team_tail_body<NT>(p, head, cta, smem, work_n, q);
+    return team_tail_body<NT, false>(p, head, cta, smem, work_n, q);
 }
 template <int NT>
 __device__ __noinline__ bool team_accept(const Params& p, PkHead& head, int cta, int o, bool sweep_done, long long nmag)
 {
-    return team_accept_body<NT>(p, head, cta, o, sweep_done, nmag);
+    return team_accept_body<NT, false>(p, head, cta, o, sweep_done, nmag);
 }
 static __device__ __noinline__ void team_setup(const Params& p, PkHead& head, int o, unsigned long long upd)
 {
@@ -772,7 +772,7 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
         }
         phase += (unsigned)p.nsteps + 1u;
         if constexpr (!kCall) {
-            if (!team_tail_body<NT>(p, head, cta, smem, work_n, q)) return;
+            if (!team_tail_body<NT, USE == kOne>(p, head, cta, smem, work_n, q)) return;
         } else {
             if (!team_tail<NT>(p, head, cta, smem, work_n, q)) return;
         }
@@ -781,7 +781,7 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
         if (head.acc || sweep_done) {
             nacc += head.acc;
             if constexpr (!kCall) {
-                if (!team_accept_body<NT>(p, head, cta, o, sweep_done, nmag)) return;
+                if (!team_accept_body<NT, USE == kOne>(p, head, cta, o, sweep_done, nmag)) return;
             } else {
                 if (!team_accept<NT>(p, head, cta, o, sweep_done, nmag)) return;
             }
