@@ -1,12 +1,14 @@
 """The packed engines beside the other calls of a chain, and where they end: a chain
 in a batch and then alone, waits that run out on a cluster,
-teams on as many nodes as the tail takes, teams beside other chains."""
+teams on as many nodes as the tail takes, teams beside other chains, and the sizes
+at the far ends of the ranges, against the oracle."""
 import time
 
 import numpy as np
 import pytest
 
 from paper_1303_6016_gb300 import inputs
+from test_gpu_packed import A, replay
 
 pytestmark = pytest.mark.gpu
 
@@ -135,3 +137,38 @@ def test_fp32_team_sums_do_not_depend_on_the_tiles(G, L, teams):
         assert np.abs(o - outs[0]).max() <= 1e-14
     for ch in chains:
         ch.close()
+
+
+@pytest.mark.parametrize("L,M,n", [(50, 16, 2), (62, 16, 1), (64, 16, 1)])
+def test_large_fp64_single_chains_match_oracle(G, L, M, n):
+    """FP64 chains alone beyond three sites per thread of the whole grid (bonds and S_{m-1} from
+    shared memory, up to six face values per thread: L = 50 to 62), and L = 64, which the
+    grid does not hold: the team engine on two vectors.  Tolerance as in test_gpu_packed."""
+    sp = inputs.von_mises_fisher(L, 2.0, L)
+    with G.Chain(L, sp, M=M, beta=12.0, mu=-2.0, seed=5, chain_id=3) as ch:
+        out = ch.updates(n)
+    replay(L, sp, M, 0, 3, out, lambda r: 1e-10 * abs(r) + 1e-13 * A, 1e-9)
+
+
+@pytest.mark.parametrize("L,M,nodes,n", [(14, 32, 0, 8), (20, 16, 0, 6), (22, 16, 0, 4), (26, 16, 32, 3),
+                                         (30, 16, 0, 2), (40, 16, 0, 2), (34, 16, 0, 2)])
+def test_larger_fp32_single_chains_match_oracle(G, L, M, nodes, n):
+    """FP32-mixed chains alone on a cluster, of 14, 16, 11 (cut along z alone), 13, 15 and 16
+    CTAs, with one, two and four pairs of sites per thread; and L = 34, which no cluster
+    takes."""
+    sp = inputs.von_mises_fisher(L, 2.0, L)
+    with G.Chain(L, sp, M=M, beta=12.0, mu=-2.0, seed=5, chain_id=3, precision="fp32_mixed", nodes=nodes) as ch:
+        out = ch.updates(n)
+    replay(L, sp, M, nodes, 3, out, lambda r: 2e-5, 1e-3)
+
+
+@pytest.mark.parametrize("L,C", [(12, 1), (24, 8)])
+def test_fp64_clusters_on_8192_nodes_match_oracle(G, L, C):
+    """The two sizes whose tail's 128 KB leave no room for a record per site, so that they run
+    pk64_steps (everything in shared memory).  Tolerance: the oracle's FP64 rounding over M = 4096
+    steps, 4096 x 2^-53 x a = 2.7e-12, taken four times."""
+    M, n = 4096, 2
+    sp = inputs.uniform_sphere(L, 9)
+    with G.Chain(L, sp, M=M, nodes=8192, beta=12.0, mu=-2.0, seed=5, chain_id=3, recursion="proposal") as ch:
+        out = G.run_clusters([ch], n, [C])[0]
+    replay(L, sp, M, 8192, 3, out, lambda r: 1.1e-11, 1e-9)
