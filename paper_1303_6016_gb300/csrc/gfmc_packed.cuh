@@ -748,12 +748,26 @@ __device__ __noinline__ void pk64_steps(const Params& p, const PkTile& tile, con
 // The odd nodes follow from theta_{K-1-k} = pi - theta_k: f -> conj f for oo, vv
 // and -conj f for A, B, hence d_{K-1-k} = conj d_k and arg d_{K-1-k} = -arg d_k.
 
+// What an update starts from and ends with, in shared memory.
+struct PkHead {
+    double2 c[kVec];             // 2^n v = 2^n Delta~ |o> at the local sites
+    double chi[8][3];            // spinors of the local sites and of the proposal
+    int loc[kVec];
+    int mom[kVec];               // moments calls: the local sites, and where their values go
+    unsigned row[2][kVec];
+    double draw[3];
+    double vv0;                  // <v|v>
+    double2 ov1;                 // <o|Htilde|v>
+    double unit[3];              // twice a unit of the sums oo, vv and ov: the recursion runs on 2^n v (pk_setup)
+    int acc;
+    int stop;                    // a CTA marked the update as failed
+};
+
 // FFT of the chain's sequences: tasks (sequence V, residue r mod Rz of the node
 // index j), task = V Rz + r, dealt round robin to the C CTAs; f of the even
 // nodes goes to p.gnode[V K + j].  work: room for work_n double2 (at least K/2).
 template <int NT>
-__device__ __forceinline__ void pk_tail_fft(const Params& p, int rank, int C, double2* work, int work_n, double vv0,
-                                            double2 ov1)
+__device__ __forceinline__ void pk_tail_fft(const Params& p, int rank, int C, double2* work, int work_n, const PkHead& head)
 {
     const int tid = threadIdx.x, K = p.K, H = K / 2, MH = p.M / 2;
     int Rz = 1;
@@ -768,14 +782,15 @@ __device__ __forceinline__ void pk_tail_fft(const Params& p, int rank, int C, do
         const int nb = min(g, mine - b), tot = nb << lg;
         for (int e = tid; e < tot; e += NT) {
             const int task = rank + (b + (e >> lg)) * C, V = task / Rz, r = task - V * Rz, q = e & (n - 1);
+            const double unit = head.unit[min(V, 2)];
             double2 x = make_double2(0.0, 0.0);
             for (int pp = q; pp < MH; pp += n) {
                 const int nn = 2 * pp + (V >> 1);
-                const double first = V == 0 ? 1.0 : V == 1 ? vv0 : V == 2 ? ov1.x : ov1.y;
+                const double first = V == 0 ? 1.0 : V == 1 ? head.vv0 : V == 2 ? head.ov1.x : head.ov1.y;
                 double a = first;
                 if (pp > 0) {
                     const long long s = (long long)__ldcg(p.gram + (size_t)(pp - 1) * kEntries + (V < 2 ? V : V + 4));
-                    a = fma((double)s, 0x1p-59, -first);  // 2 <.|.> - mu_0 (or mu_1)
+                    a = fma((double)s, unit, -first);  // 2 <.|.> - mu_0 (or mu_1)
                 }
                 a *= __ldg(p.gker + nn) * (nn == 0 ? 0.5 : 1.0);
                 double2 w = __ldg(p.twc + 2 * pp);
@@ -877,20 +892,6 @@ template <int NT> __device__ __forceinline__ void pk_tail_clear(const Params& p,
     }
 }
 
-// What an update starts from and ends with, in shared memory.
-struct PkHead {
-    double2 c[kVec], hop[kVec];  // Delta~ |o> and Htilde_{o, l_k} at the local sites
-    double chi[8][3];            // spinors of the local sites and of the proposal
-    int loc[kVec];
-    int mom[kVec];               // moments calls: the local sites, and where their values go
-    unsigned row[2][kVec];
-    double draw[3];
-    double vv0;                  // <v|v>
-    double2 ov1;                 // <o|Htilde|v>
-    int acc;
-    int stop;                    // a CTA marked the update as failed
-};
-
 // Local sites, proposal and Delta~ by warp 0, one sincos per lane (lane k the
 // polar, lane 8 + k the azimuthal angle): the FP64 pipe takes 64 cycles per
 // warp instruction, so seven threads with six sincos each took six times as
@@ -930,7 +931,6 @@ __device__ __forceinline__ void pk_setup(const Params& p, PkHead& h, int o, unsi
         cv = make_double2((-p.t * on.x + p.t * oo.x) / p.a, (-p.t * on.y + p.t * oo.y) / p.a);
         hv = hop_of(p.hop64, p.N, o, lane - 1, lk);  // Htilde_{o, l_k}
     }
-    if (lane < 7) h.c[lane] = cv;
     // <v|v> and <o|Htilde|v> = sum_k Htilde_{o, l_k} c_k over lanes 1..6
     double v0 = cv.x * cv.x + cv.y * cv.y;
     double2 o1 = dmul(cv, hv);
@@ -940,6 +940,12 @@ __device__ __forceinline__ void pk_setup(const Params& p, PkHead& h, int o, unsi
         o1.x += __shfl_xor_sync(0xffffffffu, o1.x, b);
         o1.y += __shfl_xor_sync(0xffffffffu, o1.y, b);
     }
+    // small moves: v scaled by 2^n to |v|^2 in [1/8, 1/2), so that the sums, in integers, and fixed-point
+    // vectors resolve it like a large one (the two parities do not mix, so nothing else changes)
+    const int e = (__double2hiint(v0) >> 20) - 1023, up = e > -800 && e < -3 ? (-2 - e) >> 1 : 0;
+    const double by = __hiloint2double((1023 + up) << 20, 0);
+    if (lane < 7) h.c[lane] = make_double2(cv.x * by, cv.y * by);
+    if (lane < 3) h.unit[lane] = __hiloint2double((1023 - 59 - (lane == 0 ? 0 : lane == 1 ? 2 * up : up)) << 20, 0);
     if (lane == 0) {
         h.vv0 = v0;
         h.ov1 = o1;
@@ -1041,7 +1047,7 @@ template <class R> __device__ __forceinline__ void pk_run_chain(const Params& p,
             pk64_steps<NT>(p, t, head.loc, head.c, sums);
         }
         sync(1);
-        pk_tail_fft<NT>(p, rank, C, work, work_n, head.vv0, head.ov1);
+        pk_tail_fft<NT>(p, rank, C, work, work_n, head);
         sync(2);
         pk_tail_clear<NT>(p, rank, C);
         pk_tail_phase<NT>(p, rank, C, (double*)work);

@@ -689,7 +689,7 @@ template <bool GRID> __device__ __forceinline__ void pk64_run_chain(const Params
         else ok = pk64_advance<ExN, 1, 0>(p, t, tab, head, sums, mb, ph, &s_fail);
         if (GRID && !ok) return;
         if (!sync(1)) return;
-        pk_tail_fft<kPk64Threads>(p, rank, C, work, work_n, head.vv0, head.ov1);
+        pk_tail_fft<kPk64Threads>(p, rank, C, work, work_n, head);
         if (!sync(2)) return;
         pk_tail_clear<kPk64Threads>(p, rank, C);
         pk_tail_phase<kPk64Threads>(p, rank, C, (double*)work);

@@ -679,7 +679,7 @@ __device__ __forceinline__ bool team_tail_body(const Params& p, PkHead& head, in
 {
     const int C = ONE ? 1 : p.ncta;
     if (!team_sync<ONE>(p, 1)) return false;
-    pk_tail_fft<NT>(p, cta, C, (double2*)smem, work_n, head.vv0, head.ov1);
+    pk_tail_fft<NT>(p, cta, C, (double2*)smem, work_n, head);
     if (!team_sync<ONE>(p, 2)) return false;
     pk_tail_clear<NT>(p, cta, C);
     pk_tail_phase<NT>(p, cta, C, (double*)smem);

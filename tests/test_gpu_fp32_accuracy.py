@@ -80,3 +80,21 @@ def test_one_cta_fp32_is_as_exact_as_seven_vectors(G):
     seven = squares(G, 8, exact, "single", engine="grid")
     for how, ctas in (("single", None), ("team", 1)):
         assert np.mean(squares(G, 8, exact, how, ctas)) <= np.mean(seven)
+
+
+@pytest.mark.parametrize("L", [6, 8, 10, 16, 34])
+@pytest.mark.parametrize("move", [1e-1, 1e-3, 1e-5])
+def test_small_moves(G, L, move):
+    """A proposal close to the spin: FP32-mixed Delta Omega, of the order of the move, keeps the
+    relative accuracy of a large one, on one CTA, clusters and tiles -- the sums' integers of
+    2^-41 resolve a small v only because it is scaled.  Bound: 2e-5 for Delta Omega of order 1
+    (the tolerance of FP32 moments), so 2e-5 of the move; and 1e-4 of Delta Omega itself."""
+    sp = inputs.uniform_sphere(L, 21)
+    o = L ** 3 // 2 + 1
+    th = sp[o, 0] + (0.6 if sp[o, 0] < 1.5 else -0.6) * move
+    ph = sp[o, 1] + 0.8 * move
+    kw = dict(M=128, beta=12.0, mu=-2.0)
+    with G.Chain(L, sp, **kw) as a, G.Chain(L, sp, precision="fp32_mixed", **kw) as b:
+        d64, d32 = a.delta_omega(o, th, ph), b.delta_omega(o, th, ph)
+    assert abs(d32 - d64) <= 2e-5 * move
+    assert abs(d32 - d64) <= 1e-4 * abs(d64)
