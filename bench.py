@@ -61,6 +61,11 @@ FLOP_PER_SITE_STEP_PROPOSAL = 2 * 52 + 8 * 3 + 8
 # step, the work of the FP64 chain's default engine (in fixed point).
 FLOP_PER_SITE_STEP_BIPARTITE = (364 + 147 + 49) / 2
 FLOP_PER_SITE_STEP_PACKED = 48 + 16 / 2
+# In fixed point that is, per site and step, 72 wide multiply-adds (32 x 32 + 64 bits) for the
+# stencil, 2 for S_{m-1} and 12 on average for the products; the integer multiplier of an SM
+# takes 55 per clock (measured: 2.3 cycles per warp instruction and sub-partition).
+WIDE_MADS_PER_SITE_STEP = 86
+WIDE_MADS_PER_CLOCK_SM = 55.0
 
 
 # Bytes of one site in one step of the doubling: read r_m and r_{m-1}, write
@@ -94,9 +99,9 @@ def update_flop_nonzero(L: int, M: int) -> float:
 # sources is unchanged and the launch has that many updates, and null
 # otherwise.
 TRAFFIC_SOURCES = ("gfmc_engine.cuh", "gfmc_k64.cu", "gfmc_k32.cu", "gfmc_internal.h", "gfmc_vcluster.cuh",
-                   "gfmc_kvc.cu", "gfmc_packed.cuh", "gfmc_packed64.cuh", "gfmc_kpk.cu")
-TRAFFIC_HASH = "f1314c5534c2c5a7"
-TRAFFIC_PER_LAUNCH = {"fp64": (16, 6818304 + 2359296), "fp32_mixed": (64, 1485312 + 26880)}
+                   "gfmc_kvc.cu", "gfmc_packed.cuh", "gfmc_packed64.cuh", "gfmc_team.cuh", "gfmc_kpk.cu")
+TRAFFIC_HASH = "6d5de12ad8f8a463"
+TRAFFIC_PER_LAUNCH = {"fp64": (16, 2367232 + 165120), "fp32_mixed": (64, 1137664 + 27392)}
 
 
 def engine_sources_hash() -> str:
@@ -576,6 +581,20 @@ def main():
     achieved_tf = U * flop_nz / launch_s / 1e12
     derived_tf = alu_peak_tflops("fp64", clocks.get("sm_max_mhz") or 2070.0) if clocks else alu_peak_tflops("fp64")
     peak_tf = gfmc.fma_peak_tflops("fp64", repeats=3, stream=stream.cuda_stream)
+    if L % 2 == 0:
+        # the packed recursion in fixed point: a step is bound by its latency, the unit it loads most is
+        # the integer multiplier
+        tmads = U * (M // 2 - 1) * N * WIDE_MADS_PER_SITE_STEP / launch_s / 1e12
+        peak_tmads = (WIDE_MADS_PER_CLOCK_SM * torch.cuda.get_device_properties(local).multi_processor_count *
+                      ((clocks or {}).get("sm_max_mhz") or 2070.0) * 1e6 / 1e12)
+        unit = {"bound": "latency", "achieved": tmads, "peak": peak_tmads, "unit": "T wide multiply-adds/s",
+                "frac": tmads / peak_tmads, "step_us": launch_s / U / (M // 2 - 1) * 1e6,
+                "bound_note": "one exchange of face values over the whole GPU per step; the integer multiplier "
+                              "(86 wide multiply-adds per site and step, 55 per clock and SM) is the unit loaded "
+                              "most, and its share of the time is frac",
+                "fp64_equivalent_tflops": achieved_tf, "fp64_pipe_tflops": peak_tf}
+    else:
+        unit = {"bound": "alu", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s", "frac": achieved_tf / peak_tf}
     # what the FP64 pipe needs at the engine's occupancy (one CTA of 256 per SM)
     issue = {"chains16_warps8": gfmc.fp64_issue_rate(16, 8, stream=stream.cuda_stream),
              "chains1_warps4": gfmc.fp64_issue_rate(1, 4, stream=stream.cuda_stream),
@@ -600,22 +619,22 @@ def main():
         "config": dict(workload_config(L, M, U, "fp64"), parallelism=f"replicas{world}"),
         "stencil_gbs": U * bytes_u / launch_s / 1e9,
         "latency_ms_per_update": {"p50": statistics.median(per) / U, "p99": sorted(per)[-1] / U},
-        "roofline": {"bound": "alu", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
-                     "frac": achieved_tf / peak_tf, "traffic": traffic_per_launch("fp64", U),
+        "roofline": {**unit, "traffic": traffic_per_launch("fp64", U),
                      "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
                      "flop_per_update": flop_nz,
                      "flop_note": "flop of the recursion that runs: |o> + |v| as one vector (56 per site and step "
                                   "of the M/2-1 doubling steps at even L), done in fixed point on the integer "
-                                  "multiplier; peak is the FP64 pipe's, which it replaces.  The seven unit "
+                                  "multiplier (fp64_equivalent_tflops, beside the rate of the FP64 pipe that it "
+                                  "replaces; odd L runs two vectors on that pipe).  The seven unit "
                                   "vectors of the grid engine (280; 791 with the terms that vanish by parity) "
                                   "give flop_full_per_update and stencil_gbs",
                      "flop_full_per_update": flop_u,
-                     "peak_source": "measured in this run: gfmc_measure_fma_peak (own kernel, 16 independent "
+                     "fp64_pipe_source": "measured in this run: gfmc_measure_fma_peak (own kernel, 16 independent "
                                     "double fma chains per thread, one CTA of 256 on every SM, best of 3, CUDA "
                                     "events; it retires the pipe's 2 warp-lane slots per SM clock, see "
                                     "fp64_issue)",
-                     "peak_derived": derived_tf,
-                     "peak_derived_source": "152 SMs x max SM clock x 2 FP64 FMA lanes per SM x 2 flop",
+                     "fp64_pipe_derived": derived_tf,
+                     "fp64_pipe_derived_source": "152 SMs x max SM clock x 2 FP64 FMA lanes per SM x 2 flop",
                      "flop_s8d_per_update": (M // 2) * L ** 3 * 830,
                      "frac_s8d": U * (M // 2) * L ** 3 * 830 / launch_s / 1e12 / peak_tf,
                      "s8d_note": "the per-update count (M/2) N 830 of the seven-vector algorithm, most of which this "
@@ -668,8 +687,8 @@ def main():
     if not args.no_l16:
         # the single-chain workload's smaller lattice: L=16 (N=4096), same M, both precisions
         L16, spins16 = 16, inputs.uniform_sphere(16, 0)
-        l16 = {"L": L16, "M": M, "note": "single chain, uniform spins (seed 0), M=1024; the FP32-mixed chain "
-                                          "runs the grid engine (the vector-cluster engine is for L=32)"}
+        l16 = {"L": L16, "M": M, "note": "single chain, uniform spins (seed 0), M=1024; both run the packed "
+                                          "vector on one cluster of 16 CTAs (the vector-cluster engine is for L=32)"}
         for prec, u16 in (("fp64", 64), ("fp32_mixed", 64)):
             c16 = gfmc.Chain(L16, spins16, M=M, beta=20.0, mu=-2.0, seed=1, chain_id=rank, precision=prec,
                              stream=stream.cuda_stream)

@@ -458,13 +458,14 @@ gfmc_status use_team_plan(gfmc_ctx* h, int tc)
 
 // The packed engine of a chain's Delta Omega calls (automatic engine, even L,
 // plain sums), if one takes it.  Measured, us per update at M = 1024:
-//   One CTA (gfmc_team.cuh) up to 512 sites in FP32, 256 in FP64: FP32-mixed L = 8: 246,
-//   on clusters 326-348; L = 4: 156, on a cluster 276-342 (kOneCtaExact: 173 in fixed
+//   One CTA (gfmc_team.cuh) up to 512 sites in FP32, 256 in FP64: FP32-mixed L = 8: 254,
+//   on a cluster of one CTA 367; L = 4: 156, on a cluster 329 (kOneCtaExact: 173 in fixed
 //   point).  FP64 L = 4: 173, L = 6: 332; L = 8, one site per thread of 512, 669 and on 16 CTAs 425.
-//   FP32-mixed, one cluster of C CTAs: L = 16: 1173 on 1, 443 on 4, 353 on 16; L = 24:
-//   628 on 8, 446 on 16.  So the most CTAs that split the lattice.  L = 32 stays on the
-//   seven vector clusters (767; one packed cluster 643), whose moments without the
-//   doubling are twice as accurate in FP32.
+//   FP32-mixed, one cluster of C CTAs: L = 16: 1220 on 1, 640 on 2, 368 on 16; L = 24:
+//   1175 on 4, 633 on 8, 465 on 16.  So the most CTAs that split the lattice.  L = 32 stays on the
+//   seven vector clusters (771; one packed cluster 648), whose moments without the
+//   doubling are more accurate in FP32 (rms error of Delta Omega 1.4e-8 on random and 1.7e-8 on
+//   aligned spins; a packed cluster 1.9e-8 and 2.8e-8).
 //   FP64: the cluster of the most CTAs up to L = 16 (L = 8: 418 on 16, 668 on the
 //   grid; L = 16: 614 and 651), where a CTA still has at most 256 sites, one per
 //   thread; the whole grid above.

@@ -22,11 +22,11 @@
 //
 // Bound: FP32 by shared-memory wavefronts and instruction issue on large
 // pencils, by the latency of one step (loads, sums, barrier) on small ones;
-// FP64, in fixed point, by instruction issue and the exchange.  Against the two-vector cluster engine, which advances
-// both vectors on every site (half of the values are zeros), ms per update at
-// M = 1024: FP32 L = 32 on 16 CTAs 1.44 -> 0.64, on 8 CTAs 2.03 -> 1.25, L = 16 on
-// 1 CTA 1.92 -> 1.17, L = 8 on 1 CTA 0.80 -> 0.33; FP64 L = 16 on 16 CTAs 3.12 -> 1.66
-// with FP64 arithmetic, 0.61 in fixed point (below).
+// FP64, in fixed point, by the latency of a step and its exchange (gfmc_packed64.cuh).  Against
+// the two-vector cluster engine, which advances both vectors on every site (half of the
+// values are zeros), ms per update at M = 1024: FP32 L = 32 on 16 CTAs 1.44 -> 0.65, on 8 CTAs
+// 2.03 -> 1.23, L = 16 on 1 CTA 1.92 -> 1.22, L = 8 on 1 CTA 0.80 -> 0.37; FP64 L = 16 on 16 CTAs
+// 3.12 -> 1.66 with FP64 arithmetic, 0.63 in fixed point (below).
 #pragma once
 
 #include "gfmc_engine.cuh"
@@ -93,9 +93,8 @@ template <class T> __device__ __forceinline__ T warp_reduce_scatter4(const T (&v
 // wait there, so the sums of step m are complete for every warp after the
 // barrier of step m + 1.  Every kPkGroup steps as many warps add one step each
 // into the chain's sums (at step m = 1 mod kPkGroup the steps m - kPkGroup - 1 .. m - 2; the
-// slots are written again kPkRing steps later), which keeps the additions and
-// conversions off the steps' critical path: one warp flushing one step in every step
-// cost 220-320 cycles of each.
+// slots are written again kPkRing steps later), which keeps the additions off the
+// steps' critical path: one warp flushing one step in every step cost 220-320 cycles of each.
 constexpr int kPkGroup = 8, kPkRing = 16;
 template <class R, int NW> struct PkSums {
     long long w[kPkRing][NW][4];
@@ -533,14 +532,15 @@ __device__ __forceinline__ void pk32_steps(const Params& p, const PkTile& t, con
 // ---------------------------------------------------------------------------
 // GB300's FP64 pipe retires 2 multiply-adds per clock and SM, its integer
 // multiplier about 55 32 x 32 + 64-bit multiply-adds (both measured).
-// |S_n(i)| <= 1 on every site (|T_n(Htilde)| <= 1, |v| <= |Delta~| < 0.82), so FP64
+// |S_n(i)| <= 1 on every site (|T_n(Htilde)| <= 1, |v| < 0.82: |Delta~|, or v scaled), so FP64
 // chains hold S, and 2 Htilde (|2 Htilde| < 0.34; finer than a double above 2^-8), in
 // units of 2^-60 as two limbs, x = xh 2^30 + xl with the low limb centred in
 // [-2^29, 2^29).  In the same units
 //     h s = hh sh + (hh sl + hl sh) 2^-30 + hl sl 2^-60,
 // three wide multiply-adds per real product; the last term, below a quarter
 // unit and of either sign, is left out.  A step rounds once, by half a unit
-// (4.3e-19); the FP64 recursion rounds 12 times, each by half a unit in the last
+// (4.3e-19), and leaves out 12 such terms per component, 0.29 units rms together, as much as
+// the rounding; the FP64 recursion rounds 12 times, each by half a unit in the last
 // place of its partial sums (4.3e-19 where |S_n(i)| is near 2^-8, more above).
 // Bounds: sum over the six bonds of |hh sl| <= 2.9 2^59 and of |hl sh| <= 3.5 2^59
 // (Cauchy-Schwarz, |S_n| <= 1 on a class), so a sum of the middle products stays below 2^62.

@@ -3,7 +3,10 @@
 //
 // With fixed point on the integer multiplier (gfmc_packed.cuh) a step's
 // arithmetic is short, and what is left is latency: the instructions of one site
-// (72 multiply-adds), the sums, the exchange.  A thread advances one to three
+// (72 multiply-adds), the sums, the exchange.  On the whole GPU a step takes 1.3 us at L = 8 and
+// 16 and 1.6 us at L = 32, with 64 times the sites of L = 8: 1.2 us of it do not depend on the
+// sites, and 390 instructions per site of L = 32 issue in a quarter of it.  On a cluster a step
+// of L = 16 takes 1.2 us, without sums (moments, L = 12) 0.6.  A thread advances one to three
 // sites with bonds, S_m and S_{m-1} in registers, or on the smallest tiles 1/2 or 1/4
 // of a site (a lane forms the real or the imaginary part, with 1/4 over half of
 // the bonds); it stores and sends S_{m+1} first and forms the step's sums from

@@ -6,14 +6,13 @@
 // vectors stay in registers, a step's products are formed under the next step's
 // loads, and they are added over the threads by the eight steps, not by a warp
 // reduction in each.  us per step (a default chain, before the packed recursion on one
-// CTA and now): FP32 on a team of one CTA, L = 8 0.97 -> 0.40, L = 4 0.77 -> 0.27 (0.62 in the
+// CTA and now): FP32 on a team of one CTA, L = 8 0.97 -> 0.38, L = 4 0.77 -> 0.27 (0.61 in the
 // fixed point it takes for its accuracy); FP64
 // alone, L = 4 0.82 (a cluster) -> 0.30; the tail of a team's update 49 -> 29 us.
 // Larger tiles by the latency of their loads and index arithmetic, two warps per
-// sub-partition: with the bonds in shared memory L = 16 on one CTA 5.6 -> 4.3 us, L = 24
-// on three 7.9 -> 6.8, L = 32 on eight 8.2 -> 7.3.  Sixteen warps would add a chain's FP32
-// sums in another order than a launch that also holds odd lattices; four sites per
-// pass spill (5.5 us).
+// sub-partition, with the bonds in shared memory: us per step (an update of M = 1024 over its
+// 511 steps) L = 16 on one CTA 4.6, L = 24 on three 7.3, L = 32 on eight 7.6.  Four sites per
+// pass spill.
 #pragma once
 
 #include "gfmc_packed.cuh"
@@ -310,7 +309,7 @@ __device__ __noinline__ void one_cta_steps(const Params& p, const PkHead& head, 
 template <int SPL>
 __device__ __noinline__ void one_cta_advance(const Params& p, const PkHead& head, unsigned buf, int nm, int nt)
 {
-    const int tid = threadIdx.x, N = p.N, L = p.L, nsteps = p.nsteps;
+    const int tid = threadIdx.x, N = p.N, nsteps = p.nsteps;
     const unsigned vecB = 16u * (unsigned)N;
     const int c = SPL > 1 ? tid & 1 : 0, pos = tid / SPL;
     const bool on = pos < N;
