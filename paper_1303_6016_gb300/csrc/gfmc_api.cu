@@ -351,7 +351,7 @@ gfmc_status run_engine(gfmc_ctx* h, Params& P)
         const int smem = gfmc::engine_smem_bytes(P.K);
         e = h->precision == GFMC_PREC_FP64 ? gfmc::launch_team_f64(h->d_job, 1, P.ncta, smem, h->stream)
                                             : gfmc::launch_team_f32(h->d_job, 1, P.ncta, smem, h->stream, P.comp != 0,
-                                                                    (P.nv == 2 && h->L % 2 == 0 && !P.comp) ? 1 : P.nv);
+                                                                    (P.nv == 2 && h->L % 2 == 0 && !P.comp) ? gfmc::kPackedTiles : P.nv);
     } else {
         if (h->vcl && nv == gfmc::kVec)
             e = gfmc::launch_vcluster_f32(P, h->stream);

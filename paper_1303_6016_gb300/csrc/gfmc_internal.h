@@ -279,7 +279,9 @@ cudaError_t launch_engine_f32(const Params& p, cudaStream_t s);
 cudaError_t launch_engine_f64(const Params& p, int nv, cudaStream_t s);
 cudaError_t launch_engine_f32(const Params& p, int nv, cudaStream_t s);
 cudaError_t launch_team_f64(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s);
-// nv: the vectors of every job's recursion (p.nv), 0 when they differ; 1: even lattices on two vectors only
+// nv: the vectors of every job's recursion (p.nv), 0 when they differ; 1: even lattices on two vectors only;
+// kPackedTiles: those with all vectors in global memory
+constexpr int kPackedTiles = 3;
 cudaError_t launch_team_f32(const TeamJob* d_jobs, int njobs, int grid, int smem, cudaStream_t s, bool comp, int nv);
 // co-resident CTAs of the kernel launch_team_* takes for comp and nv, and its static shared memory
 // (bytes); nv < 0: the fewest of any

@@ -80,6 +80,7 @@ static cudaError_t team_launch(const TeamJob* d_jobs, int njobs, int grid, int s
 {
     if (comp) return team_launch<0, true>(d_jobs, njobs, grid, smem, s, ex);
     if (nv == 1) return team_launch<1, false>(d_jobs, njobs, grid, smem, s, ex);
+    if (nv == kPackedTiles) return team_launch<kPackedTiles, false>(d_jobs, njobs, grid, smem, s, ex);
     if (nv == 2) return team_launch<2, false>(d_jobs, njobs, grid, smem, s, ex);
     if (nv == kVec) return team_launch<kVec, false>(d_jobs, njobs, grid, smem, s, ex);
     return team_launch<0, false>(d_jobs, njobs, grid, smem, s, ex);
@@ -109,8 +110,8 @@ cudaError_t team_max_ctas_f32(int smem, bool comp, int nv, int* out)
 {
     if (nv < 0) {  // of the kernel that holds the fewest
         *out = 1 << 30;
-        for (int k = 0; k < 5; ++k) {
-            const int kinds[5] = {0, 1, 2, kVec, 0};
+        for (int k = 0; k < 6; ++k) {
+            const int kinds[6] = {0, 1, 2, kVec, 0, kPackedTiles};
             int n = 0;
             const cudaError_t e = team_max_ctas_f32(smem, k == 4, kinds[k], &n);
             if (e != cudaSuccess) return e;
@@ -120,6 +121,7 @@ cudaError_t team_max_ctas_f32(int smem, bool comp, int nv, int* out)
     }
     if (comp) return team_occupancy<0, true>(smem, out);
     if (nv == 1) return team_occupancy<1, false>(smem, out);
+    if (nv == kPackedTiles) return team_occupancy<kPackedTiles, false>(smem, out);
     if (nv == 2) return team_occupancy<2, false>(smem, out);
     if (nv == kVec) return team_occupancy<kVec, false>(smem, out);
     return team_occupancy<0, false>(smem, out);

@@ -6,12 +6,12 @@
 // vectors stay in registers, a step's products are formed under the next step's
 // loads, and they are added over the threads by the eight steps, not by a warp
 // reduction in each.  us per step (a default chain, before the packed recursion on one
-// CTA and now): FP32 on a team of one CTA, L = 8 0.97 -> 0.38, L = 4 0.77 -> 0.27 (0.61 in the
+// CTA and now): FP32 on a team of one CTA, L = 8 0.97 -> 0.39, L = 4 0.77 -> 0.27 (0.62 in the
 // fixed point it takes for its accuracy); FP64
 // alone, L = 4 0.82 (a cluster) -> 0.30; the tail of a team's update 49 -> 29 us.
 // Larger tiles by the latency of their loads and index arithmetic, two warps per
 // sub-partition, with the bonds in shared memory: us per step (an update of M = 1024 over its
-// 511 steps) L = 16 on one CTA 4.6, L = 24 on three 7.3, L = 32 on eight 7.6.  Four sites per
+// 511 steps) L = 16 on one CTA 4.2, L = 24 on three 6.9, L = 32 on eight 6.9.  Four sites per
 // pass spill.
 #pragma once
 
@@ -74,8 +74,7 @@ __device__ __forceinline__ void add_site(R (&acc)[4], bool class_a, R2 cur, R2 n
 // that neither the tile, nor the order of its sites, nor the warps change a bit of them.
 // Added in FP32 over a tile and a warp they cost more accuracy than the recursion: rms
 // error of Delta Omega at M = 256, uniform spins, L = 16 on two CTAs 2.4e-8, so 1.1e-8, L = 32
-// on four 2.2e-8 and 1.1e-8.  The twenty instructions per site cost 7 to 15 % of a step (us per
-// update at M = 1024: L = 16 on one CTA 2048 -> 2365, L = 32 on eight 3650 -> 3917).
+// on four 2.2e-8 and 1.1e-8.  The twenty instructions per site cost 5 to 15 % of a step.
 template <class R> struct SiteSums {
     R v[4] = {0, 0, 0, 0};
     __device__ __forceinline__ void add(bool class_a, double2 cur, double2 nxt) { add_site(v, class_a, cur, nxt); }
@@ -474,7 +473,7 @@ template <class R> __device__ __forceinline__ const typename Cx<R>::T* hop_table
 // others are computed, so the neighbours' wait overlaps the rest of the step.
 // Without WIN (tiles below a plane, or too large for shared memory) all values
 // are read from global memory, in the same order.
-template <class R, bool WIN, bool WIDE>
+template <class R, bool WIN, bool WIDE, bool LATE = false>
 __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigned phase, unsigned buf, int bytes,
                                                const PkHead& head, StepSums<R>& sums)
 {
@@ -528,9 +527,10 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
     if constexpr (WIN) __syncthreads();
     else publish(p, cta, phase + 1);
 
-    // sites of the tile within a plane of its ends: [0, e0) and [e1, T).  Wherever the vectors
-    // stand (which the launch's other chains have a say in): the order of the sums follows it
-    const int e0 = (p.ncta > 1 && T > 2 * LL) ? LL : T, e1 = e0 < T ? T - LL : T;
+    // sites of the tile within a plane of its ends: [0, e0) and [e1, T).  FP64: wherever the vectors
+    // stand (which the launch's other chains have a say in), as the order of the sums follows it
+    constexpr bool kEnds = WIN || sizeof(R) == 8;
+    const int e0 = (kEnds && p.ncta > 1 && T > 2 * LL) ? LL : T, e1 = e0 < T ? T - LL : T;
     const int parts = e0 < e1 ? 2 : 1;
     const int halo = whole ? N - T : 2 * LL;
     for (int m = 1; m <= p.nsteps; ++m) {
@@ -598,7 +598,20 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
             if constexpr (WIN) q.pv = lds_v(wr + kB * (unsigned)q.w, R2());
             else q.pv = ldcg2(gw + i);
         };
-        auto step = [&](Ops& q, bool edge) {
+        // LATE: the terms of the last pass's sites wait for the next pass's loads, or for the
+        // publication, to be added under (tiles in global memory: us per update at M = 1024, L = 34 alone
+        // 1567 -> 1496, L = 64 3065 -> 2772; with the bonds in shared memory, L = 16 on one CTA, 2169 -> 2361;
+        // in a kernel of their own, kPackedTiles, L = 34 1261, L = 64 2433)
+        constexpr bool kLate = LATE && WIDE && sizeof(R) == 4;
+        [[maybe_unused]] R2 pc[2], pn[2];
+        [[maybe_unused]] bool pa[2];
+        auto late = [&]() {
+            if constexpr (kLate) {
+                acc.add(pa[0], pc[0], pn[0]);
+                acc.add(pa[1], pc[1], pn[1]);
+            }
+        };
+        auto step = [&](Ops& q, bool edge, int slot) {
             q.h[1].y = -q.h[1].y;  // backward bonds: the conjugates
             q.h[3].y = -q.h[3].y;
             q.h[5].y = -q.h[5].y;
@@ -608,7 +621,14 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
                 if constexpr (WIN) sts_v(wr + kB * (unsigned)q.w, nx);
                 if (!WIN || edge) stcg2(gw + q.i, nx);
             }
-            acc.add(((q.odd + par_o + m) & 1) == 0, q.cur, nx);
+            const bool a = ((q.odd + par_o + m) & 1) == 0;
+            if constexpr (kLate) {
+                pa[slot] = a;
+                pc[slot] = q.cur;
+                pn[slot] = nx;
+            } else {
+                acc.add(a, q.cur, nx);
+            }
         };
         // sites [0, n) of a list: k < j0 at k, the others at k + j1 - j0
         auto sites = [&](int n, int j0, int j1, bool edge) {
@@ -619,14 +639,16 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
                     Ops qa, qb;
                     load(at(k), qa);
                     if (k + kThreads < n) load(at(k + kThreads), qb);
-                    step(qa, edge);
-                    if (k + kThreads < n) step(qb, edge);
+                    if (k >= 2 * kThreads) late();
+                    step(qa, edge, 0);
+                    if (k + kThreads < n) step(qb, edge, 1);
+                    else if constexpr (kLate) pc[1] = pn[1] = c_make<R2>(0, 0);
                 }
             } else {
                 for (int k = tid; k < n; k += kThreads) {
                     Ops q;
                     load(at(k), q);
-                    step(q, edge);
+                    step(q, edge, 0);
                 }
             }
         };
@@ -636,7 +658,11 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
             sites(ends ? e0 + T - e1 : e1 - e0, ends ? e0 : 0, ends ? e1 : e0, ends && p.ncta > 1);
             if (ends) publish(p, cta, phase + (unsigned)m + 1u);
         };
-        if constexpr (sizeof(R) == 4) {
+        if constexpr (!kEnds) {
+            sites(T, T, T, true);
+            publish(p, cta, phase + (unsigned)m + 1u);
+            if (tid < T) late();
+        } else if constexpr (sizeof(R) == 4) {
 #pragma unroll 1
             for (int k = 0; k < parts; ++k) part(k == 0);
         } else {
@@ -660,8 +686,8 @@ __device__ __noinline__ bool team_packed_steps(const Params& p, int cta, unsigne
 // A chain on the p.ncta CTAs of a team, this one its CTA `cta`.  smem: room for
 // work_n double2 at least; bytes > 0: the vectors stand there too (`bytes`, at least
 // team_vec_bytes), the tail's work space in their place after the steps.  USE: kTeam all paths, kOne a chain
-// of at most NT sites on one CTA, kServer no vectors in shared memory.
-enum { kTeam, kOne, kServer };
+// of at most NT sites on one CTA, kServer and kTiles no vectors in shared memory.
+enum { kTeam, kOne, kServer, kTiles };
 template <bool ONE> __device__ __forceinline__ bool team_sync(const Params& p, int where)
 {
     if (!ONE && p.ncta > 1) return grid_barrier(p, where);
@@ -669,12 +695,9 @@ template <bool ONE> __device__ __forceinline__ bool team_sync(const Params& p, i
     return true;
 }
 
-// What an update does besides its steps.  In the FP32 kernels that also hold the steps of
-// tiles it is called: inlined, its registers live across the steps and take theirs (us per
-// update at M = 1024 with both inlined and called: L = 10 on one CTA 481 and 366, L = 16 on one
-// 2306 and 2051, L = 32 on eight 3713 and 3450).
+// What an update does besides its steps.
 template <int NT, bool ONE>
-__device__ __forceinline__ bool team_tail_body(const Params& p, PkHead& head, int cta, char* smem, int work_n, long long q)
+__device__ __forceinline__ bool team_tail(const Params& p, PkHead& head, int cta, char* smem, int work_n, long long q)
 {
     const int C = ONE ? 1 : p.ncta;
     if (!team_sync<ONE>(p, 1)) return false;
@@ -689,7 +712,7 @@ __device__ __forceinline__ bool team_tail_body(const Params& p, PkHead& head, in
 }
 // the accepted move, and the magnetisation after a sweep
 template <int NT, bool ONE>
-__device__ __forceinline__ bool team_accept_body(const Params& p, PkHead& head, int cta, int o, bool sweep_done, long long nmag)
+__device__ __forceinline__ bool team_accept(const Params& p, PkHead& head, int cta, int o, bool sweep_done, long long nmag)
 {
     if (head.acc) {
         if (cta == 0 && threadIdx.x < 7) patch_site(p, o, head.loc, head.draw[0], head.draw[1], (int)threadIdx.x);
@@ -698,27 +721,11 @@ __device__ __forceinline__ bool team_accept_body(const Params& p, PkHead& head, 
     auto sync = [&](int where) { return team_sync<ONE>(p, where); };
     return !sweep_done || pk_magnetisation<NT>(p, cta, nmag, sync);
 }
-template <int NT>
-__device__ __noinline__ bool team_tail(const Params& p, PkHead& head, int cta, char* smem, int work_n, long long q)
-{
-    return team_tail_body<NT, false>(p, head, cta, smem, work_n, q);
-}
-template <int NT>
-__device__ __noinline__ bool team_accept(const Params& p, PkHead& head, int cta, int o, bool sweep_done, long long nmag)
-{
-    return team_accept_body<NT, false>(p, head, cta, o, sweep_done, nmag);
-}
-static __device__ __noinline__ void team_setup(const Params& p, PkHead& head, int o, unsigned long long upd)
-{
-    pk_setup(p, head, o, upd);
-}
-
 template <class R, int NT, int USE>
 __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, char* smem, int work_n, int bytes)
 {
     __shared__ PkHead head;
     [[maybe_unused]] __shared__ StepSums<R> sums;
-    constexpr bool kCall = USE != kOne && sizeof(R) == 4;
     const int tid = threadIdx.x, N = p.N;
     const unsigned buf = smem_u32(smem);
     const long long nupd = (p.mode == MODE_SWEEP) ? p.n_updates : 1;
@@ -728,11 +735,10 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
     for (long long q = 0; q < nupd; ++q) {
         const unsigned long long upd = p.upd0 + (unsigned long long)q;
         const int o = (p.mode == MODE_SWEEP) ? (int)(upd % (unsigned long long)N) : (int)p.site;
-        if constexpr (!kCall) pk_setup(p, head, o, upd);
-        else team_setup(p, head, o, upd);
+        pk_setup(p, head, o, upd);
         __syncthreads();
         bool done = false;
-        if constexpr (USE != kServer) {
+        if constexpr (USE == kOne || USE == kTeam) {
             if (USE == kOne || (bytes > 0 && p.ncta == 1 && N <= one_cta_sites<R>(NT))) {
                 const unsigned ring = buf + 2u * (unsigned)(sizeof(typename OneCta<R>::V) * N);
                 const int ntr = one_cta_items(N, NT);
@@ -767,23 +773,15 @@ __device__ __forceinline__ void pk_team_chain(const Params& p, const int cta, ch
             }
         }
         if constexpr (USE != kOne) {
-            if (!done && !team_packed_steps<R, false, USE == kTeam>(p, cta, phase, buf, 0, head, sums)) return;
+            if (!done && !team_packed_steps<R, false, USE != kServer, USE == kTiles>(p, cta, phase, buf, 0, head, sums)) return;
         }
         phase += (unsigned)p.nsteps + 1u;
-        if constexpr (!kCall) {
-            if (!team_tail_body<NT, USE == kOne>(p, head, cta, smem, work_n, q)) return;
-        } else {
-            if (!team_tail<NT>(p, head, cta, smem, work_n, q)) return;
-        }
+        if (!team_tail<NT, USE == kOne>(p, head, cta, smem, work_n, q)) return;
         if (p.mode == MODE_DELTA) break;
         const bool sweep_done = (upd + 1ull) % (unsigned long long)N == 0ull;
         if (head.acc || sweep_done) {
             nacc += head.acc;
-            if constexpr (!kCall) {
-                if (!team_accept_body<NT, USE == kOne>(p, head, cta, o, sweep_done, nmag)) return;
-            } else {
-                if (!team_accept<NT>(p, head, cta, o, sweep_done, nmag)) return;
-            }
+            if (!team_accept<NT, USE == kOne>(p, head, cta, o, sweep_done, nmag)) return;
             nmag += sweep_done;
         }
     }
@@ -806,7 +804,8 @@ __global__ void __launch_bounds__(NT, 1) gfmc_one_cta(const Params p, int work_n
 
 // A batch of chains, each on its own team of CTAs (jobs sorted by cta0).
 // smem: bytes of dynamic shared memory, shared out chain by chain (team_smem_bytes).
-// NV: the recursion of all chains, 0 when they differ; 1: all on the packed recursion.
+// NV: the recursion of all chains, 0 when they differ; 1: all on the packed recursion; kPackedTiles:
+// on it with every vector in global memory.
 // With several recursions in one kernel the FP32 steps spill (seven vectors, moments
 // of L = 40: 866 us, alone 720; packed, one-CTA chain of L = 8: 0.94 us per step, alone 0.45).
 template <class R, int NV, bool COMP = false>
@@ -849,12 +848,16 @@ __global__ void __launch_bounds__(kThreads, 1) gfmc_team_engine(const TeamJob* _
         [[maybe_unused]] double2* work = dyn_all + s_vs / (int)sizeof(double2);
         [[maybe_unused]] R2* vec = s_vs ? (R2*)dyn_all : nullptr;
         if constexpr (!COMP && NV != kVec) {
+            if (NV == kPackedTiles) {
+                pk_team_chain<R, kThreads, kTiles>(sp, s_cta, (char*)dyn_all, smem / (int)sizeof(double2), 0);
+                continue;
+            }
             if (NV == 1 || (sp.nv == 2 && sp.L % 2 == 0)) {
                 pk_team_chain<R, kThreads, kTeam>(sp, s_cta, (char*)dyn_all, smem / (int)sizeof(double2), s_vs ? smem : 0);
                 continue;
             }
         }
-        if constexpr (NV >= 2) run_chain<R, 1, NV, kThreads, true, COMP>(sp, s_cta, work, vec);
+        if constexpr (NV == 2 || NV == kVec) run_chain<R, 1, NV, kThreads, true, COMP>(sp, s_cta, work, vec);
         if constexpr (NV == 0) {
             if (sp.nv == 2) run_chain<R, 1, 2, kThreads, true, COMP>(sp, s_cta, work, vec);
             else run_chain<R, 1, kVec, kThreads, true, COMP>(sp, s_cta, work, vec);
